@@ -5,6 +5,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/aim.h"
@@ -46,7 +47,7 @@ aim_status check_device(const aim_ctx* ctx);
 enum KernelId {
   K_ROW_FWD = 0, K_COL_CONV, K_ROW_INV, K_GATHER, K_GRAM,
   K_SETUP_SAMPLE, K_SETUP_DFT, K_SETUP_PACK, K_SETUP_SEGPAIRS, K_SETUP_NEAR,
-  K_RHS, K_GMRES, K_MULTI, K_DFT_STAGE, K_COUNT
+  K_RHS, K_GMRES, K_MULTI, K_DFT_STAGE, K_ANTERP, K_COUNT
 };
 void count_launches(int id, int n);   // counted, not timed
 void thread_launch_counts(long long* out);   // this host thread's counts, K_COUNT entries
@@ -59,6 +60,36 @@ struct ProfScope {
   cudaStream_t st;
   int slot;
 };
+
+// ------------------------------------------------------------------------------------
+// chained launches
+// ------------------------------------------------------------------------------------
+// The kernels of a product follow one another on one stream, each reading what the one before wrote.
+// They are launched with programmatic stream serialization: a kernel's CTAs may be placed while the
+// previous kernel drains, run up to grid_dependency_wait(), which returns when the previous grid is
+// complete and its writes are visible, and touch nothing that any earlier kernel writes or reads
+// before that. Every such kernel calls grid_dependency_wait() in every CTA, so when a kernel runs,
+// all earlier ones on the stream are complete, not only its direct predecessor.
+template <typename... P, typename... A>
+aim_status launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  AIM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return AIM_OK;
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
 
 // ------------------------------------------------------------------------------------
 // sizes
@@ -120,7 +151,7 @@ bool schedule_feasible(int precision, int logH, int logP, const Schedule& s);
 struct PassSpec {
   int nproj;                       // projections applied to each rhs (N: 3, S: 1)
   int proj[kMaxProj];              // which projection weights
-  double2 coef[kMaxProj];          // gather coefficient per projection
+  double coef[kMaxProj];           // gather coefficient per projection
   bool filtered;                   // spectrum choice
   const NearField* near;           // near-field correction (nullptr: none)
   int near_which;                  // which near value array
@@ -135,6 +166,7 @@ struct aim_ctx {
   int n = 0, m = 0, P = 0, H = 0, logH = 0, logP = 0, s = 0, p = 0;
   double k = 0, L = 0, eps = 0, alpha = 0, near_radius = 0;
   int filter_enabled = 0;
+  int qcut = 0;             // the filtered spectrum vanishes on columns q with min(q, P - q) > qcut
   int device = 0;
   // active grid set
   int n_act = 0, row_lo = 0, row_hi = -1, nrows = 0;
@@ -175,6 +207,7 @@ struct aim_ctx {
   // defaults: measured at the single-solve scale (2048^2 grid, P = 4096), feasible at every P
   aim::Schedule sched[3] = {{2, 128, 0, 8}, {2, 128, 0, 16}, {2, 128, 0, 16}};
   // bookkeeping
+  std::vector<std::pair<const void*, size_t>> smem_raised;   // dynamic shared memory limits raised so far
   std::vector<void*> allocations;
   size_t device_bytes = 0;
   double setup_seconds = 0;

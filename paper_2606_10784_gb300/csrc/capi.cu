@@ -120,9 +120,9 @@ static PassSpec make_spec(const aim_ctx* ctx, aim_op op) {
     case AIM_OP_N:
       s.nproj = 3;
       s.proj[0] = 1; s.proj[1] = 2; s.proj[2] = 3;
-      s.coef[0] = double2{1.0, 0.0};
-      s.coef[1] = double2{-k2, 0.0};
-      s.coef[2] = double2{-k2, 0.0};
+      s.coef[0] = 1.0;
+      s.coef[1] = -k2;
+      s.coef[2] = -k2;
       s.filtered = false;
       s.near = &ctx->near;
       s.near_which = 1;
@@ -130,9 +130,9 @@ static PassSpec make_spec(const aim_ctx* ctx, aim_op op) {
     case AIM_OP_N_ALPHA:
       s.nproj = 3;
       s.proj[0] = 1; s.proj[1] = 2; s.proj[2] = 3;
-      s.coef[0] = double2{1.0, 0.0};
-      s.coef[1] = double2{-k2, 0.0};
-      s.coef[2] = double2{-k2, 0.0};
+      s.coef[0] = 1.0;
+      s.coef[1] = -k2;
+      s.coef[2] = -k2;
       s.filtered = true;
       s.near = nullptr;
       break;
@@ -140,14 +140,14 @@ static PassSpec make_spec(const aim_ctx* ctx, aim_op op) {
     case AIM_OP_EFIE_ALPHA:
       s.nproj = 1;
       s.proj[0] = 0;
-      s.coef[0] = double2{1.0, 0.0};
+      s.coef[0] = 1.0;
       s.filtered = true;
       s.near = nullptr;
       break;
     default:   // S and the TM EFIE
       s.nproj = 1;
       s.proj[0] = 0;
-      s.coef[0] = double2{1.0, 0.0};
+      s.coef[0] = 1.0;
       s.filtered = false;
       s.near = &ctx->near;
       s.near_which = 0;
@@ -368,6 +368,11 @@ aim_status derive_params(aim_ctx* ctx, const aim_geometry* geometry, double k, c
   ctx->near_radius = stencil->near_radius > 0.0 ? stencil->near_radius : ctx->s * ctx->eps;
   ctx->filter_enabled = filter ? filter->enabled : AIM_FILTER_NONE;
   ctx->alpha = ctx->filter_enabled ? filter->alpha : 0.0;
+  // the last column of the mask's disc (Eq. 10), with a margin of rounding: one column too many
+  // only costs its transforms. Without a mask every column counts.
+  ctx->qcut = ctx->H;
+  if (ctx->filter_enabled == AIM_FILTER_NUMERICAL)
+    while (ctx->qcut > 0 && 2.0 * M_PI / (P * ctx->eps) * ctx->qcut > ctx->alpha * (1.0 + 1e-9)) --ctx->qcut;
   return AIM_OK;
 }
 

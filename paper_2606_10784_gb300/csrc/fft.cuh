@@ -35,6 +35,14 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   const float2 p = __fmul2_rn(make_float2(a.y, a.y), make_float2(b.y, b.x));
   return __ffma2_rn(make_float2(a.x, a.x), make_float2(b.x, -b.y), p);
 }
+// binary64 products with explicit fused multiply-adds, so that every kernel rounds them alike (left
+// to the compiler, the contraction of a b - c d may differ from one kernel to the next)
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+  return double2{__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.x, b.y, __dmul_rn(a.y, b.x))};
+}
+__device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
+  return double2{__fma_rn(a.x, b.x, __dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, -__dmul_rn(a.x, b.y))};
+}
 template <typename T2> __device__ __forceinline__ T2 mul_minus_i(T2 a) { return T2{a.y, -a.x}; }
 template <typename T2> __device__ __forceinline__ T2 mul_plus_i(T2 a) { return T2{-a.y, a.x}; }
 

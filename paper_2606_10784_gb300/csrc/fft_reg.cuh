@@ -55,7 +55,7 @@ __device__ __forceinline__ T2 rot16(T2 d, int e) {
         default: c = -C1; s = S1; break;   // 7
       }
       const T cc = (T)c, ss = INV ? (T)(-s) : (T)s;
-      return T2{d.x * cc + d.y * ss, d.y * cc - d.x * ss};
+      return T2{fma(d.x, cc, d.y * ss), fma(d.y, cc, -(d.x * ss))};
     }
   }
 }
@@ -155,13 +155,21 @@ __device__ __forceinline__ int fft_npass(int logH) { return logH / LOGE + (logH 
 template <int LOGE>
 __device__ __forceinline__ int fft_logr(int pass, int logH) { return pass < logH / LOGE ? LOGE : logH % LOGE; }
 
+// Reads element i of transform f from shared memory (the default input of a pass).
+template <int NF, int LOGE, typename T2>
+struct PlainLoad {
+  const T2* sm;
+  const int (&fb)[NF];
+  __device__ __forceinline__ T2 operator()(int f, int i) const { return sm[fb[f] + padi<LOGE>(i)]; }
+};
+
 // One pass over NF transforms owned by this thread group, shared memory in and out.
 // Each thread works on butterflies b = j + t*tpf (t < E/R) of each of its transforms, whose
-// padded bases in shared memory are fb[f]. `post(f, out_index, value)` may rewrite a value
-// before it is stored (identity for plain passes). Barrier before and after the stores.
-template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Post>
-__device__ __forceinline__ void smem_pass(T2* __restrict__ sm, const int (&fb)[NF], int j, int tpf, int logH,
-                                          int logNs, const T2* __restrict__ tw, int logP, Post post) {
+// padded bases in shared memory are fb[f]. `load(f, i)` reads input i of transform f. Barrier
+// before and after the stores.
+template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Load>
+__device__ __forceinline__ void smem_pass_from(T2* __restrict__ sm, const int (&fb)[NF], int j, int tpf, int logH,
+                                               int logNs, const T2* __restrict__ tw, int logP, Load load) {
   constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
   const int lognb = logH - LOGR;
   const int nsm = (1 << logNs) - 1;
@@ -172,7 +180,7 @@ __device__ __forceinline__ void smem_pass(T2* __restrict__ sm, const int (&fb)[N
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[f][t][r] = sm[fb[f] + padi<LOGE>(b + (r << lognb))];
+      for (int r = 0; r < R; ++r) v[f][t][r] = load(f, b + (r << lognb));
     bfly_shared<LOGR, INV>(v, t, b & nsm, logNs, tw, logP);
   }
   __syncthreads();
@@ -186,17 +194,23 @@ __device__ __forceinline__ void smem_pass(T2* __restrict__ sm, const int (&fb)[N
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int o = base + (r << logNs);
-        sm[fb[f] + padi<LOGE>(o)] = post(f, o, v[f][t][r]);
+        sm[fb[f] + padi<LOGE>(o)] = v[f][t][r];
       }
     }
   __syncthreads();
 }
 
-// Last pass: shared memory in, `emit(t, r, out_index, values[NF])` out (no stores to shared
-// memory here; callers that write shared memory in `emit` must place a barrier first).
-template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Emit>
-__device__ __forceinline__ void last_pass(const T2* __restrict__ sm, const int (&fb)[NF], int j, int tpf, int logH,
-                                          int logNs, const T2* __restrict__ tw, int logP, Emit emit) {
+template <int LOGR, bool INV, int NF, int LOGE, typename T2>
+__device__ __forceinline__ void smem_pass(T2* __restrict__ sm, const int (&fb)[NF], int j, int tpf, int logH,
+                                          int logNs, const T2* __restrict__ tw, int logP) {
+  smem_pass_from<LOGR, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP, PlainLoad<NF, LOGE, T2>{sm, fb});
+}
+
+// Last pass: `load(f, i)` in, `emit(out_index, values[NF])` out (no stores to shared memory here;
+// callers that write shared memory in `emit` must place a barrier first).
+template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Load, typename Emit>
+__device__ __forceinline__ void last_pass_from(int j, int tpf, int logH, int logNs, const T2* __restrict__ tw, int logP,
+                                               Load load, Emit emit) {
   constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
   const int lognb = logH - LOGR;
   const int nsm = (1 << logNs) - 1;
@@ -208,7 +222,7 @@ __device__ __forceinline__ void last_pass(const T2* __restrict__ sm, const int (
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[f][0][r] = sm[fb[f] + padi<LOGE>(b + (r << lognb))];
+      for (int r = 0; r < R; ++r) v[f][0][r] = load(f, b + (r << lognb));
     bfly_shared<LOGR, INV>(v, 0, k, logNs, tw, logP);
     const int base = ((b - k) << LOGR) + k;
 #pragma unroll
@@ -221,19 +235,25 @@ __device__ __forceinline__ void last_pass(const T2* __restrict__ sm, const int (
   }
 }
 
+template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Emit>
+__device__ __forceinline__ void last_pass(const T2* __restrict__ sm, const int (&fb)[NF], int j, int tpf, int logH,
+                                          int logNs, const T2* __restrict__ tw, int logP, Emit emit) {
+  last_pass_from<LOGR, INV, NF, LOGE>(j, tpf, logH, logNs, tw, logP, PlainLoad<NF, LOGE, T2>{sm, fb}, emit);
+}
+
 // Runs passes [p0, p1) of a length-2^logH transform in shared memory, dispatching the radix.
-template <bool INV, int NF, int LOGE, typename T2, typename Post>
+template <bool INV, int NF, int LOGE, typename T2>
 __device__ __forceinline__ void smem_passes(T2* sm, const int (&fb)[NF], int j, int tpf, int logH, int p0, int p1,
-                                            int logNs, const T2* tw, int logP, Post post) {
+                                            int logNs, const T2* tw, int logP) {
   for (int p = p0; p < p1; ++p) {
     const int lr = fft_logr<LOGE>(p, logH);
     if (lr == LOGE) {
-      smem_pass<LOGE, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP, post);
+      smem_pass<LOGE, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP);
     } else {
       switch (lr) {
-        case 3: if constexpr (LOGE > 3) smem_pass<3, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP, post); break;
-        case 2: smem_pass<2, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP, post); break;
-        default: smem_pass<1, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP, post); break;
+        case 3: if constexpr (LOGE > 3) smem_pass<3, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP); break;
+        case 2: smem_pass<2, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP); break;
+        default: smem_pass<1, INV, NF, LOGE>(sm, fb, j, tpf, logH, logNs, tw, logP); break;
       }
     }
     logNs += lr;
@@ -309,10 +329,5 @@ __device__ __forceinline__ void conv_mid_dispatch(int lr, T2* sm, const int (&fb
     }
   }
 }
-
-struct Identity {
-  template <typename T2>
-  __device__ __forceinline__ T2 operator()(int, int, T2 v) const { return v; }
-};
 
 }  // namespace aim

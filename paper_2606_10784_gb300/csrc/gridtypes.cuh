@@ -65,10 +65,46 @@ __device__ __forceinline__ float2 cto_vt(float2 v, double s) { return float2{v.x
 __device__ __forceinline__ double2 cto_vt(double2 v, double s) { return cto_d2(v, s); }
 __device__ __forceinline__ double2 cto_vt(dfc v, double s) { return cto_d2(v, s); }
 
+// one part (0: real, 1: imaginary) of cto_vt
+__device__ __forceinline__ float cto_vt_part(float2 v, int part, double s) { return (part ? v.y : v.x) * (float)s; }
+__device__ __forceinline__ double cto_vt_part(double2 v, int part, double s) { return (part ? v.y : v.x) * s; }
+__device__ __forceinline__ double cto_vt_part(dfc v, int part, double s) {
+  const float h = part ? v.yh : v.xh, l = part ? v.yl : v.xl;
+  return ((double)h + (double)l) * s;
+}
+
 // tables of double-float values are float4 (xh, yh, xl, yl), the order of dfc
 __device__ __forceinline__ dfc ldro(const dfc* p) {
   const float4 v = __ldg(reinterpret_cast<const float4*>(p));
   return dfc{v.x, v.y, v.z, v.w};
+}
+
+// two neighbouring values as one vector access: 32 bytes for the 16-byte types (p 32-byte aligned),
+// 16 bytes for complex64 (p 16-byte aligned)
+__device__ __forceinline__ void store_pair(float2* p, float2 a, float2 b) {
+  *reinterpret_cast<float4*>(p) = float4{a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ void store_pair(double2* p, double2 a, double2 b) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
+}
+__device__ __forceinline__ void store_pair(dfc* p, dfc a, dfc b) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.xh), "f"(a.yh), "f"(a.xl),
+               "f"(a.yl), "f"(b.xh), "f"(b.yh), "f"(b.xl), "f"(b.yl)
+               : "memory");
+}
+__device__ __forceinline__ void load_pair(const float2* p, float2& a, float2& b) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  a = float2{v.x, v.y};
+  b = float2{v.z, v.w};
+}
+__device__ __forceinline__ void load_pair(const double2* p, double2& a, double2& b) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a.x), "=d"(a.y), "=d"(b.x), "=d"(b.y) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void load_pair(const dfc* p, dfc& a, dfc& b) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(a.xh), "=f"(a.yh), "=f"(a.xl), "=f"(a.yl), "=f"(b.xh), "=f"(b.yh), "=f"(b.xl), "=f"(b.yl)
+               : "l"(p)
+               : "memory");
 }
 
 // value held by the partner lane (lane ^ 1); all 32 lanes must call it together

@@ -15,6 +15,8 @@ constexpr int kGramLanes = 8;
 
 __global__ void k_gram_inv(const double* __restrict__ gi, int blo, int cnt, int n, int nrhs,
                            const double2* __restrict__ x, double2* __restrict__ y) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long o = t / kGramLanes;
   const int g = threadIdx.x & (kGramLanes - 1);
@@ -62,13 +64,13 @@ aim_status gram_inv_apply(aim_ctx* ctx, int nrhs, const double2* x, double2* y, 
   if (ctx->gram_inv == nullptr) return fail(AIM_ESTATE, "no Gram matrix on a TM context");
   const int blo = ctx->gram_band;
   const int cnt = (blo * 2 + 1 <= ctx->n) ? 2 * blo + 1 : ctx->n;
-  const int total = ctx->n * nrhs;
+  const long long threads = (long long)ctx->n * nrhs * kGramLanes;
+  const int tpb = gather_threads(threads);
   {
     ProfScope ps(K_GRAM, st);
-    k_gram_inv<<<(unsigned)(((long long)total * kGramLanes + 255) / 256), 256, 0, st>>>(ctx->gram_inv, blo, cnt,
-                                                                                        ctx->n, nrhs, x, y);
+    AIM_TRY(launch_chained(k_gram_inv, dim3((unsigned)((threads + tpb - 1) / tpb)), tpb, 0, st,
+                           static_cast<const double*>(ctx->gram_inv), blo, cnt, ctx->n, nrhs, x, y));
   }
-  AIM_CUDA_TRY(cudaGetLastError());
   return AIM_OK;
 }
 

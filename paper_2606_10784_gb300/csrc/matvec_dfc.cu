@@ -1,12 +1,11 @@
-// The grid product (Eq. 8 / Eq. 10) compiled for double-float complex (FP64 mode) grid arithmetic. One translation unit per
-// element type keeps the build parallel.
+// Grid product in double-float arithmetic: single-context launches (the 16-element passes are in matvec_dfc_e16.cu).
 #include "matvec_kernels.cuh"
 
 namespace aim {
 
+extern template aim_status launch_tpt<dfc, 1, 4>(aim_ctx*, int, bool, RowFwdArgs, RowInvArgs, void*, const Schedule&, cudaStream_t);
+extern template aim_status launch_tpt<dfc, 2, 4>(aim_ctx*, int, bool, RowFwdArgs, RowInvArgs, void*, const Schedule&, cudaStream_t);
 template aim_status grid_pass<dfc>(aim_ctx*, const PassSpec&, int, const double2*, double2*, cudaStream_t);
-template aim_status grid_product_dense<dfc>(aim_ctx*, bool, int, const double2*, double2*, void*, size_t,
-                                          cudaStream_t);
-template aim_status grid_pass_multi<dfc>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
+template aim_status grid_product_dense<dfc>(aim_ctx*, bool, int, const double2*, double2*, void*, size_t, cudaStream_t);
 
 }  // namespace aim

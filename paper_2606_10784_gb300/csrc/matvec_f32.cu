@@ -1,12 +1,11 @@
-// The grid product (Eq. 8 / Eq. 10) compiled for complex64 (mixed precision) grid arithmetic. One translation unit per
-// element type keeps the build parallel.
+// Grid product in complex64 arithmetic: single-context launches (the 16-element passes are in matvec_f32_e16.cu).
 #include "matvec_kernels.cuh"
 
 namespace aim {
 
+extern template aim_status launch_tpt<float2, 1, 4>(aim_ctx*, int, bool, RowFwdArgs, RowInvArgs, void*, const Schedule&, cudaStream_t);
+extern template aim_status launch_tpt<float2, 2, 4>(aim_ctx*, int, bool, RowFwdArgs, RowInvArgs, void*, const Schedule&, cudaStream_t);
 template aim_status grid_pass<float2>(aim_ctx*, const PassSpec&, int, const double2*, double2*, cudaStream_t);
-template aim_status grid_product_dense<float2>(aim_ctx*, bool, int, const double2*, double2*, void*, size_t,
-                                          cudaStream_t);
-template aim_status grid_pass_multi<float2>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
+template aim_status grid_product_dense<float2>(aim_ctx*, bool, int, const double2*, double2*, void*, size_t, cudaStream_t);
 
 }  // namespace aim

@@ -2,9 +2,9 @@
 //
 // For each channel (one projection of one right-hand side) the product
 //     y = P_t^T [ F^-1( F(c) .* F(b) ) ]_restr ,   b = zero-padded P_s x
-// runs as three grid passes and a gather:
-//   k_row_fwd   sparse anterpolation of x onto grid row iy (u = P_s x, deterministic,
-//               no atomics) fused with the forward P-point row DFT. The row has nonzeros
+// runs as an anterpolation, three grid passes and a gather:
+//   k_anterpolate  u = P_s x at the active grid points (deterministic, no atomics).
+//   k_row_fwd   the forward P-point row DFT of u. The row has nonzeros
 //               only in its first m <= P/2 entries, so X[2k] = DFT_H(a)[k] and
 //               X[2k+1] = DFT_H(a w^n)[k], H = P/2, w = exp(-2 pi i/P).
 //   k_col_conv  per column q: the same pruned forward DFT along the rows, the product with
@@ -40,32 +40,235 @@
 namespace aim {
 
 // ------------------------------------------------------------------------------------
-// row pass, forward
+// anterpolation
 // ------------------------------------------------------------------------------------
-struct RowFwdArgs {
-  const double2* x;     // sparse mode: n * nrhs vectors; dense mode: m*m grid per channel
-  int dense;
-  int n, m, nrhs;
-  const int* row_ptr;
-  const int* act_ix;
+struct AntArgs {
+  const double2* x;    // n * nrhs
+  int n, nrhs, n_act;
   const int* sc_ptr;
   const int* sc_col;
   const double* w[kMaxProj];
+  void* u;             // element type of the grid, channel-major, n_act per channel
+};
+
+// u = P_s x at the active points, NP projections of one right-hand side per thread: the row pass
+// then starts from values instead of from four dependent loads (row range, entry range, column,
+// vector) that one warp of its CTA chases while the others wait at a barrier. Grid-point-major
+// lists, so deterministic without atomics. A point has a handful of entries (about 7): the loads
+// of up to kAntChunk entries are issued together before their FMAs, which run in entry order as a
+// plain loop would.
+constexpr int kAntChunk = 8, kAntThreads = 64;
+
+template <typename CT, int NP>
+__device__ __forceinline__ void ant_item(const AntArgs& a, long long t) {
+  if (t >= (long long)a.n_act * a.nrhs) return;
+  const int r = (int)(t / a.n_act), ap = (int)(t - (long long)r * a.n_act);
+  const double2* xv = a.x + (size_t)r * a.n;
+  double re[NP], im[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) re[q] = im[q] = 0.0;
+  const int e0 = a.sc_ptr[ap], e1 = a.sc_ptr[ap + 1];
+  for (int e = e0; e < e1; e += kAntChunk) {
+    int col[kAntChunk];
+    double ww[NP][kAntChunk];
+    double2 xx[kAntChunk];
+#pragma unroll
+    for (int u = 0; u < kAntChunk; ++u) {
+      col[u] = e + u < e1 ? a.sc_col[e + u] : 0;
+#pragma unroll
+      for (int q = 0; q < NP; ++q) ww[q][u] = e + u < e1 ? a.w[q][e + u] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kAntChunk; ++u) xx[u] = e + u < e1 ? xv[col[u]] : double2{0.0, 0.0};
+#pragma unroll
+    for (int u = 0; u < kAntChunk; ++u) {
+      if (e + u < e1) {
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+          re[q] = fma(ww[q][u], xx[u].x, re[q]);
+          im[q] = fma(ww[q][u], xx[u].y, im[q]);
+        }
+      }
+    }
+  }
+  CT* out = static_cast<CT*>(a.u) + (size_t)r * a.n_act + ap;
+#pragma unroll
+  for (int q = 0; q < NP; ++q) out[(size_t)q * a.nrhs * a.n_act] = cfrom<CT>(re[q], im[q]);
+}
+
+template <typename CT, int NP>
+__global__ void __launch_bounds__(kAntThreads) k_anterpolate(AntArgs a) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
+  ant_item<CT, NP>(a, (long long)blockIdx.x * kAntThreads + threadIdx.x);
+}
+
+// ------------------------------------------------------------------------------------
+// row pass, forward
+// ------------------------------------------------------------------------------------
+struct RowFwdArgs {
+  const double2* x;     // dense mode: m*m grid per channel
+  const void* u;        // sparse mode: values at the active points, channel-major
+  int dense;
+  int m, n_act;
+  const int* row_ptr;
+  const int* act_ix;
   void* inter;
   const void* tw;
   int logH, logP, row_lo, nrows;
   int rows_per_cta;
+  int qcut;            // columns q with min(q, P - q) > qcut carry a zero spectrum: not stored
+  int sparse;          // few active points per row: the first radix runs at the active points only
 };
 
+// Output k of a row's transforms into the tiled intermediate: X[2k] and X[2k + 1] are neighbours in
+// a tile. With both in the thread they go out as one vector store (32 bytes for the 16-byte types: a
+// whole sector; as two stores each was half a sector written twice, 73 of 280 us of the double-float
+// pass at 2048 points).
+template <typename CT, int TPT>
+__device__ __forceinline__ void store_row(CT* out, const RowFwdArgs& a, int rloc, bool live, int half, int k,
+                                          const CT (&v)[TPT]) {
+  constexpr int W = GridT<CT>::W;
+  const int P = 1 << a.logP;
+  if (!live) return;
+  if constexpr (TPT == 2) {
+    const int q = 2 * k;
+    if (min(q, P - 1 - q) <= a.qcut) store_pair(&out[((size_t)(q / W) * a.nrows + rloc) * W + (q % W)], v[0], v[1]);
+  } else {
+    const int q = 2 * k + half;
+    if (min(q, P - q) <= a.qcut) out[((size_t)(q / W) * a.nrows + rloc) * W + (q % W)] = v[0];
+  }
+}
+
+// ------------------------------------------------------------------------------------
+// sparse rows
+// ------------------------------------------------------------------------------------
+// A grid row of a contour holds few active points (about 18 of 2048 at the single-solve scale).
+// The length-H transforms of a row split as H = R0 J, n = j + J r: the radix-R0 pass over r has at
+// most one nonzero butterfly per active point, so it runs as a scatter of the active points into
+// the R0 outputs of their j (forward), or as a sum over the R0 sub-transforms at the active points
+// only (inverse), and only the J-point transforms are dense. J is a power of E, so the dense part
+// has one or two radix-E passes instead of the three or four of the whole length.
+template <int LOGE>
+__host__ __device__ __forceinline__ int sparse_logj(int logH) {
+  // two dense passes when the sparse radix then stays >= 2, else one
+  return logH > 2 * LOGE ? 2 * LOGE : LOGE;
+}
+
+// The sparse radix of a transform length: R0 = 2^l0 <= 32, K2 = 2 R0 terms per point (both halves).
+struct SparseGeom {
+  int logj, l0, k2;
+};
+template <int LOGE>
+__host__ __device__ __forceinline__ SparseGeom sparse_geom(int logH) {
+  SparseGeom s;
+  s.logj = sparse_logj<LOGE>(logH);
+  s.l0 = logH - s.logj;
+  s.k2 = 2 << s.l0;
+  return s;
+}
+
+// Shared memory of the sparse stages behind the transforms' buffers: the forward pass's K2 roots of
+// unity, w^j for j < J and, per row, the J masks of active r; the inverse pass's row ranges.
+template <typename CT, int LOGE>
+__host__ __device__ __forceinline__ size_t sparse_smem(int logH, int rows) {
+  const SparseGeom s = sparse_geom<LOGE>(logH);
+  return (size_t)(s.k2 + (1 << s.logj)) * sizeof(CT) + ((size_t)rows << s.logj) * 4 + (size_t)(rows + 1) * 4;
+}
+
+// Whether a context's rows take the sparse stages. Counting operations, a point costs 2 R0 products
+// and sums where the dense radix-R0 passes cost about 0.57 J log2(R0) of them per row; the line lies
+// at half of that because the operations on single points are slower than those of the dense passes.
+template <int LOGE>
+static bool sparse_rows(const aim_ctx* ctx) {
+  const int logj = sparse_logj<LOGE>(ctx->logH), l0 = ctx->logH - logj;
+  return 4LL * ctx->n_act <= ((long long)ctx->nrows * l0) << logj;
+}
+
+// Forward row pass of sparse rows. The points of a row go to their places j + J r of the row's two
+// buffers (u in the even half's, u w^j in the odd half's) and into the masks that say which r of a j
+// hold one; nothing else is written, so nothing is zeroed. The first dense pass forms its inputs
+//     X0_half[j R0 + k1] = sum over the active r of j of u w^(half j) W_{2 R0}^{r (2 k1 + half)}
+// from them in registers (r ascending) and goes on at Ns = R0. (Scattering every point into the R0
+// outputs of its j by read-modify-write of shared memory took 38 of 280 us of the double-float pass
+// at 2048 points, and 13 of 33 us at 512 points, where the rows along the contour's tangents set the
+// time of the whole launch.)
+template <typename CT, int TPT, int LOGE>
+__device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_block, int c, unsigned char* smraw) {
+  using T2 = CT;
+  constexpr int NF = TPT, LPT = 3 - TPT;
+  T2* sm = reinterpret_cast<T2*>(smraw);
+  const int H = 1 << a.logH, P = 1 << a.logP, tpf = H >> LOGE, HS = padded_len<LOGE>(H);
+  const int per_row = LPT * tpf;
+  const int g = threadIdx.x / per_row, rem = threadIdx.x - g * per_row;
+  const int half = TPT == 1 ? (rem & 1) : 0, j = TPT == 1 ? (rem >> 1) : rem;
+  const int row0 = row_block * a.rows_per_cta, rloc = row0 + g;
+  const bool live = rloc < a.nrows;
+  const T2* tw = static_cast<const T2*>(a.tw);
+  int fb[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) fb[f] = (2 * g + (TPT == 1 ? half : f)) * HS;
+  const SparseGeom sg = sparse_geom<LOGE>(a.logH);
+  const int J = 1 << sg.logj;
+  T2* roots = sm + 2 * a.rows_per_cta * HS;
+  T2* wjs = roots + sg.k2;
+  unsigned* masks = reinterpret_cast<unsigned*>(wjs + J);
+  {
+    const int p0 = live ? a.row_ptr[a.row_lo + rloc] : 0, p1 = live ? a.row_ptr[a.row_lo + rloc + 1] : 0;
+    for (int i = threadIdx.x; i < sg.k2; i += blockDim.x) roots[i] = ldro(&tw[i << sg.logj]);
+    for (int i = threadIdx.x; i < J; i += blockDim.x) wjs[i] = ldro(&tw[i]);
+    for (int i = rem; i < J; i += per_row) masks[(g << sg.logj) + i] = 0;
+    int ix = p0 + rem < p1 ? a.act_ix[p0 + rem] : 0;
+    const T2* uv = static_cast<const T2*>(a.u) + (size_t)c * a.n_act;
+    __syncthreads();
+    grid_dependency_wait();
+    for (int ap = p0 + rem; ap < p1; ap += per_row) {
+      if (ap != p0 + rem) ix = a.act_ix[ap];
+      const T2 u = uv[ap];
+      sm[2 * g * HS + padi<LOGE>(ix)] = u;
+      sm[(2 * g + 1) * HS + padi<LOGE>(ix)] = cmul(u, wjs[ix & (J - 1)]);
+      atomicOr(&masks[(g << sg.logj) + (ix & (J - 1))], 1u << (ix >> sg.logj));
+    }
+  }
+  __syncthreads();
+  const unsigned* rowmask = masks + (g << sg.logj);
+  auto load = [&](int f, int i) {
+    const int jj = i >> sg.l0, kk = 2 * (i & ((1 << sg.l0) - 1)) + (TPT == 1 ? half : f);
+    const T2* src = sm + fb[f];
+    unsigned m = rowmask[jj];
+    T2 acc = czero<T2>();
+    bool first = true;
+    while (m) {
+      const int r = __ffs(m) - 1;
+      m &= m - 1;
+      const T2 v = cmul(src[padi<LOGE>(jj + (r << sg.logj))], roots[(r * kk) & (sg.k2 - 1)]);
+      acc = first ? v : cadd(acc, v);
+      first = false;
+    }
+    return acc;
+  };
+  T2* out = static_cast<T2*>(a.inter) + (size_t)c * P * a.nrows;
+  auto emit = [&](int k, const T2 (&v)[NF]) { store_row<CT, TPT>(out, a, rloc, live, half, k, v); };
+  if (sg.logj == LOGE) {
+    last_pass_from<LOGE, false, NF, LOGE>(j, tpf, a.logH, sg.l0, tw, a.logP, load, emit);
+  } else {
+    smem_pass_from<LOGE, false, NF, LOGE>(sm, fb, j, tpf, a.logH, sg.l0, tw, a.logP, load);
+    last_pass<LOGE, false, NF, LOGE>(sm, fb, j, tpf, a.logH, sg.l0 + LOGE, tw, a.logP, emit);
+  }
+}
+
 // CTA: rows_per_cta rows of one channel; (3 - TPT) * H/E threads per row (E = 2^LOGE elements each).
-constexpr int kAntChunk = 8;
 
 // One work item of the forward row pass: rows [row_block * rows_per_cta, +rows_per_cta) of channel c.
 // Every thread of the CTA calls it (it holds barriers); `smraw` is the CTA's dynamic shared memory.
 template <typename CT, int TPT, int LOGE>
 __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block, int c, unsigned char* smraw) {
+  if (a.sparse) {
+    row_fwd_sparse<CT, TPT, LOGE>(a, row_block, c, smraw);
+    return;
+  }
   using T2 = CT;
-  constexpr int W = GridT<CT>::W, NF = TPT, LPT = 3 - TPT;
+  constexpr int NF = TPT, LPT = 3 - TPT;
   T2* sm = reinterpret_cast<T2*>(smraw);
   const int H = 1 << a.logH, P = 1 << a.logP, tpf = H >> LOGE, HS = padded_len<LOGE>(H);
   const int per_row = LPT * tpf;
@@ -79,7 +282,7 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
   int fb[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) fb[f] = (2 * g + (TPT == 1 ? half : f)) * HS;
-  // zero the row buffer, then anterpolate u = P_s x into it (the row's active-point range is
+  // zero the row buffer, then put the row's values into it (the row's active-point range is
   // loaded first so that its latency overlaps the zeroing). Forming u w^n here, at the active
   // points only and into a second zeroed buffer, was measured: 0.6 % faster in double-float and
   // 3 % slower in complex64, so pass 0 keeps the products.
@@ -90,6 +293,7 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
   }
   for (int i = rem; i < HS; i += per_row) sm[fbA + i] = czero<T2>();
   __syncthreads();
+  grid_dependency_wait();
   if (live) {
     if (a.dense) {
       const double2* u = a.x + (size_t)c * a.m * a.m + (size_t)iy * a.m;
@@ -98,41 +302,8 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
         sm[fbA + padi<LOGE>(ix)] = cfrom<T2>(v.x, v.y);
       }
     } else {
-      const int pj = c / a.nrhs, r = c - pj * a.nrhs;
-      // projection weights by unrolled compare (indexing the argument array with a runtime
-      // index would copy it to local memory)
-      const double* w = a.w[0];
-#pragma unroll
-      for (int q = 1; q < kMaxProj; ++q)
-        if (q == pj) w = a.w[q];
-      const double2* xv = a.x + (size_t)r * a.n;
-      for (int ap = a0 + rem; ap < a1; ap += per_row) {
-        // a grid row holds few active points (tens), each with a handful of entries, so most of
-        // the CTA waits here: the loads of up to kAntChunk entries are issued together before
-        // their FMAs, which run in entry order as a plain loop would
-        double re = 0.0, im = 0.0;
-        const int e0 = a.sc_ptr[ap], e1 = a.sc_ptr[ap + 1];
-        for (int e = e0; e < e1; e += kAntChunk) {
-          int col[kAntChunk];
-          double ww[kAntChunk];
-          double2 xx[kAntChunk];
-#pragma unroll
-          for (int u = 0; u < kAntChunk; ++u) {
-            col[u] = e + u < e1 ? a.sc_col[e + u] : 0;
-            ww[u] = e + u < e1 ? w[e + u] : 0.0;
-          }
-#pragma unroll
-          for (int u = 0; u < kAntChunk; ++u) xx[u] = e + u < e1 ? xv[col[u]] : double2{0.0, 0.0};
-#pragma unroll
-          for (int u = 0; u < kAntChunk; ++u) {
-            if (e + u < e1) {
-              re = fma(ww[u], xx[u].x, re);
-              im = fma(ww[u], xx[u].y, im);
-            }
-          }
-        }
-        sm[fbA + padi<LOGE>(a.act_ix[ap])] = cfrom<T2>(re, im);
-      }
+      const T2* uv = static_cast<const T2*>(a.u) + (size_t)c * a.n_act;
+      for (int ap = a0 + rem; ap < a1; ap += per_row) sm[fbA + padi<LOGE>(a.act_ix[ap])] = uv[ap];
     }
   }
   __syncthreads();
@@ -157,23 +328,19 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
     __syncthreads();
   }
   const int np = fft_npass<LOGE>(a.logH);
-  smem_passes<false, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP, Identity{});
+  smem_passes<false, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP);
   int logNs = 0;
   for (int p = 0; p < np - 1; ++p) logNs += fft_logr<LOGE>(p, a.logH);
   // last pass: X[2k + half] straight to the tiled intermediate
   T2* out = static_cast<T2*>(a.inter) + (size_t)c * P * a.nrows;
   last_pass_dispatch<false, NF, LOGE>(sm, fb, j, tpf, a.logH, logNs, tw, a.logP, [&](int k, const T2 (&v)[NF]) {
-    if (!live) return;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const int q = 2 * k + (TPT == 1 ? half : f);
-      out[((size_t)(q / W) * a.nrows + rloc) * W + (q % W)] = v[f];
-    }
+    store_row<CT, TPT>(out, a, rloc, live, half, k, v);
   });
 }
 
 template <typename CT, int TPT, int LOGE>
 __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_row_fwd(RowFwdArgs a) {
+  grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   row_fwd_item<CT, TPT, LOGE>(a, blockIdx.x, blockIdx.y, smraw);
 }
@@ -184,7 +351,7 @@ __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_row_fwd(Row
 struct ColArgs {
   void* inter;
   const void* spec;
-  const int* live;     // filtered spectrum: per column q' <= P/2, 0 where the mask zeroes it; else null
+  int qcut;            // columns q with min(q, P - q) > qcut carry a zero spectrum: neither read nor written
   const void* tw;
   int logH, logP, row_lo, nrows;
   int log_cols;        // log2 of the columns of one channel per CTA
@@ -224,23 +391,14 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
   const int colc = g * cw + wl;                         // column within the CTA
   const int qcol = (ctile << a.log_cols) + colc;   // column of the grid
   const int w = qcol & (W - 1), tile = qcol / W;
-  if (a.live != nullptr) {
-    // the filtered spectrum (Eq. 10) vanishes on columns beyond the mask radius: when it does on
-    // every column of this CTA their product is zero, so write zeros and skip the transforms
-    // (the same decision in every thread: the early return is uniform)
-    bool any = false;
-    for (int cc = 0; cc < (1 << a.log_cols); ++cc) {
-      const int q = (ctile << a.log_cols) + cc;
-      any = any || a.live[min(q, P - q)] != 0;
-    }
-    if (!any) {
-      T2* base = static_cast<T2*>(a.inter) + (size_t)c * P * a.nrows;
-      const int total = (1 << a.log_cols) * a.nrows;
-      for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        const int cc = e / a.nrows, row = e - cc * a.nrows;
-        const int q = (ctile << a.log_cols) + cc;
-        base[((size_t)(q / W) * a.nrows + row) * W + (q & (W - 1))] = czero<T2>();
-      }
+  {
+    // the filtered spectrum (Eq. 10) vanishes on columns beyond the mask radius. The row passes
+    // neither store nor load those, so a CTA that holds nothing else has no work (a CTA's columns
+    // are an aligned run, so its smallest distance from column 0 is at one of its ends; the same
+    // decision in every thread: the early return is uniform)
+    const int qa = ctile << a.log_cols, qb = qa + (1 << a.log_cols) - 1;
+    if (min(min(qa, P - qa), min(qb, P - qb)) > a.qcut) {
+      grid_dependency_wait();   // a launch of such CTAs alone must not complete before its predecessor
       return;
     }
   }
@@ -250,6 +408,7 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
   const T2* tw = static_cast<const T2*>(a.tw);
   T2* blk = static_cast<T2*>(a.inter) + (size_t)c * P * a.nrows + (size_t)tile * a.nrows * W;
   const int row_hi = a.row_lo + a.nrows - 1;
+  grid_dependency_wait();
   // pass 0 from global: a[n] and/or a[n] w^n, n = j + (H/E)-stride
   {
     const int lognb = a.logH - LOGE;
@@ -271,7 +430,7 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
   }
   const int np = fft_npass<LOGE>(a.logH);
   // remaining forward passes but the last
-  smem_passes<false, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP, Identity{});
+  smem_passes<false, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP);
   // last forward pass, product with the spectrum column, first inverse pass (same radix), in
   // registers; the inverse then runs its radix-E passes
   const int lr0 = fft_logr<LOGE>(np - 1, a.logH);
@@ -287,7 +446,7 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
     conv_mid_dispatch<NF, LOGE>(lr0, sm, fb, j, tpf, a.logH, tw, a.logP, spec_mul);
   }
   for (int p = 1; p < np - 1; ++p)
-    smem_pass<LOGE, true, NF, LOGE>(sm, fb, j, tpf, a.logH, lr0 + LOGE * (p - 1), tw, a.logP, Identity{});
+    smem_pass<LOGE, true, NF, LOGE>(sm, fb, j, tpf, a.logH, lr0 + LOGE * (p - 1), tw, a.logP);
   // last inverse pass (radix E, Ns = H/E) recombines y[n] = A[n] + conj(w^n) B[n] for kept rows
   last_pass<LOGE, true, NF, LOGE>(sm, fb, j, tpf, a.logH, a.logH - LOGE, tw, a.logP, [&](int nn, const T2 (&v)[NF]) {
     const T2 y = recombine<TPT>(v, half, tw, nn);
@@ -297,6 +456,7 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
 
 template <typename CT, int TPT, int LOGE>
 __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_col_conv(ColArgs a) {
+  grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   // with many channels they run along x: the channels of one column tile run back to back and
   // share its spectrum column through L2 (64 right-hand sides: 2.82 -> 2.67 ms per launch);
@@ -319,7 +479,29 @@ struct RowInvArgs {
   int logH, logP, row_lo, nrows;
   double scale;
   int rows_per_cta;
+  int qcut;            // as in RowFwdArgs
+  int sparse;
 };
+
+// value of another lane (xor of the lane index); all 32 lanes call it together
+__device__ __forceinline__ float2 shfl_xor_c(float2 v, int off) {
+  return float2{__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off)};
+}
+__device__ __forceinline__ double2 shfl_xor_c(double2 v, int off) {
+  return double2{__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off)};
+}
+__device__ __forceinline__ dfc shfl_xor_c(dfc v, int off) {
+  dfc r;
+  r.xh = __shfl_xor_sync(0xffffffffu, v.xh, off);
+  r.yh = __shfl_xor_sync(0xffffffffu, v.yh, off);
+  r.xl = __shfl_xor_sync(0xffffffffu, v.xl, off);
+  r.yl = __shfl_xor_sync(0xffffffffu, v.yl, off);
+  return r;
+}
+
+// Lanes that share one active point of a sparse row: four terms of its sum each (with one term each
+// a point costs more in the shuffle tree than in products), at least two lanes.
+__device__ __forceinline__ int sparse_point_lanes(int k2) { return max(2, k2 >> 2); }
 
 // One work item of the inverse row pass: rows [row_block * rows_per_cta, +rows_per_cta) of channel c.
 template <typename CT, int TPT, int LOGE>
@@ -341,17 +523,53 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
 #pragma unroll
   for (int f = 0; f < NF; ++f) fb[f] = (2 * g + (TPT == 1 ? half : f)) * HS;
   const T2* blk = static_cast<const T2*>(a.inter) + (size_t)c * P * a.nrows;
+  // sparse rows: the CTA's active points, flat over its rows, lpp lanes each; the first
+  // round's point and its root are loaded here, so that their latency overlaps the transforms
+  const int lpp = sparse_point_lanes(sparse_geom<LOGE>(a.logH).k2);
+  int A0 = 0, A1 = 0, ix0 = 0;
+  T2 z0 = czero<T2>();
+  int* rps = reinterpret_cast<int*>(sm + 2 * a.rows_per_cta * HS);
+  if (a.sparse) {
+    const int row0 = row_block * a.rows_per_cta;
+    A0 = a.row_ptr[a.row_lo + row0];
+    A1 = a.row_ptr[a.row_lo + min(row0 + a.rows_per_cta, a.nrows)];
+    for (int i = threadIdx.x; i <= a.rows_per_cta; i += blockDim.x) rps[i] = a.row_ptr[a.row_lo + min(row0 + i, a.nrows)];
+  }
+  grid_dependency_wait();
   // pass 0 (inverse, radix E, Ns = 1) from global: Y[2k] and/or Y[2k+1]
   {
     const int lognb = a.logH - LOGE;
     T2 v[NF][1 << LOGE];
 #pragma unroll
     for (int r = 0; r < (1 << LOGE); ++r) {
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        const int q = 2 * (j + (r << lognb)) + (TPT == 1 ? half : f);
-        v[f][r] = live ? blk[((size_t)(q / W) * a.nrows + rloc) * W + (q % W)] : czero<T2>();
+      // every load is issued (from the channel's first tile where there is nothing to load) before
+      // any value is looked at: a branch or a select per load would expose its latency 2^LOGE times
+      if constexpr (TPT == 2) {
+        // Y[2k] and Y[2k + 1] are neighbours in a tile: one vector load
+        const int q = 2 * (j + (r << lognb));
+        const bool ok = live && min(q, P - 1 - q) <= a.qcut;
+        load_pair(&blk[ok ? ((size_t)(q / W) * a.nrows + rloc) * W + (q % W) : 0], v[0][r], v[1][r]);
+      } else {
+        const int q = 2 * (j + (r << lognb)) + half;
+        const bool ok = live && min(q, P - q) <= a.qcut;
+        v[0][r] = blk[ok ? ((size_t)(q / W) * a.nrows + rloc) * W + (q % W) : 0];
       }
+    }
+    if (a.sparse) {   // behind the loads above: their latencies overlap
+      const int ap = A0 + threadIdx.x / lpp;
+      if (ap < A1) {
+        ix0 = a.act_ix[ap];
+        z0 = ldro(&tw[ix0]);
+      }
+    }
+    if (!live || a.qcut < (P >> 1)) {   // zero the columns beyond the mask's disc
+#pragma unroll
+      for (int r = 0; r < (1 << LOGE); ++r)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          const int q = 2 * (j + (r << lognb)) + (TPT == 1 ? half : f);
+          if (!live || min(q, P - q) > a.qcut) v[f][r] = czero<T2>();
+        }
     }
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -361,8 +579,46 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
     }
     __syncthreads();
   }
+  if (a.sparse) {
+    const int logj = sparse_logj<LOGE>(a.logH), J = 1 << logj, k2 = 2 << (a.logH - logj), tpl = k2 / lpp;
+    if (logj > LOGE) smem_pass<LOGE, true, NF, LOGE>(sm, fb, j, tpf, a.logH, LOGE, tw, a.logP);
+    // now sub-transform k1 of half h holds its J outputs at k1 J of the half's buffer, and
+    //     y[n] = sum over k' = 2 k1 + h of Z_h[k1][n mod J] W_P^{-n k'}:
+    // each lane of a point sums tpl consecutive k' by Horner's rule in W_P^{-n}, and the lanes add
+    // up over a fixed shuffle tree (the order depends on the transform length alone)
+    const int l = threadIdx.x & (lpp - 1), grp = threadIdx.x / lpp, ngrp = blockDim.x / lpp;
+    using VP = decltype(VT::x);
+    VP* out = static_cast<VP*>(a.vact) + 2 * (size_t)c * a.n_act;
+    for (int base = A0; base < A1; base += ngrp) {
+      const int ap = base + grp;
+      const bool valid = ap < A1;
+      T2 acc = czero<T2>();
+      if (valid) {
+        const int ix = base == A0 ? ix0 : a.act_ix[ap];
+        const T2 z = base == A0 ? z0 : ldro(&tw[ix]);
+        int lo = 0, hi = a.rows_per_cta;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (rps[mid] <= ap) lo = mid; else hi = mid;
+        }
+        const T2* zb = sm + (size_t)(2 * lo) * HS;
+        const int jj = ix & (J - 1), k0 = l * tpl;
+        for (int t = tpl - 1; t >= 0; --t) {
+          const int kk = k0 + t;
+          const T2 v = zb[(kk & 1) * HS + padi<LOGE>(((kk >> 1) << logj) + jj)];
+          acc = t == tpl - 1 ? v : cadd(cmulc(acc, z), v);
+        }
+        acc = cmulc(acc, ldro(&tw[(ix * k0) & (P - 1)]));
+      }
+      for (int off = lpp >> 1; off > 0; off >>= 1) acc = cadd(acc, shfl_xor_c(acc, off));
+      // lane 0 stores the real part, lane 1 the imaginary part (every lane holds the sum): the
+      // conversions of the double-float types run at the FP64 rate, once per component and warp
+      if (valid && l < 2) out[2 * ap + l] = cto_vt_part(acc, l, a.scale);
+    }
+    return;
+  }
   const int np = fft_npass<LOGE>(a.logH);
-  smem_passes<true, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP, Identity{});
+  smem_passes<true, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP);
   int logNs = 0;
   for (int p = 0; p < np - 1; ++p) logNs += fft_logr<LOGE>(p, a.logH);
   const double sc = a.scale;
@@ -377,7 +633,7 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
   // sparse mode: the last pass as one more shared-memory pass leaves both half-transforms in
   // natural order in their own buffers, and the recombination y = Y_even + w^-n Y_odd runs only
   // at the row's active points (tens of the H outputs)
-  smem_passes<true, NF, LOGE>(sm, fb, j, tpf, a.logH, np - 1, np, logNs, tw, a.logP, Identity{});
+  smem_passes<true, NF, LOGE>(sm, fb, j, tpf, a.logH, np - 1, np, logNs, tw, a.logP);
   if (live) {
     VT* out = static_cast<VT*>(a.vact) + (size_t)c * a.n_act;
     const int a1 = a.row_ptr[iy + 1];
@@ -391,6 +647,7 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
 
 template <typename CT, int TPT, int LOGE>
 __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_row_inv(RowInvArgs a) {
+  grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   row_inv_item<CT, TPT, LOGE>(a, blockIdx.x, blockIdx.y, smraw);
 }
@@ -400,133 +657,171 @@ __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_row_inv(Row
 // ------------------------------------------------------------------------------------
 struct GatherArgs {
   const void* vact;
-  int n_act, n, nrhs, nproj;
+  int n_act, n, nrhs;
   const int* ga_ptr;
   const int* ga_act;
   const double* w[kMaxProj];
-  double2 coef[kMaxProj];
+  double coef[kMaxProj];
   const int* nptr;
   const int* ncol;
   const void* nval;
   const double2* x;
   double2 out_scale;
   double2* y;
-  int accumulate;
 };
 
-// A group of kGatherLanes adjacent lanes per unknown i and block of up to kGatherRhs right-hand
-// sides (1 when there is only one), four groups to a warp: the CSR entries of row i (weights,
-// active-point indices, near-field values and columns) are loaded once and used for every
-// right-hand side of the block. For each right-hand side, lane g of the group sums the entries
-// e = e0 + g, e0 + g + 8, ... in order, and the group then adds its partial sums by xor shuffles,
-// so the result does not depend on the block size. The FP64 pipe sets the cost here: a whole
-// warp per unknown spent more FP64 instructions on coefficient products and its five-step
-// shuffle tree than on the entries themselves. With a complex64 grid (mixed precision) the
-// projection sums run in FP32 (Acc): converting every grid value to FP64 cost as much as the
-// FP64 products, conversions running at the FP64 rate here. The coefficient products, the
-// near-field rows and the sums over projections stay in FP64.
+// A group of kGatherLanes adjacent lanes per unknown i and block of up to RB right-hand sides, four
+// groups to a warp: the CSR entries of row i (weights, active-point indices, near-field values and
+// columns) are loaded once and used for every right-hand side of the block. For each right-hand
+// side, lane g of the group sums the entries e = e0 + g, e0 + g + 8, ... in order, projection by
+// projection, and the group then adds its partial sums over a fixed tree, so the result does not
+// depend on the block size. The FP64 pipe (1/64 of the FP32 rate, shared by the whole SM) sets the
+// cost: the tree halves the values a lane still carries at each step (at xor distance 4, a lane
+// keeps the right-hand sides of its half and passes the others on) instead of adding all of them
+// in every lane, 14 additions for eight right-hand sides instead of 48, and small products spread
+// over many short CTAs (gather_threads) so that they use many SMs' pipes. With a complex64 grid
+// (mixed precision) the projection sums run in FP32 (Acc): converting every grid value to FP64 cost
+// as much as the FP64 products. The coefficient products, the near-field rows and the sums over
+// projections stay in FP64.
 constexpr int kGatherLanes = 8;
 
 // Gather for the threads of virtual block `vblock` (blockDim.x threads each); all 32 lanes of every
 // warp call it (the group sums are shuffles).
-template <typename T2, int kGatherRhs>
+template <typename T2, int NP, int RB>
 __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vblock) {
-  static_assert(kGatherRhs <= kGatherLanes, "lane g writes right-hand side r0 + g");
+  static_assert(RB == 1 || RB == 2 || RB == 4 || RB == 8, "a power of two of at most kGatherLanes");
   using Acc = typename std::conditional<std::is_same<T2, float2>::value, float, double>::type;
   const long long grp = (vblock * blockDim.x + threadIdx.x) / kGatherLanes;
   const int g = threadIdx.x & (kGatherLanes - 1);
-  const int nblk = (a.nrhs + kGatherRhs - 1) / kGatherRhs;
+  const int nblk = (a.nrhs + RB - 1) / RB;
   const bool valid = grp < (long long)a.n * nblk;
   const int rb = valid ? (int)(grp / a.n) : 0, i = valid ? (int)(grp - (long long)rb * a.n) : 0;
-  const int r0 = rb * kGatherRhs, nr = min(kGatherRhs, a.nrhs - r0);
-  double re[kGatherRhs], im[kGatherRhs];
+  const int r0 = rb * RB, nr = min(RB, a.nrhs - r0);
+  double re[RB], im[RB];
 #pragma unroll
-  for (int q = 0; q < kGatherRhs; ++q) re[q] = im[q] = 0.0;
+  for (int q = 0; q < RB; ++q) re[q] = im[q] = 0.0;
   if (valid) {
     const int e0 = a.ga_ptr[i], e1 = a.ga_ptr[i + 1];
-    for (int pj = 0; pj < a.nproj; ++pj) {
-      const T2* v = static_cast<const T2*>(a.vact) + (size_t)(pj * a.nrhs + r0) * a.n_act;
-      const double* w = a.w[pj];
-      Acc cr[kGatherRhs], ci[kGatherRhs];
+    const T2* v = static_cast<const T2*>(a.vact) + (size_t)r0 * a.n_act;
+    // one or two right-hand sides: all projections of an entry together (their loads are
+    // independent); more: projection by projection, which keeps the sums in registers. The sums
+    // of a projection run over the same entries in the same order either way.
+    constexpr int PG = RB <= 2 ? NP : 1;
 #pragma unroll
-      for (int q = 0; q < kGatherRhs; ++q) cr[q] = ci[q] = Acc(0);
+    for (int p0 = 0; p0 < NP; p0 += PG) {
+      Acc cr[PG][RB], ci[PG][RB];
+#pragma unroll
+      for (int p = 0; p < PG; ++p)
+#pragma unroll
+        for (int q = 0; q < RB; ++q) cr[p][q] = ci[p][q] = Acc(0);
+#pragma unroll 2
       for (int e = e0 + g; e < e1; e += kGatherLanes) {
-        const Acc ww = static_cast<Acc>(w[e]);
         const int act = a.ga_act[e];
 #pragma unroll
-        for (int q = 0; q < kGatherRhs; ++q) {
-          if (q < nr) {
-            const T2 val = v[(size_t)q * a.n_act + act];
-            cr[q] = fma(ww, static_cast<Acc>(val.x), cr[q]);
-            ci[q] = fma(ww, static_cast<Acc>(val.y), ci[q]);
+        for (int p = 0; p < PG; ++p) {
+          const Acc ww = static_cast<Acc>(a.w[p0 + p][e]);
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            if (q < nr) {
+              const T2 val = v[((size_t)(p0 + p) * a.nrhs + q) * a.n_act + act];
+              cr[p][q] = fma(ww, static_cast<Acc>(val.x), cr[p][q]);
+              ci[p][q] = fma(ww, static_cast<Acc>(val.y), ci[p][q]);
+            }
           }
         }
       }
-      const double2 cf = a.coef[pj];
 #pragma unroll
-      for (int q = 0; q < kGatherRhs; ++q) {
-        const double crq = cr[q], ciq = ci[q];
-        re[q] += cf.x * crq - cf.y * ciq;
-        im[q] += cf.x * ciq + cf.y * crq;
+      for (int p = 0; p < PG; ++p) {
+        const double cf = a.coef[p0 + p];
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          re[q] = fma(cf, (double)cr[p][q], re[q]);
+          im[q] = fma(cf, (double)ci[p][q], im[q]);
+        }
       }
     }
     if (a.nptr != nullptr) {
       const T2* val = static_cast<const T2*>(a.nval);
       const int n1 = a.nptr[i + 1];
+#pragma unroll 2
       for (int e = a.nptr[i] + g; e < n1; e += kGatherLanes) {
         const T2 cv = val[e];
+        const double cx = cv.x, cy = cv.y;
         const int col = a.ncol[e];
 #pragma unroll
-        for (int q = 0; q < kGatherRhs; ++q) {
+        for (int q = 0; q < RB; ++q) {
           if (q < nr) {
             const double2 xx = a.x[(size_t)(r0 + q) * a.n + col];
-            re[q] += (double)cv.x * xx.x - (double)cv.y * xx.y;
-            im[q] += (double)cv.x * xx.y + (double)cv.y * xx.x;
+            re[q] = fma(cx, xx.x, fma(-cy, xx.y, re[q]));
+            im[q] = fma(cx, xx.y, fma(cy, xx.x, im[q]));
           }
         }
       }
     }
   }
-  // every lane of the warp takes part in the shuffles (groups past the end carry zeros)
+  // the tree: cnt right-hand sides left per lane; at each step a lane with bit `off` set keeps the
+  // upper half of them (every lane of the warp takes part; groups past the end carry zeros)
+  int q0 = 0;
 #pragma unroll
-  for (int q = 0; q < kGatherRhs; ++q) {
+  for (int off = kGatherLanes / 2, cnt = RB; off > 0; off >>= 1) {
+    if (cnt > 1) {
+      cnt >>= 1;
+      const bool up = (g & off) != 0;
+      if (up) q0 += cnt;
 #pragma unroll
-    for (int off = kGatherLanes / 2; off > 0; off >>= 1) {
-      re[q] += __shfl_xor_sync(0xffffffffu, re[q], off);
-      im[q] += __shfl_xor_sync(0xffffffffu, im[q], off);
+      for (int q = 0; q < cnt; ++q) {
+        const double sr = up ? re[q] : re[q + cnt], si = up ? im[q] : im[q + cnt];
+        const double kr = up ? re[q + cnt] : re[q], ki = up ? im[q + cnt] : im[q];
+        re[q] = kr + __shfl_xor_sync(0xffffffffu, sr, off);
+        im[q] = ki + __shfl_xor_sync(0xffffffffu, si, off);
+      }
+    } else {
+      re[0] += __shfl_xor_sync(0xffffffffu, re[0], off);
+      im[0] += __shfl_xor_sync(0xffffffffu, im[0], off);
     }
   }
-  if (valid && g < nr) {
-    // lane g writes right-hand side r0 + g (select by unrolled compare: no local-memory indexing)
-    double xr = 0.0, xi = 0.0;
-#pragma unroll
-    for (int q = 0; q < kGatherRhs; ++q)
-      if (q == g) { xr = re[q]; xi = im[q]; }
+  if (valid && (g & (kGatherLanes / RB - 1)) == 0 && q0 < nr) {
     const double2 s = a.out_scale;
-    double2 o = double2{s.x * xr - s.y * xi, s.x * xi + s.y * xr};
-    double2* dst = a.y + (size_t)(r0 + g) * a.n + i;
-    if (a.accumulate) {
-      const double2 prev = *dst;
-      o.x += prev.x;
-      o.y += prev.y;
-    }
-    *dst = o;
+    a.y[(size_t)(r0 + q0) * a.n + i] =
+        double2{fma(s.x, re[0], -(s.y * im[0])), fma(s.x, im[0], s.y * re[0])};
   }
 }
 
-template <typename T2, int kGatherRhs>
-__global__ void k_gather(GatherArgs a) {
-  gather_item<T2, kGatherRhs>(a, blockIdx.x);
+template <typename T2, int NP, int RB>
+__global__ void __launch_bounds__(256) k_gather(GatherArgs a) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
+  gather_item<T2, NP, RB>(a, blockIdx.x);
 }
+
+// Threads of a gather CTA: 256, fewer while that leaves fewer CTAs than twice the SMs.
+inline int gather_threads(long long threads) {
+  int tpb = 256;
+  while (tpb > 32 && threads / tpb < 304) tpb >>= 1;
+  return tpb;
+}
+
+// Right-hand sides of a gather group: the power of two at or above their number, at most 8 (64
+// lanes' worth of sums would spill).
+inline int gather_rhs_block(int nrhs) { return nrhs >= 5 ? 8 : nrhs >= 3 ? 4 : nrhs; }
 
 // ------------------------------------------------------------------------------------
 // launch configuration
 // ------------------------------------------------------------------------------------
+// Raises a kernel's dynamic shared memory limit; the context remembers what it has raised.
 template <typename K>
-static aim_status ensure_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) {
-    AIM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  }
+static aim_status ensure_smem(aim_ctx* ctx, K kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return AIM_OK;
+  const void* id = reinterpret_cast<const void*>(kernel);
+  for (auto& kb : ctx->smem_raised)
+    if (kb.first == id && kb.second >= bytes) return AIM_OK;
+  AIM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  for (auto& kb : ctx->smem_raised)
+    if (kb.first == id) {
+      kb.second = bytes;
+      return AIM_OK;
+    }
+  ctx->smem_raised.emplace_back(id, bytes);
   return AIM_OK;
 }
 
@@ -596,7 +891,7 @@ static bool feasible_for(const Schedule& s, int logH, int logP) {
 }
 
 template <typename CT, int TPT, int LOGE>
-static aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdArgs fa, RowInvArgs ia,
+aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdArgs fa, RowInvArgs ia,
                              void* inter, const Schedule& sc, cudaStream_t st) {
   const int min_row_threads = sc.min_row_threads;
   using T2 = CT;
@@ -613,7 +908,10 @@ static aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdAr
          2 * rpc * LPT * tpf <= LaunchMax<CT, TPT, LOGE>::value)
     rpc *= 2;
   const int row_blocks = (ctx->nrows + rpc - 1) / rpc;
-  const size_t sm_row = 2 * (size_t)rpc * HS * sizeof(T2);
+  const int sparse = !fa.dense && sparse_rows<LOGE>(ctx);
+  const size_t sm_row =
+      2 * (size_t)rpc * HS * sizeof(T2) + (sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
+  const int qcut = filtered ? ctx->qcut : ctx->H;
 
   fa.tw = tw;
   fa.logH = ctx->logH;
@@ -622,12 +920,13 @@ static aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdAr
   fa.nrows = ctx->nrows;
   fa.inter = inter;
   fa.rows_per_cta = rpc;
-  AIM_TRY(ensure_smem(k_row_fwd<CT, TPT, LOGE>, sm_row));
+  fa.qcut = qcut;
+  fa.sparse = sparse;
+  AIM_TRY(ensure_smem(ctx, k_row_fwd<CT, TPT, LOGE>, sm_row));
   {
     ProfScope ps(K_ROW_FWD, st);
-    k_row_fwd<CT, TPT, LOGE><<<dim3(row_blocks, channels), rpc * LPT * tpf, sm_row, st>>>(fa);
+    AIM_TRY(launch_chained(k_row_fwd<CT, TPT, LOGE>, dim3(row_blocks, channels), rpc * LPT * tpf, sm_row, st, fa));
   }
-  AIM_CUDA_TRY(cudaGetLastError());
 
   // column pass
   const int cols = col_cols_of<CT, TPT, LOGE>(sc, ctx->logH, ctx->logP);
@@ -636,7 +935,7 @@ static aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdAr
   ColArgs ca;
   ca.inter = inter;
   ca.spec = spec;
-  ca.live = filtered ? ctx->specA_live : nullptr;
+  ca.qcut = qcut;
   ca.tw = tw;
   ca.logH = ctx->logH;
   ca.logP = ctx->logP;
@@ -646,14 +945,13 @@ static aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdAr
   const size_t sm_col = 2 * (size_t)cols * HS * sizeof(T2);
   if (ctx->P / cols > 65535) return fail(AIM_EINVAL, "too many column tiles for one column-pass grid");
   constexpr int kChanX = 8;   // channels from which the column-pass grid runs channels along x
-  AIM_TRY(ensure_smem(k_col_conv<CT, TPT, LOGE>, sm_col));
+  AIM_TRY(ensure_smem(ctx, k_col_conv<CT, TPT, LOGE>, sm_col));
   {
     ProfScope ps(K_COL_CONV, st);
     ca.chan_x = channels >= kChanX;
     const dim3 grid = ca.chan_x ? dim3(channels, ctx->P / cols) : dim3(ctx->P / cols, channels);
-    k_col_conv<CT, TPT, LOGE><<<grid, cols * LPT * tpf, sm_col, st>>>(ca);
+    AIM_TRY(launch_chained(k_col_conv<CT, TPT, LOGE>, grid, cols * LPT * tpf, sm_col, st, ca));
   }
-  AIM_CUDA_TRY(cudaGetLastError());
 
   // row inverse
   ia.inter = inter;
@@ -664,12 +962,13 @@ static aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdAr
   ia.nrows = ctx->nrows;
   ia.scale = 1.0 / ((double)ctx->P * (double)ctx->P);
   ia.rows_per_cta = rpc;
-  AIM_TRY(ensure_smem(k_row_inv<CT, TPT, LOGE>, sm_row));
+  ia.qcut = qcut;
+  ia.sparse = sparse;
+  AIM_TRY(ensure_smem(ctx, k_row_inv<CT, TPT, LOGE>, sm_row));
   {
     ProfScope ps(K_ROW_INV, st);
-    k_row_inv<CT, TPT, LOGE><<<dim3(row_blocks, channels), rpc * LPT * tpf, sm_row, st>>>(ia);
+    AIM_TRY(launch_chained(k_row_inv<CT, TPT, LOGE>, dim3(row_blocks, channels), rpc * LPT * tpf, sm_row, st, ia));
   }
-  AIM_CUDA_TRY(cudaGetLastError());
   return AIM_OK;
 }
 
@@ -693,42 +992,28 @@ static aim_status launch_three_passes(aim_ctx* ctx, int channels, bool filtered,
   }
 }
 
+inline AntArgs ant_args(const aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2* x) {
+  AntArgs aa{};
+  aa.x = x;
+  aa.n = ctx->n;
+  aa.nrhs = nrhs;
+  aa.n_act = ctx->n_act;
+  aa.sc_ptr = ctx->prj.sc_ptr;
+  aa.sc_col = ctx->prj.sc_col;
+  for (int pj = 0; pj < spec.nproj; ++pj) aa.w[pj] = ctx->prj.sc_w[spec.proj[pj]];
+  // u and the restricted values are never alive together: the inverse row pass starts when the
+  // forward row pass, the last reader of u, is long complete
+  aa.u = ctx->vact;
+  return aa;
+}
+
 template <typename CT>
-aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2* x, double2* y,
-                     cudaStream_t st) {
-  using VT = typename GridT<CT>::VT;
-  const int precision = precision_of((CT*)nullptr);
-  const int channels = spec.nproj * nrhs;
-  if (inter_bytes_needed(ctx, channels, precision) > ctx->inter_bytes ||
-      (size_t)channels * ctx->n_act * sizeof(VT) > ctx->vact_bytes)
-    return fail(AIM_ESTATE, "grid workspace not reserved for this many right-hand sides");
-
-  RowFwdArgs fa{};
-  fa.x = x;
-  fa.dense = 0;
-  fa.n = ctx->n;
-  fa.m = ctx->m;
-  fa.nrhs = nrhs;
-  fa.row_ptr = ctx->row_ptr;
-  fa.act_ix = ctx->act_ix;
-  fa.sc_ptr = ctx->prj.sc_ptr;
-  fa.sc_col = ctx->prj.sc_col;
-  for (int pj = 0; pj < spec.nproj; ++pj) fa.w[pj] = ctx->prj.sc_w[spec.proj[pj]];
-  RowInvArgs ia{};
-  ia.vact = ctx->vact;
-  ia.dense = 0;
-  ia.m = ctx->m;
-  ia.n_act = ctx->n_act;
-  ia.row_ptr = ctx->row_ptr;
-  ia.act_ix = ctx->act_ix;
-  AIM_TRY(launch_three_passes<CT>(ctx, channels, spec.filtered, fa, ia, ctx->inter, st));
-
+GatherArgs gather_args(const aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2* x, double2* y) {
   GatherArgs ga{};
   ga.vact = ctx->vact;
   ga.n_act = ctx->n_act;
   ga.n = ctx->n;
   ga.nrhs = nrhs;
-  ga.nproj = spec.nproj;
   ga.ga_ptr = ctx->prj.ga_ptr;
   ga.ga_act = ctx->prj.ga_act;
   for (int pj = 0; pj < spec.nproj; ++pj) {
@@ -743,20 +1028,60 @@ aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2
   ga.x = x;
   ga.out_scale = spec.out_scale;
   ga.y = y;
-  ga.accumulate = 0;
-  constexpr int kRhsBlock = 8;
-  const int rb = nrhs == 1 ? 1 : kRhsBlock;
-  const long long groups = (long long)ctx->n * ((nrhs + rb - 1) / rb);
-  const int tpb = 256;
-  const long long blocks = (groups * kGatherLanes + tpb - 1) / tpb;
+  return ga;
+}
+
+template <typename CT>
+aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2* x, double2* y,
+                     cudaStream_t st) {
+  using VT = typename GridT<CT>::VT;
+  const int precision = precision_of((CT*)nullptr);
+  const int channels = spec.nproj * nrhs;
+  if (inter_bytes_needed(ctx, channels, precision) > ctx->inter_bytes ||
+      (size_t)channels * ctx->n_act * sizeof(VT) > ctx->vact_bytes)
+    return fail(AIM_ESTATE, "grid workspace not reserved for this many right-hand sides");
+
+  const AntArgs aa = ant_args(ctx, spec, nrhs, x);
+  {
+    ProfScope ps(K_ANTERP, st);
+    const long long blocks = ((long long)ctx->n_act * nrhs + kAntThreads - 1) / kAntThreads;
+    AIM_TRY(launch_chained(spec.nproj == 1 ? k_anterpolate<CT, 1> : k_anterpolate<CT, 3>, dim3((unsigned)blocks),
+                           kAntThreads, 0, st, aa));
+  }
+  RowFwdArgs fa{};
+  fa.u = ctx->vact;
+  fa.dense = 0;
+  fa.m = ctx->m;
+  fa.n_act = ctx->n_act;
+  fa.row_ptr = ctx->row_ptr;
+  fa.act_ix = ctx->act_ix;
+  RowInvArgs ia{};
+  ia.vact = ctx->vact;
+  ia.dense = 0;
+  ia.m = ctx->m;
+  ia.n_act = ctx->n_act;
+  ia.row_ptr = ctx->row_ptr;
+  ia.act_ix = ctx->act_ix;
+  AIM_TRY(launch_three_passes<CT>(ctx, channels, spec.filtered, fa, ia, ctx->inter, st));
+
+  const GatherArgs ga = gather_args<CT>(ctx, spec, nrhs, x, y);
+  const int rb = gather_rhs_block(nrhs);
+  const long long threads = (long long)ctx->n * ((nrhs + rb - 1) / rb) * kGatherLanes;
+  const int tpb = gather_threads(threads);
+  const dim3 blocks((unsigned)((threads + tpb - 1) / tpb));
   {
     ProfScope ps(K_GATHER, st);
-    if (rb == 1)
-      k_gather<VT, 1><<<(unsigned)blocks, tpb, 0, st>>>(ga);
-    else
-      k_gather<VT, kRhsBlock><<<(unsigned)blocks, tpb, 0, st>>>(ga);
+    auto run = [&](auto np) {
+      constexpr int NP = decltype(np)::value;
+      switch (rb) {
+        case 1: return launch_chained(k_gather<VT, NP, 1>, blocks, tpb, 0, st, ga);
+        case 2: return launch_chained(k_gather<VT, NP, 2>, blocks, tpb, 0, st, ga);
+        case 4: return launch_chained(k_gather<VT, NP, 4>, blocks, tpb, 0, st, ga);
+        default: return launch_chained(k_gather<VT, NP, 8>, blocks, tpb, 0, st, ga);
+      }
+    };
+    AIM_TRY(spec.nproj == 1 ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 3>{}));
   }
-  AIM_CUDA_TRY(cudaGetLastError());
   return AIM_OK;
 }
 
@@ -764,8 +1089,8 @@ aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2
 // several grid passes (contexts of any size) in one persistent launch
 // ------------------------------------------------------------------------------------
 // One job is a whole grid pass of one context (its channels, its spectrum, its gather). The
-// persistent kernel runs four phases over all jobs' work items: forward row pass, column pass,
-// inverse row pass, gather. Every CTA takes items c, c + G, c + 2G, ... of the flattened item list
+// persistent kernel runs five phases over all jobs' work items: anterpolation, forward row pass,
+// column pass, inverse row pass, gather. Every CTA takes items c, c + G, c + 2G, ... of the flattened item list
 // of a phase (G = CTAs of the launch); each item fills the CTA's threads with lines (rows or
 // columns) of its job, so a job with a shorter transform puts more lines into one item. A grid
 // barrier separates the phases. The launch is cooperative, so all CTAs are resident and the
@@ -774,6 +1099,7 @@ aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2
 constexpr int kMaxMultiJobs = 32;
 
 struct MultiJob {
+  AntArgs aa;
   RowFwdArgs fa;
   ColArgs ca;
   RowInvArgs ia;
@@ -782,7 +1108,8 @@ struct MultiJob {
   int col_items;       // column tiles per channel
   int channels;
   int tile_major;      // column items ordered tile by tile (the channels of a tile adjacent)
-  int gather_rb;       // right-hand sides per gather group (1 or 8)
+  int nproj;           // 1 or 3
+  int gather_rb;       // right-hand sides per gather group
 };
 
 // The whole job table travels as the kernel's parameter (read-only, in the constant bank: a
@@ -790,7 +1117,7 @@ struct MultiJob {
 struct MultiArgs {
   MultiJob jobs[kMaxMultiJobs];
   int njobs;
-  long long off[4][kMaxMultiJobs + 1];   // prefix sums of the items of each phase over the jobs
+  long long off[5][kMaxMultiJobs + 1];   // prefix sums of the items of each phase over the jobs
   unsigned* bar;                         // [arrivals, generation], zero at launch
   int* err;                              // 1 when a barrier wait gave up
   long long max_spins;
@@ -832,7 +1159,7 @@ template <typename CT, int TPT, int LOGE>
 __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_grid_multi(const __grid_constant__ MultiArgs m) {
   using VT = typename GridT<CT>::VT;
   extern __shared__ __align__(16) unsigned char smraw[];
-  for (int phase = 0; phase < 4; ++phase) {
+  for (int phase = 0; phase < 5; ++phase) {
     const long long total = m.off[phase][m.njobs];
     for (long long it = blockIdx.x; it < total; it += gridDim.x) {
       int jb = 0;
@@ -840,23 +1167,30 @@ __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_grid_multi(
       const MultiJob& J = m.jobs[jb];
       const long long local = it - m.off[phase][jb];
       if (phase == 0) {
-        row_fwd_item<CT, TPT, LOGE>(J.fa, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
+        const long long t = local * blockDim.x + threadIdx.x;
+        if (J.nproj == 1) ant_item<CT, 1>(J.aa, t); else ant_item<CT, 3>(J.aa, t);
       } else if (phase == 1) {
+        row_fwd_item<CT, TPT, LOGE>(J.fa, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
+      } else if (phase == 2) {
         // many channels (right-hand sides): the channels of one column tile run back to back and
         // share its spectrum column through L2, as the single-context launch orders them
         const int tile = J.tile_major ? (int)(local / J.channels) : (int)(local % J.col_items);
         const int ch = J.tile_major ? (int)(local % J.channels) : (int)(local / J.col_items);
         col_conv_item<CT, TPT, LOGE>(J.ca, tile, ch, smraw);
-      } else if (phase == 2) {
+      } else if (phase == 3) {
         row_inv_item<CT, TPT, LOGE>(J.ia, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
-      } else if (J.gather_rb == 1) {
-        gather_item<VT, 1>(J.ga, local);
       } else {
-        gather_item<VT, 8>(J.ga, local);
+        auto gather = [&](auto np) {
+          constexpr int NP = decltype(np)::value;
+          if (J.gather_rb == 1) gather_item<VT, NP, 1>(J.ga, local);
+          else if (J.gather_rb == 4) gather_item<VT, NP, 4>(J.ga, local);
+          else gather_item<VT, NP, 8>(J.ga, local);
+        };
+        if (J.nproj == 1) gather(std::integral_constant<int, 1>{}); else gather(std::integral_constant<int, 3>{});
       }
       __syncthreads();   // the next item reuses the shared memory
     }
-    if (phase < 3 && !multi_grid_barrier(m)) return;
+    if (phase < 4 && !multi_grid_barrier(m)) return;
   }
 }
 
@@ -916,20 +1250,19 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
     if (inter_bytes_needed(ctx, channels, precision) > ctx->inter_bytes ||
         (size_t)channels * ctx->n_act * sizeof(VT) > ctx->vact_bytes)
       return fail(AIM_ESTATE, "grid workspace not reserved for this many right-hand sides");
-    smem = std::max(smem, 2 * (size_t)lines * HS * sizeof(T2));
+    const int sparse = sparse_rows<LOGE>(ctx), qcut = spec.filtered ? ctx->qcut : ctx->H;
+    smem = std::max(smem, 2 * (size_t)lines * HS * sizeof(T2) + (sparse ? sparse_smem<CT, LOGE>(ctx->logH, lines) : 0));
     MultiJob& J = m.jobs[i];
     const void* tw = twiddles(ctx, (CT*)nullptr);
+    J.aa = ant_args(ctx, spec, ps.nrhs, ps.x);
+    J.nproj = spec.nproj;
     RowFwdArgs& fa = J.fa;
-    fa.x = ps.x;
+    fa.u = ctx->vact;
     fa.dense = 0;
-    fa.n = ctx->n;
     fa.m = ctx->m;
-    fa.nrhs = ps.nrhs;
+    fa.n_act = ctx->n_act;
     fa.row_ptr = ctx->row_ptr;
     fa.act_ix = ctx->act_ix;
-    fa.sc_ptr = ctx->prj.sc_ptr;
-    fa.sc_col = ctx->prj.sc_col;
-    for (int pj = 0; pj < spec.nproj; ++pj) fa.w[pj] = ctx->prj.sc_w[spec.proj[pj]];
     fa.inter = ctx->inter;
     fa.tw = tw;
     fa.logH = ctx->logH;
@@ -937,10 +1270,12 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
     fa.row_lo = ctx->row_lo;
     fa.nrows = ctx->nrows;
     fa.rows_per_cta = lines;
+    fa.qcut = qcut;
+    fa.sparse = sparse;
     ColArgs& ca = J.ca;
     ca.inter = ctx->inter;
     ca.spec = spectrum(ctx, spec.filtered, (CT*)nullptr);
-    ca.live = spec.filtered ? ctx->specA_live : nullptr;
+    ca.qcut = qcut;
     ca.tw = tw;
     ca.logH = ctx->logH;
     ca.logP = ctx->logP;
@@ -965,42 +1300,25 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
     ia.nrows = ctx->nrows;
     ia.scale = 1.0 / ((double)P * (double)P);
     ia.rows_per_cta = lines;
-    GatherArgs& ga = J.ga;
-    ga.vact = ctx->vact;
-    ga.n_act = ctx->n_act;
-    ga.n = ctx->n;
-    ga.nrhs = ps.nrhs;
-    ga.nproj = spec.nproj;
-    ga.ga_ptr = ctx->prj.ga_ptr;
-    ga.ga_act = ctx->prj.ga_act;
-    for (int pj = 0; pj < spec.nproj; ++pj) {
-      ga.w[pj] = ctx->prj.ga_w[spec.proj[pj]];
-      ga.coef[pj] = spec.coef[pj];
-    }
-    if (spec.near != nullptr && spec.near->nnz > 0) {
-      ga.nptr = spec.near->ptr;
-      ga.ncol = spec.near->col;
-      ga.nval = near_values(spec.near, spec.near_which, (CT*)nullptr);
-    }
-    ga.x = ps.x;
-    ga.out_scale = spec.out_scale;
-    ga.y = ps.y;
-    ga.accumulate = 0;
-    J.gather_rb = ps.nrhs == 1 ? 1 : 8;
+    ia.qcut = qcut;
+    ia.sparse = sparse;
+    J.ga = gather_args<CT>(ctx, spec, ps.nrhs, ps.x, ps.y);
+    J.gather_rb = ps.nrhs == 1 ? 1 : ps.nrhs <= 4 ? 4 : 8;
     J.row_items = (ctx->nrows + lines - 1) / lines;
     J.col_items = P / lines;
     J.channels = channels;
     J.tile_major = channels >= 8;
     const long long groups = (long long)ctx->n * ((ps.nrhs + J.gather_rb - 1) / J.gather_rb);
     const long long gblocks = (groups * kGatherLanes + B - 1) / B;
-    m.off[0][i + 1] = m.off[0][i] + (long long)J.row_items * channels;
-    m.off[1][i + 1] = m.off[1][i] + (long long)J.col_items * channels;
-    m.off[2][i + 1] = m.off[2][i] + (long long)J.row_items * channels;
-    m.off[3][i + 1] = m.off[3][i] + gblocks;
+    m.off[0][i + 1] = m.off[0][i] + ((long long)ctx->n_act * ps.nrhs + B - 1) / B;
+    m.off[1][i + 1] = m.off[1][i] + (long long)J.row_items * channels;
+    m.off[2][i + 1] = m.off[2][i] + (long long)J.col_items * channels;
+    m.off[3][i + 1] = m.off[3][i] + (long long)J.row_items * channels;
+    m.off[4][i + 1] = m.off[4][i] + gblocks;
   }
   if (smem > kMaxDynSmem) return fail(AIM_EINVAL, "multi-context launch needs too much shared memory");
   auto kernel = k_grid_multi<CT, TPT, LOGE>;
-  AIM_TRY(ensure_smem(kernel, smem));
+  AIM_TRY(ensure_smem(passes[0].ctx, kernel, smem));
   int dev = 0, sms = 0, per_sm = 0, coop = 0;
   AIM_CUDA_TRY(cudaGetDevice(&dev));
   AIM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1009,7 +1327,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
   AIM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, B, smem));
   if (per_sm < 1) return fail(AIM_EINVAL, "multi-context kernel does not fit an SM");
   long long most = 0;
-  for (int ph = 0; ph < 4; ++ph) most = std::max(most, m.off[ph][count]);
+  for (int ph = 0; ph < 5; ++ph) most = std::max(most, m.off[ph][count]);
   const int grid = (int)std::max(1LL, std::min<long long>((long long)sms * per_sm, most));
   AIM_CUDA_TRY(cudaMemsetAsync(scratch, 0, 2 * sizeof(unsigned), st));   // the barrier words (not the error flag)
   {
@@ -1024,7 +1342,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
 // Splits the passes into the fewest launches whose contexts can share one CTA size (longest
 // transforms first; a context too short for the CTA size of a longer one goes to a later launch).
 template <typename CT, int TPT, int LOGE>
-static aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host,
+aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host,
                                       cudaStream_t st) {
   std::vector<int> left(count);
   for (int i = 0; i < count; ++i) left[i] = i;
@@ -1080,9 +1398,7 @@ aim_status grid_product_dense(aim_ctx* ctx, bool filtered, int nrhs, const doubl
   RowFwdArgs fa{};
   fa.x = u;
   fa.dense = 1;
-  fa.n = ctx->n;
   fa.m = ctx->m;
-  fa.nrhs = nrhs;
   RowInvArgs ia{};
   ia.dense = 1;
   ia.dense_out = v;

@@ -9,7 +9,7 @@
 namespace aim {
 
 static const char* kKernelNames[K_COUNT] = {
-    "row_fwd (anterpolation + forward row DFT)",
+    "row_fwd (forward row DFT)",
     "col_conv (column DFT x spectrum x inverse column DFT)",
     "row_inv (inverse row DFT + restriction)",
     "gather (interpolation + near-field SpMV)",
@@ -23,6 +23,7 @@ static const char* kKernelNames[K_COUNT] = {
     "gmres_arnoldi (DCGS2 projections and updates; timed per step)",
     "grid_multi (persistent: row passes, column pass and gathers of several contexts)",
     "dft_stage (radix-16 pass measurement: CUDA cores or tensor cores)",
+    "anterpolate (u = P x at the active grid points)",
 };
 
 namespace {
