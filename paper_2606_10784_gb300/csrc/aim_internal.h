@@ -203,9 +203,8 @@ struct aim_ctx {
   double* red = nullptr; size_t red_bytes = 0;          // reduction scratch (dot products)
   double* red_host = nullptr; size_t red_host_bytes = 0;
   int reserved_rhs[3] = {0, 0, 0};   // per precision (AIM_FP64, AIM_MIXED, AIM_FP64_NATIVE)
-  // launch schedule per precision; defaults measured on GB300, aim_autotune re-measures
-  // defaults: measured at the single-solve scale (2048^2 grid, P = 4096), feasible at every P
-  aim::Schedule sched[3] = {{2, 128, 0, 8}, {2, 128, 0, 16}, {2, 128, 0, 16}};
+  // launch schedule per precision: default_schedule, aim_set_schedule or aim_autotune
+  aim::Schedule sched[3] = {};
   // bookkeeping
   std::vector<std::pair<const void*, size_t>> smem_raised;   // dynamic shared memory limits raised so far
   std::vector<void*> allocations;
@@ -215,6 +214,24 @@ struct aim_ctx {
 };
 
 namespace aim {
+
+// The schedule a context starts with, feasible at every P. Elements per thread decide the rounding,
+// so they depend on the context alone: 8 in double-float (16 overflow the instruction cache); 8 in
+// complex64 up to P = 1024, where the shorter chains of radix-8 passes and the doubled threads count
+// (operator N, one vector: P = 64 column pass 10.1 -> 6.7 us, P = 1024 23.2 -> 20.5 us), 16 beyond
+// (P = 2048: 68 us with 16, more with 8); 16 in binary64. Transforms per thread and columns per CTA
+// are then chosen launch by launch (pass_tpt, col_cols_of).
+inline Schedule default_schedule(int precision, int P) {
+  return {2, 128, 0, precision == AIM_FP64 || (precision == AIM_MIXED && P <= 1024) ? 8 : 16};
+}
+inline bool sched_is_default(const aim_ctx* ctx, int precision) {
+  const Schedule &a = ctx->sched[precision], b = default_schedule(precision, ctx->P);
+  return a.tpt == b.tpt && a.min_row_threads == b.min_row_threads && a.col_cols == b.col_cols && a.elems == b.elems;
+}
+// the geometry a context stands for in the check of a multi-context call
+inline Schedule multi_geometry(const aim_ctx* ctx, int precision) {
+  return sched_is_default(ctx, precision) ? default_schedule(precision, kMaxP) : ctx->sched[precision];
+}
 
 // allocation helpers (tracked by the context)
 aim_status dev_alloc(aim_ctx* ctx, void** p, size_t bytes);

@@ -363,6 +363,7 @@ aim_status derive_params(aim_ctx* ctx, const aim_geometry* geometry, double k, c
   ctx->logP = ilog2(P);
   ctx->H = P / 2;
   ctx->logH = ctx->logP - 1;
+  for (int p = 0; p < 3; ++p) ctx->sched[p] = default_schedule(p, P);
   ctx->L = grid->half_side_L > 0.0 ? grid->half_side_L : host_grid_half_side(geometry->xy, ctx->n, ctx->m, ctx->s);
   ctx->eps = 2.0 * ctx->L / (ctx->m - 1);
   ctx->near_radius = stencil->near_radius > 0.0 ? stencil->near_radius : ctx->s * ctx->eps;

@@ -850,13 +850,18 @@ struct Supports {
 
 inline int loge_of(const Schedule& sc) { return sc.elems == 8 ? 3 : 4; }
 
-// columns per column-pass CTA: the schedule's choice, else the fewest whole tiles of W
-// columns that give at least 128 threads
+// columns per column-pass CTA: the schedule's choice. By default one column as soon as it has 128
+// threads (64 with 16 complex64 elements per thread): CTAs of one column wait at barriers of their
+// own, and several fit an SM, which gains more than the half or quarter sectors they load cost
+// (operator N at P = 4096: double-float 1273 -> 1163 us, complex64 329 -> 277 us; complex64 at
+// P = 2048, 32 right-hand sides: 2062 -> 1925 us). Shorter columns: the fewest whole tiles of W
+// columns that give at least 128 threads.
 template <typename CT, int TPT, int LOGE>
 static int col_cols_of(const Schedule& sc, int logH, int logP) {
   constexpr int W = GridT<CT>::W, LPT = 3 - TPT;
   if (sc.col_cols > 0) return sc.col_cols;
   const int tpf = (1 << logH) >> LOGE, ntiles = (1 << logP) / W;
+  if (LPT * tpf >= (std::is_same<CT, float2>::value && LOGE == 4 ? 64 : 128)) return 1;
   int tpc = 1;
   while (tpc * LPT * W * tpf < 128 && tpc < ntiles) tpc *= 2;
   return tpc * W;
@@ -890,86 +895,76 @@ static bool feasible_for(const Schedule& s, int logH, int logP) {
   return s.tpt == 1 ? feasible_tpt<CT, 1, 4>(s, logH, logP) : feasible_tpt<CT, 2, 4>(s, logH, logP);
 }
 
+// rows per CTA: at least min_row_threads threads (fewer when the grid has fewer rows, but
+// never less than a full warp: the recombination shuffles need all 32 lanes; rows past the
+// last one load zeros and store nothing), within the launch bound
 template <typename CT, int TPT, int LOGE>
-aim_status launch_tpt(aim_ctx* ctx, int channels, bool filtered, RowFwdArgs fa, RowInvArgs ia,
-                             void* inter, const Schedule& sc, cudaStream_t st) {
-  const int min_row_threads = sc.min_row_threads;
-  using T2 = CT;
+static int rows_per_cta(const aim_ctx* ctx, const Schedule& sc) {
   constexpr int LPT = 3 - TPT;
-  const int H = ctx->H, tpf = H >> LOGE, HS = padded_len<LOGE>(H);
-  const void* tw = twiddles(ctx, (CT*)nullptr);
-  const void* spec = spectrum(ctx, filtered, (CT*)nullptr);
-
-  // rows per CTA: at least min_row_threads threads (fewer when the grid has fewer rows, but
-  // never less than a full warp: the recombination shuffles need all 32 lanes; rows past the
-  // last one load zeros and store nothing), within the launch bound
+  const int tpf = ctx->H >> LOGE;
   int rpc = 1;
-  while (((rpc * LPT * tpf < min_row_threads && rpc < ctx->nrows) || rpc * LPT * tpf < 32) &&
+  while (((rpc * LPT * tpf < sc.min_row_threads && rpc < ctx->nrows) || rpc * LPT * tpf < 32) &&
          2 * rpc * LPT * tpf <= LaunchMax<CT, TPT, LOGE>::value)
     rpc *= 2;
-  const int row_blocks = (ctx->nrows + rpc - 1) / rpc;
-  const int sparse = !fa.dense && sparse_rows<LOGE>(ctx);
-  const size_t sm_row =
-      2 * (size_t)rpc * HS * sizeof(T2) + (sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
-  const int qcut = filtered ? ctx->qcut : ctx->H;
+  return rpc;
+}
 
-  fa.tw = tw;
-  fa.logH = ctx->logH;
-  fa.logP = ctx->logP;
-  fa.row_lo = ctx->row_lo;
-  fa.nrows = ctx->nrows;
-  fa.inter = inter;
+template <typename CT, int TPT, int LOGE>
+aim_status launch_row_fwd(aim_ctx* ctx, int channels, RowFwdArgs fa, const Schedule& sc, cudaStream_t st) {
+  constexpr int LPT = 3 - TPT;
+  const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
+  fa.sparse = !fa.dense && sparse_rows<LOGE>(ctx);
   fa.rows_per_cta = rpc;
-  fa.qcut = qcut;
-  fa.sparse = sparse;
-  AIM_TRY(ensure_smem(ctx, k_row_fwd<CT, TPT, LOGE>, sm_row));
-  {
-    ProfScope ps(K_ROW_FWD, st);
-    AIM_TRY(launch_chained(k_row_fwd<CT, TPT, LOGE>, dim3(row_blocks, channels), rpc * LPT * tpf, sm_row, st, fa));
-  }
+  const size_t smem =
+      2 * (size_t)rpc * padded_len<LOGE>(ctx->H) * sizeof(CT) + (fa.sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
+  AIM_TRY(ensure_smem(ctx, k_row_fwd<CT, TPT, LOGE>, smem));
+  ProfScope ps(K_ROW_FWD, st);
+  return launch_chained(k_row_fwd<CT, TPT, LOGE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, fa);
+}
 
-  // column pass
-  const int cols = col_cols_of<CT, TPT, LOGE>(sc, ctx->logH, ctx->logP);
-  int log_cols = 0;
-  while ((1 << log_cols) < cols) ++log_cols;
-  ColArgs ca;
-  ca.inter = inter;
-  ca.spec = spec;
-  ca.qcut = qcut;
-  ca.tw = tw;
-  ca.logH = ctx->logH;
-  ca.logP = ctx->logP;
-  ca.row_lo = ctx->row_lo;
-  ca.nrows = ctx->nrows;
-  ca.log_cols = log_cols;
-  const size_t sm_col = 2 * (size_t)cols * HS * sizeof(T2);
-  if (ctx->P / cols > 65535) return fail(AIM_EINVAL, "too many column tiles for one column-pass grid");
+template <typename CT, int TPT, int LOGE>
+aim_status launch_col_conv(aim_ctx* ctx, int channels, ColArgs ca, const Schedule& sc, cudaStream_t st) {
+  constexpr int LPT = 3 - TPT;
   constexpr int kChanX = 8;   // channels from which the column-pass grid runs channels along x
-  AIM_TRY(ensure_smem(ctx, k_col_conv<CT, TPT, LOGE>, sm_col));
-  {
-    ProfScope ps(K_COL_CONV, st);
-    ca.chan_x = channels >= kChanX;
-    const dim3 grid = ca.chan_x ? dim3(channels, ctx->P / cols) : dim3(ctx->P / cols, channels);
-    AIM_TRY(launch_chained(k_col_conv<CT, TPT, LOGE>, grid, cols * LPT * tpf, sm_col, st, ca));
-  }
+  const int tpf = ctx->H >> LOGE, cols = col_cols_of<CT, TPT, LOGE>(sc, ctx->logH, ctx->logP);
+  ca.log_cols = 0;
+  while ((1 << ca.log_cols) < cols) ++ca.log_cols;
+  if (ctx->P / cols > 65535) return fail(AIM_EINVAL, "too many column tiles for one column-pass grid");
+  const size_t smem = 2 * (size_t)cols * padded_len<LOGE>(ctx->H) * sizeof(CT);
+  AIM_TRY(ensure_smem(ctx, k_col_conv<CT, TPT, LOGE>, smem));
+  ca.chan_x = channels >= kChanX;
+  const dim3 grid = ca.chan_x ? dim3(channels, ctx->P / cols) : dim3(ctx->P / cols, channels);
+  ProfScope ps(K_COL_CONV, st);
+  return launch_chained(k_col_conv<CT, TPT, LOGE>, grid, cols * LPT * tpf, smem, st, ca);
+}
 
-  // row inverse
-  ia.inter = inter;
-  ia.tw = tw;
-  ia.logH = ctx->logH;
-  ia.logP = ctx->logP;
-  ia.row_lo = ctx->row_lo;
-  ia.nrows = ctx->nrows;
-  ia.scale = 1.0 / ((double)ctx->P * (double)ctx->P);
+template <typename CT, int TPT, int LOGE>
+aim_status launch_row_inv(aim_ctx* ctx, int channels, RowInvArgs ia, const Schedule& sc, cudaStream_t st) {
+  constexpr int LPT = 3 - TPT;
+  const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
+  ia.sparse = !ia.dense && sparse_rows<LOGE>(ctx);
   ia.rows_per_cta = rpc;
-  ia.qcut = qcut;
-  ia.sparse = sparse;
-  AIM_TRY(ensure_smem(ctx, k_row_inv<CT, TPT, LOGE>, sm_row));
-  {
-    ProfScope ps(K_ROW_INV, st);
-    AIM_TRY(launch_chained(k_row_inv<CT, TPT, LOGE>, dim3(row_blocks, channels), rpc * LPT * tpf, sm_row, st, ia));
-  }
-  return AIM_OK;
+  const size_t smem =
+      2 * (size_t)rpc * padded_len<LOGE>(ctx->H) * sizeof(CT) + (ia.sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
+  AIM_TRY(ensure_smem(ctx, k_row_inv<CT, TPT, LOGE>, smem));
+  ProfScope ps(K_ROW_INV, st);
+  return launch_chained(k_row_inv<CT, TPT, LOGE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, ia);
+}
+
+// Transforms per thread of a pass of `lines` lines whose two-transform form has tpf threads a line.
+// The results do not depend on it. A schedule that the caller or the autotuner set is obeyed; with
+// the context's default, one transform per thread where two leave the SMs short of warps: one has
+// half the serial work per thread, two share their twiddles. The lines lie between the sizes where
+// either was faster: row passes in double-float 26.0 against 28.7 us at 81 thousand threads and 76.0
+// against more at 324 thousand, in complex64 9.7 against 13.9 us at 27 thousand and 14.0 against 14.7 at
+// 81 thousand; column passes 14.5 against 18.5 us at 16 thousand (S^alpha, P = 512) and 26.6 against
+// 22.5 at 65 thousand (P = 1024).
+template <typename CT>
+static int pass_tpt(const aim_ctx* ctx, const Schedule& sc, bool rows, long long lines) {
+  if (std::is_same<CT, double2>::value || !sched_is_default(ctx, precision_of((CT*)nullptr))) return sc.tpt;
+  const long long threads = lines * (ctx->H >> loge_of(sc));
+  const long long most = !rows ? 32 << 10 : std::is_same<CT, float2>::value ? 64 << 10 : 128 << 10;
+  return threads <= most ? 1 : 2;
 }
 
 template <typename CT>
@@ -977,19 +972,58 @@ static aim_status launch_three_passes(aim_ctx* ctx, int channels, bool filtered,
                                       void* inter, cudaStream_t st) {
   if (channels > 65535) return fail(AIM_EINVAL, "too many channels in one grid pass");
   if (ctx->H < 32) return fail(AIM_EINVAL, "embedding side P must be >= 64");
-  const int p = precision_of((CT*)nullptr);
-  const Schedule sc = ctx->sched[p];
+  const Schedule sc = ctx->sched[precision_of((CT*)nullptr)];
   if (!feasible_for<CT>(sc, ctx->logH, ctx->logP)) return fail(AIM_EINVAL, "launch schedule not feasible");
-  if constexpr (std::is_same<CT, double2>::value) {
-    return launch_tpt<CT, 2, 4>(ctx, channels, filtered, fa, ia, inter, sc, st);
-  } else {
-    if (loge_of(sc) == 3) {
-      if (sc.tpt == 1) return launch_tpt<CT, 1, 3>(ctx, channels, filtered, fa, ia, inter, sc, st);
-      return launch_tpt<CT, 2, 3>(ctx, channels, filtered, fa, ia, inter, sc, st);
+  const void* tw = twiddles(ctx, (CT*)nullptr);
+  const int qcut = filtered ? ctx->qcut : ctx->H;
+  fa.tw = tw;
+  fa.logH = ctx->logH;
+  fa.logP = ctx->logP;
+  fa.row_lo = ctx->row_lo;
+  fa.nrows = ctx->nrows;
+  fa.inter = inter;
+  fa.qcut = qcut;
+  ColArgs ca{};
+  ca.inter = inter;
+  ca.spec = spectrum(ctx, filtered, (CT*)nullptr);
+  ca.qcut = qcut;
+  ca.tw = tw;
+  ca.logH = ctx->logH;
+  ca.logP = ctx->logP;
+  ca.row_lo = ctx->row_lo;
+  ca.nrows = ctx->nrows;
+  ia.inter = inter;
+  ia.tw = tw;
+  ia.logH = ctx->logH;
+  ia.logP = ctx->logP;
+  ia.row_lo = ctx->row_lo;
+  ia.nrows = ctx->nrows;
+  ia.scale = 1.0 / ((double)ctx->P * (double)ctx->P);
+  ia.qcut = qcut;
+  const long long rows = (long long)channels * ctx->nrows, cols = (long long)channels * std::min(ctx->P, 2 * qcut + 1);
+  auto run = [&](auto tpt, auto loge, int pass) -> aim_status {
+    constexpr int TPT = decltype(tpt)::value, LOGE = decltype(loge)::value;
+    if (pass == 0) return launch_row_fwd<CT, TPT, LOGE>(ctx, channels, fa, sc, st);
+    if (pass == 1) return launch_col_conv<CT, TPT, LOGE>(ctx, channels, ca, sc, st);
+    return launch_row_inv<CT, TPT, LOGE>(ctx, channels, ia, sc, st);
+  };
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
+  using I3 = std::integral_constant<int, 3>;
+  using I4 = std::integral_constant<int, 4>;
+  for (int pass = 0; pass < 3; ++pass) {
+    const int tpt = pass_tpt<CT>(ctx, sc, pass != 1, pass != 1 ? rows : cols);
+    aim_status s;
+    if constexpr (std::is_same<CT, double2>::value) {
+      s = run(I2{}, I4{}, pass);
+    } else if (loge_of(sc) == 3) {
+      s = tpt == 1 ? run(I1{}, I3{}, pass) : run(I2{}, I3{}, pass);
+    } else {
+      s = tpt == 1 ? run(I1{}, I4{}, pass) : run(I2{}, I4{}, pass);
     }
-    if (sc.tpt == 1) return launch_tpt<CT, 1, 4>(ctx, channels, filtered, fa, ia, inter, sc, st);
-    return launch_tpt<CT, 2, 4>(ctx, channels, filtered, fa, ia, inter, sc, st);
+    AIM_TRY(s);
   }
+  return AIM_OK;
 }
 
 inline AntArgs ant_args(const aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2* x) {
@@ -1342,12 +1376,10 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
 // Splits the passes into the fewest launches whose contexts can share one CTA size (longest
 // transforms first; a context too short for the CTA size of a longer one goes to a later launch).
 template <typename CT, int TPT, int LOGE>
-aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host,
-                                      cudaStream_t st) {
+aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned* scratch, cudaStream_t st) {
   std::vector<int> left(count);
   for (int i = 0; i < count; ++i) left[i] = i;
   std::stable_sort(left.begin(), left.end(), [&](int a, int b) { return passes[a].ctx->H > passes[b].ctx->H; });
-  AIM_CUDA_TRY(cudaMemsetAsync(scratch + 2, 0, sizeof(int), st));   // the stage's error flag
   std::vector<MultiPassSpec> group;
   while (!left.empty()) {
     const int B = multi_cta_threads<CT, TPT, LOGE>(passes[left[0]].ctx->H);
@@ -1357,11 +1389,9 @@ aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned*
       if (multi_fits<CT, TPT, LOGE>(B, passes[i].ctx->H)) group.push_back(passes[i]);
       else rest.push_back(i);
     }
-    const aim_status gs = launch_multi<CT, TPT, LOGE>(group.data(), (int)group.size(), scratch, st);
-    if (gs != AIM_OK) return gs;
+    AIM_TRY((launch_multi<CT, TPT, LOGE>(group.data(), (int)group.size(), scratch, st)));
     left.swap(rest);
   }
-  AIM_CUDA_TRY(cudaMemcpyAsync(err_host, scratch + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
   return AIM_OK;
 }
 
@@ -1369,22 +1399,30 @@ template <typename CT>
 aim_status grid_pass_multi(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host, cudaStream_t st) {
   if (count < 1 || count > kMaxMultiJobs) return fail(AIM_EINVAL, "1 to 32 passes per multi-context launch");
   const int p = precision_of((CT*)nullptr);
-  const Schedule sc = passes[0].ctx->sched[p];
+  // Contexts may share a call when their pass geometries agree, a context on its default schedule
+  // standing for the geometry of the largest grids: such contexts differ in elements per thread by
+  // size, and each runs with its own (so that its results are those of a launch of its own).
+  const Schedule sc = multi_geometry(passes[0].ctx, p);
   for (int i = 1; i < count; ++i) {
-    const Schedule& o = passes[i].ctx->sched[p];
+    const Schedule o = multi_geometry(passes[i].ctx, p);
     if (o.tpt != sc.tpt || loge_of(o) != loge_of(sc))
       return fail(AIM_EINVAL, "contexts of one multi-context launch must share the pass geometry of their schedule");
   }
+  AIM_CUDA_TRY(cudaMemsetAsync(scratch + 2, 0, sizeof(int), st));   // the stage's error flag
   if constexpr (std::is_same<CT, double2>::value) {
-    return launch_multi_groups<CT, 2, 4>(passes, count, scratch, err_host, st);
+    AIM_TRY((launch_multi_groups<CT, 2, 4>(passes, count, scratch, st)));
   } else {
-    if (loge_of(sc) == 3) {
-      if (sc.tpt == 1) return launch_multi_groups<CT, 1, 3>(passes, count, scratch, err_host, st);
-      return launch_multi_groups<CT, 2, 3>(passes, count, scratch, err_host, st);
-    }
-    if (sc.tpt == 1) return launch_multi_groups<CT, 1, 4>(passes, count, scratch, err_host, st);
-    return launch_multi_groups<CT, 2, 4>(passes, count, scratch, err_host, st);
+    std::vector<MultiPassSpec> of[2];
+    for (int i = 0; i < count; ++i) of[loge_of(passes[i].ctx->sched[p]) - 3].push_back(passes[i]);
+    if (!of[0].empty())
+      AIM_TRY((sc.tpt == 1 ? launch_multi_groups<CT, 1, 3>(of[0].data(), (int)of[0].size(), scratch, st)
+                           : launch_multi_groups<CT, 2, 3>(of[0].data(), (int)of[0].size(), scratch, st)));
+    if (!of[1].empty())
+      AIM_TRY((sc.tpt == 1 ? launch_multi_groups<CT, 1, 4>(of[1].data(), (int)of[1].size(), scratch, st)
+                           : launch_multi_groups<CT, 2, 4>(of[1].data(), (int)of[1].size(), scratch, st)));
   }
+  AIM_CUDA_TRY(cudaMemcpyAsync(err_host, scratch + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
+  return AIM_OK;
 }
 
 
