@@ -125,6 +125,8 @@ __device__ __forceinline__ double2 to_d2(float h_re, float l_re, float h_im, flo
 }
 
 __global__ void k_to_dfc(const double2* __restrict__ src, int count, dfc* __restrict__ dst) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < count) dst[t] = to_dfc(src[t]);
 }
@@ -225,6 +227,8 @@ __global__ void __launch_bounds__(32 * kDot2Warps) k_multidot2_partial_df(const 
                                                                           const dfc* __restrict__ R1, int n, int nrhs,
                                                                           int J, double2* __restrict__ part0,
                                                                           double2* __restrict__ part1) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = blockIdx.x * kDot2Warps + wid, r = blockIdx.y, z = blockIdx.z;
   if (l >= J) return;   // whole warps; the kernel has no block-wide barrier
@@ -261,6 +265,8 @@ __global__ void __launch_bounds__(32 * kDot2Warps) k_multidot2_partial_df(const 
 __global__ void k_dcgs2_finish(const double2* __restrict__ part0, const double2* __restrict__ part1, int nz, int J,
                                int nrhs, int j, int restart, double2* __restrict__ D0, double2* __restrict__ D1,
                                dfc* __restrict__ D0df, dfc* __restrict__ H) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int count = J * nrhs;
   if (t >= count) return;
@@ -323,6 +329,8 @@ __global__ void __launch_bounds__(256) k_dcgs2_hs_scal(const dfc* H, const dfc* 
                                                        int final_step, double2* __restrict__ hs,
                                                        double2* __restrict__ colout, dfc* Hw,
                                                        double2* __restrict__ scal) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
   const int r = blockIdx.y;
   const int nrow_blocks = final_step ? 0 : (j + kHsRows - 1) / kHsRows;
   const size_t hb = (size_t)r * hess_entries(restart);
@@ -397,6 +405,8 @@ __global__ void k_dcgs2_coeffs(const double2* __restrict__ D0, const double2* __
                                const double2* __restrict__ hs, const double2* __restrict__ scal, int j, int nrhs,
                                int restart, int final_step, dfc* __restrict__ H, double2* __restrict__ colout,
                                dfc* __restrict__ a1, dfc* __restrict__ g) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= j * nrhs) return;
   const int l = t / nrhs, r = t - l * nrhs;
@@ -416,75 +426,162 @@ __global__ void k_dcgs2_coeffs(const double2* __restrict__ D0, const double2* __
   H[hb + hess_index(l, j)] = to_dfc(c);
 }
 
-// Stage 1 of the two updates of a step, over one read of the basis: part1[chunk][r][i] =
-// sum over the chunk of V[l][r][i] a1[l], part2 the same with g
-__global__ void k_vcombine2_partial_df(const dfc* __restrict__ V, const dfc* __restrict__ a1, const dfc* __restrict__ g,
-                                       int J, int n, int nrhs, dfc* __restrict__ part1, dfc* __restrict__ part2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int chunk = blockIdx.y, r = blockIdx.z;
-  if (i >= n) return;
-  const int j0 = chunk * kCgsChunk, j1 = min(J, j0 + kCgsChunk);
-  // products and sums as paired instructions on the (re, im) lanes (cmul, cadd)
-  dfc acc1 = dfc{0.f, 0.f, 0.f, 0.f}, acc2 = dfc{0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-  for (int l = j0; l < j1; ++l) {
-    const dfc v = V[((size_t)l * nrhs + r) * n + i];
-    acc1 = cadd(acc1, cmul(v, a1[(size_t)l * nrhs + r]));
-    acc2 = cadd(acc2, cmul(v, g[(size_t)l * nrhs + r]));
-  }
-  const size_t o = ((size_t)chunk * nrhs + r) * n + i;
-  part1[o] = acc1;
-  part2[o] = acc2;
-}
+// The coefficients of one step in one launch, for the first kStepJ steps of a cycle: one CTA per
+// right-hand side does what k_dcgs2_finish, k_dcgs2_hs_scal and k_dcgs2_coeffs do in three launches
+// (H s is then at most 8 thousand products, a microsecond for one SM, and a launch costs two to three). With the updates in one launch and the
+// columns written to host memory by the kernels, 60 steps of an N = 600 system with 4 right-hand sides
+// went from 50.8 to 33.4 us a step, 400 steps at N = 10000 from 86 to 62 us.
+constexpr int kStepJ = 128, kStepThreads = 512, kStepWarps = kStepThreads / 32;
 
-// Stage 2: v_j = u / beta - V a1 into slot j (u is read there first), u_{j+1} = w / beta - kappa u -
-// V g into slot j+1 and, in binary64, into cur (the next product's input). Eight adjacent threads
-// per element sum every eighth chunk; a fixed shuffle tree adds their sums.
-constexpr int kFinishLanes = 8;
-
-__global__ void k_vcombine2_finish_df(const dfc* __restrict__ part1, const dfc* __restrict__ part2, int nchunks, int n,
-                                      int nrhs, const double2* __restrict__ scal, dfc* __restrict__ Vj,
-                                      const double2* __restrict__ w, dfc* __restrict__ Vnext, double2* __restrict__ cur) {
-  const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = (int)(gt / kFinishLanes), q = (int)(gt % kFinishLanes);
-  const bool live = t < n * nrhs;   // whole groups of four: the shuffles below need every lane
-  float a_rh = 0.f, a_rl = 0.f, a_ih = 0.f, a_il = 0.f;
-  float b_rh = 0.f, b_rl = 0.f, b_ih = 0.f, b_il = 0.f;
-  if (live) {
-#pragma unroll 2
-    for (int ch = q; ch < nchunks; ch += kFinishLanes) {
-      const dfc p = part1[(size_t)ch * n * nrhs + t], pp = part2[(size_t)ch * n * nrhs + t];
-      df_add(a_rh, a_rl, p.xh, p.xl, a_rh, a_rl);
-      df_add(a_ih, a_il, p.yh, p.yl, a_ih, a_il);
-      df_add(b_rh, b_rl, pp.xh, pp.xl, b_rh, b_rl);
-      df_add(b_ih, b_il, pp.yh, pp.yl, b_ih, b_il);
+__global__ void __launch_bounds__(kStepThreads) k_dcgs2_step(const double2* __restrict__ part0,
+                                                             const double2* __restrict__ part1, int nz, int nrhs, int j,
+                                                             int restart, const int* __restrict__ active,
+                                                             dfc* __restrict__ H, double2* __restrict__ colout,
+                                                             double2* __restrict__ scal, dfc* __restrict__ a1,
+                                                             dfc* __restrict__ g) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
+  const bool final_step = part1 == nullptr;
+  const int r = blockIdx.x, J = j + 1, count = J * nrhs, tid = threadIdx.x;
+  dfc* Hr = H + (size_t)r * hess_entries(restart);
+  __shared__ double2 s[kStepJ + 1], t[kStepJ + 1];
+  __shared__ dfc sdf[kStepJ + 1];
+  __shared__ dfc part[kStepWarps][kStepJ];
+  __shared__ double sh[32][3];
+  __shared__ double2 sc[3];
+  // chunk sums in chunk order, and the delayed second pass of column j - 1
+  for (int l = tid; l < J; l += kStepThreads) {
+    double re = 0.0, im = 0.0, re1 = 0.0, im1 = 0.0;
+    for (int z = 0; z < nz; ++z) {
+      const double2 a = part0[(size_t)z * count + (size_t)l * nrhs + r];
+      re += a.x;
+      im += a.y;
+      if (!final_step) {
+        const double2 b = part1[(size_t)z * count + (size_t)l * nrhs + r];
+        re1 += b.x;
+        im1 += b.y;
+      }
+    }
+    s[l] = double2{re, im};
+    t[l] = double2{re1, im1};
+    const dfc sd = to_dfc(double2{re, im});
+    sdf[l] = sd;
+    if (l < j) {
+      dfc& h = Hr[hess_index(l, j - 1)];
+      dfc o;
+      df_add(h.xh, h.xl, sd.xh, sd.xl, o.xh, o.xl);
+      df_add(h.yh, h.yl, sd.yh, sd.yl, o.yh, o.yl);
+      h = o;
+      colout[(size_t)l * nrhs + r] = to_d2(o.xh, o.xl, o.yh, o.yl);
     }
   }
-#pragma unroll
-  for (int off = 1; off < kFinishLanes; off <<= 1) {
-    const float o0 = __shfl_xor_sync(0xffffffffu, a_rh, off), o1 = __shfl_xor_sync(0xffffffffu, a_rl, off);
-    const float o2 = __shfl_xor_sync(0xffffffffu, a_ih, off), o3 = __shfl_xor_sync(0xffffffffu, a_il, off);
-    const float o4 = __shfl_xor_sync(0xffffffffu, b_rh, off), o5 = __shfl_xor_sync(0xffffffffu, b_rl, off);
-    const float o6 = __shfl_xor_sync(0xffffffffu, b_ih, off), o7 = __shfl_xor_sync(0xffffffffu, b_il, off);
-    df_add(a_rh, a_rl, o0, o1, a_rh, a_rl);
-    df_add(a_ih, a_il, o2, o3, a_ih, a_il);
-    df_add(b_rh, b_rl, o4, o5, b_rh, b_rl);
-    df_add(b_ih, b_il, o6, o7, b_ih, b_il);
+  __syncthreads();
+  double ss = 0.0, st_re = 0.0, st_im = 0.0;
+  for (int l = tid; l < j; l += kStepThreads) {
+    ss += s[l].x * s[l].x + s[l].y * s[l].y;
+    const double2 c = zconjmul(s[l], t[l]);
+    st_re += c.x;
+    st_im += c.y;
   }
-  if (!live || q != 0) return;
-  const int r = t / n;
-  const double2 P1 = to_d2(a_rh, a_rl, a_ih, a_il), P2 = to_d2(b_rh, b_rl, b_ih, b_il);
+  block_sum3(ss, st_re, st_im, sh);   // its barrier also covers H's column j - 1
+  if (tid == 0) {
+    const double q = s[j].x, b2 = q - ss;
+    // a non-finite value reaches the host through beta (the norm it checks); b2 <= 0 is a breakdown
+    const double beta = !active[r] ? 0.0 : !isfinite(b2) ? b2 : b2 > 0.0 ? sqrt(b2) : 0.0;
+    const double ib = beta > 0.0 ? 1.0 / beta : 0.0;
+    if (j >= 1) {
+      colout[(size_t)j * nrhs + r] = double2{beta, 0.0};
+      Hr[hess_index(j, j - 1)] = to_dfc(double2{beta, 0.0});
+    }
+    if (!final_step) {
+      const double2 slast = j >= 1 ? s[j - 1] : double2{0.0, 0.0};
+      double2 d = double2{(t[j].x - st_re) * ib * ib - slast.x, (t[j].y - st_im) * ib * ib - slast.y};
+      if (beta == 0.0) d = double2{0.0, 0.0};
+      const double2 kappa = double2{(slast.x + d.x) * ib, (slast.y + d.y) * ib};
+      scal[r] = sc[0] = double2{ib, 0.0};
+      scal[nrhs + r] = sc[1] = kappa;
+      scal[2 * nrhs + r] = d;
+      Hr[hess_index(j, j)] = to_dfc(d);
+    }
+  }
+  if (final_step) return;
+  // H s: lanes over the rows l of H, warps over its columns m >= l - 1, then the warps' sums in order.
+  // H[j][j-1] = beta, which thread 0 is writing, has l = j and is not part of it.
+  const int wid = tid >> 5, lane = tid & 31;
+  for (int l = lane; l < j; l += 32) {
+    dfc acc = dfc{0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int m = wid; m < j; m += kStepWarps)
+      if (l <= m + 1) acc = cadd(acc, cmul(Hr[hess_index(l, m)], sdf[m]));
+    part[wid][l] = acc;
+  }
+  __syncthreads();
+  for (int l = tid; l < j; l += kStepThreads) {
+    dfc acc = part[0][l];
+#pragma unroll
+    for (int w = 1; w < kStepWarps; ++w) acc = cadd(acc, part[w][l]);
+    const double2 hv = to_d2(acc.xh, acc.xl, acc.yh, acc.yl), sv = s[l], tv = t[l], kappa = sc[1];
+    const double ib = sc[0].x;
+    const double2 c = double2{(tv.x - hv.x) * ib, (tv.y - hv.y) * ib};
+    const double2 ks = zmul(kappa, sv);
+    g[(size_t)l * nrhs + r] = to_dfc(double2{hv.x * ib + c.x - ks.x, hv.y * ib + c.y - ks.y});
+    a1[(size_t)l * nrhs + r] = to_dfc(double2{sv.x * ib, sv.y * ib});
+    Hr[hess_index(l, j)] = to_dfc(c);
+  }
+}
+
+// The two updates of a step over one read of the basis: v_j = u / beta - V a1 into slot j (u is read
+// there first), u_{j+1} = w / beta - kappa u - V g into slot j + 1 and, in binary64, into cur (the next
+// product's input). A CTA takes 32 elements; its 16 warps take the basis vectors l = warp, warp + 16,
+// ... in order and a fixed tree adds their sums. (Chunks of 32 vectors per CTA with their sums in
+// memory and a second kernel to add them cost a launch, and at 1700 vectors 17 us for that kernel.)
+constexpr int kUpdateWarps = 16;
+
+__global__ void __launch_bounds__(32 * kUpdateWarps) k_vcombine2_df(const dfc* __restrict__ V, const dfc* __restrict__ a1,
+                                                                   const dfc* __restrict__ g, int J, int n, int nrhs,
+                                                                   const double2* __restrict__ scal, dfc* Vj,
+                                                                   const double2* __restrict__ w, dfc* Vnext,
+                                                                   double2* __restrict__ cur) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, r = blockIdx.y;
+  const int i = blockIdx.x * 32 + lane;
+  // products and sums as paired instructions on the (re, im) lanes (cmul, cadd)
+  dfc acc1 = dfc{0.f, 0.f, 0.f, 0.f}, acc2 = dfc{0.f, 0.f, 0.f, 0.f};
+  if (i < n) {
+#pragma unroll 4
+    for (int l = wid; l < J; l += kUpdateWarps) {
+      const dfc v = V[((size_t)l * nrhs + r) * n + i];
+      acc1 = cadd(acc1, cmul(v, a1[(size_t)l * nrhs + r]));
+      acc2 = cadd(acc2, cmul(v, g[(size_t)l * nrhs + r]));
+    }
+  }
+  __shared__ dfc sm[2][kUpdateWarps][32];
+  sm[0][wid][lane] = acc1;
+  sm[1][wid][lane] = acc2;
+#pragma unroll
+  for (int off = kUpdateWarps / 2; off > 0; off >>= 1) {
+    __syncthreads();
+    if (wid < 2 * off) {   // the lower half of these warps adds the first sums, the upper half the second
+      const int k = wid < off ? 0 : 1, q = wid < off ? wid : wid - off;
+      sm[k][q][lane] = cadd(sm[k][q][lane], sm[k][q + off][lane]);
+    }
+  }
+  __syncthreads();
+  if (wid != 0 || i >= n) return;
+  const size_t o = (size_t)r * n + i;
+  const dfc p1 = sm[0][0][lane], p2 = sm[1][0][lane], ud = Vj[o];
+  const double2 P1 = to_d2(p1.xh, p1.xl, p1.yh, p1.yl), P2 = to_d2(p2.xh, p2.xl, p2.yh, p2.yl);
   const double ib = scal[r].x;
   const double2 kappa = scal[nrhs + r];
-  const dfc ud = Vj[t];
   const double2 u = to_d2(ud.xh, ud.xl, ud.yh, ud.yl);
-  const double2 wv = w[t];
+  const double2 wv = w[o];
   const double2 vj = double2{u.x * ib - P1.x, u.y * ib - P1.y};
   const double2 ku = zmul(kappa, u);
   const double2 un = double2{wv.x * ib - ku.x - P2.x, wv.y * ib - ku.y - P2.y};
-  Vj[t] = to_dfc(vj);
-  Vnext[t] = to_dfc(un);
-  cur[t] = un;
+  Vj[o] = to_dfc(vj);
+  Vnext[o] = to_dfc(un);
+  cur[o] = un;
 }
 
 // v = w[r] / sqrt(nrm2[r].x) (zero if the norm vanished, or active[r] == 0): the new basis
@@ -526,10 +623,10 @@ struct Workspace {
   double2 *w, *r, *cur, *tmp, *dots, *dots2, *nrm;
   dfc *wdf, *dots_df, *dots2_df;
   int* active;
-  // delayed reorthogonalisation: Hessenberg matrix (row-packed, per rhs), H s, the final column
-  // staged for the host, the update coefficients and the two scalars (1/beta, kappa) per rhs
+  // delayed reorthogonalisation: Hessenberg matrix (row-packed, per rhs), H s, the update
+  // coefficients and the scalars (1/beta, kappa, d) per rhs
   dfc* H;
-  double2 *hs, *colout, *scal;
+  double2 *hs, *scal;
   dfc* g;
 };
 
@@ -638,9 +735,9 @@ size_t krylov_bytes(size_t n, int nrhs, int restart) {
 }
 
 size_t reduction_bytes(int nrhs, int restart) {
-  // dots, dots2, norms, double-float copies, H s, the staged column, g, the step scalars, and
-  // the active flags
-  return ((size_t)(restart + 2) * 8 + 3) * nrhs * sizeof(double2) + nrhs * sizeof(int);
+  // dots, dots2, norms, double-float copies, H s, g, the step scalars, and the active flags (the
+  // pinned host copy of this size takes the two staged columns)
+  return ((size_t)(restart + 2) * 7 + 3) * nrhs * sizeof(double2) + nrhs * sizeof(int);
 }
 
 static aim_status ensure_krylov(aim_ctx* ctx, int nrhs, int restart) {
@@ -700,10 +797,9 @@ static aim_status gmres_core(aim_ctx* ctx, aim_op op, int precision, int nrhs, c
   ws.dots_df = reinterpret_cast<dfc*>(red + (size_t)(restart + 2) * 3 * nrhs);   // (restart+1) * nrhs
   ws.dots2_df = reinterpret_cast<dfc*>(red + (size_t)(restart + 2) * 4 * nrhs);  // (restart+1) * nrhs
   ws.hs = red + (size_t)(restart + 2) * 5 * nrhs;                                  // (restart+1) * nrhs
-  ws.colout = red + (size_t)(restart + 2) * 6 * nrhs;                              // (restart+2) * nrhs
-  ws.g = reinterpret_cast<dfc*>(red + (size_t)(restart + 2) * 7 * nrhs);           // (restart+1) * nrhs
-  ws.scal = red + (size_t)(restart + 2) * 8 * nrhs;                                // 2 * nrhs
-  ws.active = reinterpret_cast<int*>(red + ((size_t)(restart + 2) * 8 + 3) * nrhs);
+  ws.g = reinterpret_cast<dfc*>(red + (size_t)(restart + 2) * 6 * nrhs);           // (restart+1) * nrhs
+  ws.scal = red + (size_t)(restart + 2) * 7 * nrhs;                                // 3 * nrhs
+  ws.active = reinterpret_cast<int*>(red + ((size_t)(restart + 2) * 7 + 3) * nrhs);
   {
     const size_t nz = ((size_t)n + kDotChunk - 1) / kDotChunk;
     const size_t part_vecs =
@@ -770,7 +866,7 @@ static aim_status gmres_core(aim_ctx* ctx, aim_op op, int precision, int nrhs, c
     }
     // Arnoldi step j (delayed reorthogonalisation, see the kernels above): w = A u_j, both sets of
     // projections over one read of the basis, the coefficients, and v_j and u_{j+1} from one more
-    // read; step j (j >= 1) finalises Hessenberg column j - 1 and copies it to host slot
+    // read; step j (j >= 1) finalises Hessenberg column j - 1 and writes it to host slot
     // (j - 1) % 2. Step `restart` only finalises the last column (no product). A step needs
     // nothing from the host, so steps c + 1 and c + 2 are queued before the host waits for column
     // c: the Givens updates overlap the device work, and at most two queued steps are discarded
@@ -787,51 +883,48 @@ static aim_status gmres_core(aim_ctx* ctx, aim_op op, int precision, int nrhs, c
           AIM_TRY(solver_apply(ctx, op, nrhs, ws.cur, ws.w, precision, st));
         }
       }
-      // 7 launches (4 in the final step), timed as one group when profiling
+      // 4 launches in the first steps, 6 later (2 and 4 in the final step), timed as one group when
+      // profiling
       ProfScope group(K_GMRES, st, /*count_launch=*/false);
       const int J = j + 1;   // v_0..v_{j-1} and the candidate u_j in slot j
       const int nz = (n + kDotChunk - 1) / kDotChunk;
+      const dfc *V = ws.V, *wdf = final_step ? nullptr : ws.wdf;
+      // the kernels write the final column straight into its pinned host slot: a copy behind them
+      // would stand between this step's kernels and the next product
+      double2* col_slot = hred + (size_t)((j + 1) & 1) * (restart + 2) * nrhs;   // column j - 1
       double2* part0 = ws.tmp;
-      double2* part1 = ws.tmp + (size_t)nz * J * nrhs;
+      double2* part1 = final_step ? nullptr : ws.tmp + (size_t)nz * J * nrhs;
       if (!final_step) {
         count_launches(K_GMRES, 1);
-        k_to_dfc<<<nb, tpb, 0, st>>>(ws.w, (int)vsz, ws.wdf);
+        AIM_TRY(launch_chained(k_to_dfc, dim3(nb), tpb, 0, st, static_cast<const double2*>(ws.w), (int)vsz, ws.wdf));
       }
-      count_launches(K_GMRES, 3);
-      k_multidot2_partial_df<<<dim3((J + kDot2Warps - 1) / kDot2Warps, nrhs, nz), 32 * kDot2Warps, 0, st>>>(
-          ws.V, Vj, final_step ? nullptr : ws.wdf, n, nrhs, J, part0, final_step ? nullptr : part1);
-      k_dcgs2_finish<<<blocks_for((long long)J * nrhs, tpb), tpb, 0, st>>>(part0, final_step ? nullptr : part1, nz, J,
-                                                                          nrhs, j, restart, ws.dots, ws.dots2,
-                                                                          ws.dots_df, ws.H);
-      const int hs_blocks = final_step ? 0 : (j + kHsRows - 1) / kHsRows;
-      k_dcgs2_hs_scal<<<dim3(hs_blocks + 1, nrhs), 256, 0, st>>>(ws.H, ws.dots_df, ws.dots, ws.dots2, ws.active, j, nrhs,
-                                                                 restart, final_step ? 1 : 0, ws.hs, ws.colout, ws.H,
-                                                                 ws.scal);
-      if (j >= 1) {
+      count_launches(K_GMRES, 1);
+      AIM_TRY(launch_chained(k_multidot2_partial_df, dim3((J + kDot2Warps - 1) / kDot2Warps, nrhs, nz), 32 * kDot2Warps, 0, st,
+                             V, static_cast<const dfc*>(Vj), wdf, n, nrhs, J, part0, part1));
+      const double2 *cpart0 = part0, *cpart1 = part1;
+      if (j < kStepJ) {
         count_launches(K_GMRES, 1);
-        k_dcgs2_coeffs<<<blocks_for((long long)j * nrhs, tpb), tpb, 0, st>>>(ws.dots, ws.dots2, ws.hs, ws.scal, j, nrhs,
-                                                                             restart, final_step ? 1 : 0, ws.H,
-                                                                             ws.colout, ws.dots2_df, ws.g);
+        AIM_TRY(launch_chained(k_dcgs2_step, dim3(nrhs), kStepThreads, 0, st, cpart0, cpart1, nz, nrhs, j, restart,
+                               static_cast<const int*>(ws.active), ws.H, col_slot, ws.scal, ws.dots2_df, ws.g));
+      } else {
+        count_launches(K_GMRES, 3);
+        AIM_TRY(launch_chained(k_dcgs2_finish, dim3(blocks_for((long long)J * nrhs, tpb)), tpb, 0, st, cpart0, cpart1, nz, J,
+                               nrhs, j, restart, ws.dots, ws.dots2, ws.dots_df, ws.H));
+        const int hs_blocks = final_step ? 0 : (j + kHsRows - 1) / kHsRows;
+        const double2 *D0 = ws.dots, *D1 = ws.dots2, *hs = ws.hs, *scal = ws.scal;
+        AIM_TRY(launch_chained(k_dcgs2_hs_scal, dim3(hs_blocks + 1, nrhs), 256, 0, st, static_cast<const dfc*>(ws.H),
+                               static_cast<const dfc*>(ws.dots_df), D0, D1, static_cast<const int*>(ws.active), j, nrhs,
+                               restart, final_step ? 1 : 0, ws.hs, col_slot, ws.H, ws.scal));
+        AIM_TRY(launch_chained(k_dcgs2_coeffs, dim3(blocks_for((long long)j * nrhs, tpb)), tpb, 0, st, D0, D1, hs, scal, j,
+                               nrhs, restart, final_step ? 1 : 0, ws.H, col_slot, ws.dots2_df, ws.g));
       }
       if (!final_step) {
-        const int nch = (j + kCgsChunk - 1) / kCgsChunk;
-        dfc* p1 = reinterpret_cast<dfc*>(ws.tmp);
-        dfc* p2 = p1 + (size_t)nch * vsz;
-        if (nch > 0) {
-          count_launches(K_GMRES, 1);
-          k_vcombine2_partial_df<<<dim3((n + 255) / 256, nch, nrhs), 256, 0, st>>>(ws.V, ws.dots2_df, ws.g, j, n, nrhs,
-                                                                                   p1, p2);
-        }
         count_launches(K_GMRES, 1);
-        k_vcombine2_finish_df<<<blocks_for((long long)vsz * kFinishLanes, tpb), tpb, 0, st>>>(p1, p2, nch, n, nrhs, ws.scal,
-                                                                                             Vj, ws.w, Vj + vsz, ws.cur);
+        AIM_TRY(launch_chained(k_vcombine2_df, dim3((n + 31) / 32, nrhs), 32 * kUpdateWarps, 0, st, V,
+                               static_cast<const dfc*>(ws.dots2_df), static_cast<const dfc*>(ws.g), j, n, nrhs,
+                               static_cast<const double2*>(ws.scal), Vj, static_cast<const double2*>(ws.w), Vj + vsz, ws.cur));
       }
-      AIM_CUDA_TRY(cudaGetLastError());
-      if (j >= 1) {
-        double2* slot = hred + (size_t)((j - 1) & 1) * (restart + 2) * nrhs;
-        AIM_CUDA_TRY(cudaMemcpyAsync(slot, ws.colout, (size_t)(j + 1) * nrhs * sizeof(double2), cudaMemcpyDeviceToHost, st));
-        AIM_CUDA_TRY(cudaEventRecord(col_ready.e[(j - 1) & 1], st));
-      }
+      if (j >= 1) AIM_CUDA_TRY(cudaEventRecord(col_ready.e[(j - 1) & 1], st));
       return AIM_OK;
     };
     int jdone = 0;
