@@ -158,6 +158,8 @@ struct PassSpec {
   double2 out_scale;               // overall factor on the gathered result
 };
 
+struct MultiLauncher;
+
 }  // namespace aim
 
 struct aim_ctx {
@@ -189,6 +191,7 @@ struct aim_ctx {
   // Gram inverse, row i: entries for columns (i + d) mod n, d = -band..band
   double* gram_inv = nullptr;
   int gram_band = 0;
+  int gram_d0 = 0, gram_cnt = 0;   // the offsets [d0, d0 + cnt) of a row that are applied (gram_window)
   // entry counts of the scatter and gather lists and of gram_inv (for aim_export_setup)
   size_t n_sc = 0, n_ga = 0, n_gram = 0;
   // geometry: host copy and device vertices
@@ -205,6 +208,7 @@ struct aim_ctx {
   int reserved_rhs[3] = {0, 0, 0};   // per precision (AIM_FP64, AIM_MIXED, AIM_FP64_NATIVE)
   // launch schedule per precision: default_schedule, aim_set_schedule or aim_autotune
   aim::Schedule sched[3] = {};
+  aim::MultiLauncher* multi = nullptr;   // buffers of the multi-context calls that this context leads
   // bookkeeping
   std::vector<std::pair<const void*, size_t>> smem_raised;   // dynamic shared memory limits raised so far
   std::vector<void*> allocations;
@@ -311,6 +315,17 @@ template <typename T>
 aim_status grid_product_dense(aim_ctx* ctx, bool filtered, int nrhs, const double2* u, double2* v, void* inter,
                               size_t inter_bytes, cudaStream_t st);
 aim_status gram_inv_apply(aim_ctx* ctx, int nrhs, const double2* x, double2* y, cudaStream_t st);
+// y = G^-1 x of several contexts in one launch
+constexpr int kMaxMultiJobs = 32;
+struct GramCall {
+  const aim_ctx* ctx;
+  int nrhs;
+  const double2* x;
+  double2* y;
+};
+aim_status gram_inv_apply_multi(const GramCall* calls, int count, cudaStream_t st);
+// the applied window of the stored rows of G^-1 (host values), set in the context
+void gram_window(aim_ctx* ctx, const double* gi);
 size_t inter_bytes_needed(const aim_ctx* ctx, int channels, int precision);
 
 // several grid passes of several contexts in one persistent launch (matvec_kernels.cuh)
@@ -329,13 +344,15 @@ aim_status apply_op(aim_ctx* ctx, aim_op op, int nrhs, const double2* x, double2
                     cudaStream_t st);
 aim_status reserve(aim_ctx* ctx, int nrhs, int precision);
 
-// Buffers of a multi-context launch: the barrier words and the error flags of its stages
-// (pinned). Owned by one caller at a time.
+// Buffers of a multi-context launch: per stage the barrier words and the error flag the waits poll
+// (device), and the flag the host reads (pinned, written by a CTA that gives up). The barrier counts
+// back to zero and the flags stay zero as long as no launch gives up, so they are zeroed once, and
+// again after a failure. Owned by one caller at a time: a batcher, or the first context of a call.
 struct MultiLauncher {
   unsigned* scratch = nullptr;   // 4 words per stage
-  int* err_host = nullptr;       // one flag per stage (pinned)
-  aim_status init();
-  aim_status check();            // after a synchronisation: AIM_ETIMEOUT if a launch gave up
+  int* err_host = nullptr;       // one flag per stage
+  aim_status init(cudaStream_t st);
+  aim_status check(cudaStream_t st);   // after a synchronisation: AIM_ETIMEOUT if a launch gave up
   ~MultiLauncher();
 };
 // y_i = A_i x_i for `count` contexts (device vectors), every grid pass stage of all of them in one

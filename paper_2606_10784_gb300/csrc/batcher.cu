@@ -175,7 +175,7 @@ aim_status aim_batcher_create(int max_wait_us, aim_batcher** out) {
   b->events.resize(64, nullptr);
   for (auto& e : b->events)
     if (s == AIM_OK && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) s = fail(AIM_ECUDA, "batcher event");
-  if (s == AIM_OK) s = b->ml.init();
+  if (s == AIM_OK) s = b->ml.init(b->stream);
   if (s != AIM_OK) {
     aim_batcher_destroy(b);
     return s;
@@ -224,7 +224,7 @@ aim_status aim_solve_batched(aim_batcher* b, aim_ctx* ctx, aim_op system, int nr
     // a fused launch whose grid barrier gave up (its flag is read once the launches are done)
     std::lock_guard<std::mutex> lk(b->mu);
     if (cudaStreamQuery(b->stream) == cudaSuccess) {
-      const aim_status e = b->ml.check();
+      const aim_status e = b->ml.check(b->stream);
       if (e != AIM_OK) b->broken = s = e;
     }
   }

@@ -209,24 +209,32 @@ aim_status device_spectra_and_near(aim_ctx* ctx, const HostSetup& hs, cudaStream
 // ------------------------------------------------------------------------------------
 constexpr int kMultiStages = 2;
 
-aim_status MultiLauncher::init() {
+aim_status MultiLauncher::init(cudaStream_t st) {
   if (scratch != nullptr) return AIM_OK;
   void* p = nullptr;
-  AIM_CUDA_TRY(cudaMalloc(&p, kMultiStages * 4 * sizeof(unsigned)));
-  scratch = static_cast<unsigned*>(p);
   AIM_CUDA_TRY(cudaMallocHost(&p, kMultiStages * sizeof(int)));
   err_host = static_cast<int*>(p);
   for (int i = 0; i < kMultiStages; ++i) err_host[i] = 0;
+  AIM_CUDA_TRY(cudaMalloc(&p, kMultiStages * 4 * sizeof(unsigned)));
+  const cudaError_t e = cudaMemsetAsync(p, 0, kMultiStages * 4 * sizeof(unsigned), st);
+  if (e != cudaSuccess) {
+    cudaFree(p);
+    return fail(AIM_ECUDA, std::string("multi-context buffers: ") + cudaGetErrorString(e));
+  }
+  scratch = static_cast<unsigned*>(p);
   return AIM_OK;
 }
 
-aim_status MultiLauncher::check() {
-  for (int i = 0; i < kMultiStages; ++i)
-    if (err_host != nullptr && err_host[i] != 0) {
-      err_host[i] = 0;
-      return fail(AIM_ETIMEOUT, "a grid barrier of the multi-context launch gave up waiting");
-    }
-  return AIM_OK;
+aim_status MultiLauncher::check(cudaStream_t st) {
+  bool bad = false;
+  for (int i = 0; i < kMultiStages; ++i) {
+    bad = bad || (err_host != nullptr && err_host[i] != 0);
+    if (err_host != nullptr) err_host[i] = 0;
+  }
+  if (!bad) return AIM_OK;
+  cudaMemsetAsync(scratch, 0, kMultiStages * 4 * sizeof(unsigned), st);
+  cudaStreamSynchronize(st);   // the next call may use another stream
+  return fail(AIM_ETIMEOUT, "a grid barrier of the multi-context launch gave up waiting");
 }
 
 MultiLauncher::~MultiLauncher() {
@@ -246,8 +254,9 @@ static aim_status multi_stage(MultiLauncher& ml, int stage, const std::vector<Mu
 
 aim_status apply_op_multi(MultiLauncher& ml, int count, aim_ctx* const* ctxs, const aim_op* ops, const int* nrhs,
                           const double2* const* x, double2* const* y, int precision, cudaStream_t st) {
-  AIM_TRY(ml.init());
+  AIM_TRY(ml.init(st));
   std::vector<MultiPassSpec> first, second;
+  std::vector<GramCall> between, last;
   for (int i = 0; i < count; ++i) {
     aim_ctx* ctx = ctxs[i];
     const bool te = ctx->form == AIM_TE_P1_GALERKIN;
@@ -270,13 +279,16 @@ aim_status apply_op_multi(MultiLauncher& ml, int count, aim_ctx* const* ctxs, co
         break;
       case AIM_OP_GRAM_INV:
         if (!te) return fail(AIM_ESTATE, "G is a TE operator");
+        between.push_back({ctx, nrhs[i], x[i], y[i]});
         break;
       case AIM_OP_CALDERON: case AIM_OP_CALDERON_ALPHA: case AIM_OP_CALDERON_ALPHA2: {
         if (!te) return fail(AIM_ESTATE, "the Calderon product is a TE operator");
         double2* t1 = ctx->vec_ws;
         double2* t2 = ctx->vec_ws + (size_t)nrhs[i] * ctx->n;
         first.push_back({ctx, make_spec(ctx, op == AIM_OP_CALDERON_ALPHA2 ? AIM_OP_N_ALPHA : AIM_OP_N), nrhs[i], x[i], t1});
+        between.push_back({ctx, nrhs[i], t1, t2});
         second.push_back({ctx, make_spec(ctx, op == AIM_OP_CALDERON ? AIM_OP_S : AIM_OP_S_ALPHA), nrhs[i], t2, t1});
+        last.push_back({ctx, nrhs[i], t1, y[i]});
         break;
       }
       default:
@@ -285,21 +297,10 @@ aim_status apply_op_multi(MultiLauncher& ml, int count, aim_ctx* const* ctxs, co
   }
   // stage 1: every context's first grid pass, then the Gram inverses between the Calderon factors
   AIM_TRY(multi_stage(ml, 0, first, precision, st));
-  for (int i = 0; i < count; ++i) {
-    aim_ctx* ctx = ctxs[i];
-    const aim_op op = ops[i];
-    if (op == AIM_OP_GRAM_INV) AIM_TRY(gram_inv_apply(ctx, nrhs[i], x[i], y[i], st));
-    if (op == AIM_OP_CALDERON || op == AIM_OP_CALDERON_ALPHA || op == AIM_OP_CALDERON_ALPHA2)
-      AIM_TRY(gram_inv_apply(ctx, nrhs[i], ctx->vec_ws, ctx->vec_ws + (size_t)nrhs[i] * ctx->n, st));
-  }
+  AIM_TRY(gram_inv_apply_multi(between.data(), (int)between.size(), st));
   // stage 2: the single-layer factors of the Calderon products, then their last Gram inverse
   AIM_TRY(multi_stage(ml, 1, second, precision, st));
-  for (int i = 0; i < count; ++i) {
-    const aim_op op = ops[i];
-    if (op == AIM_OP_CALDERON || op == AIM_OP_CALDERON_ALPHA || op == AIM_OP_CALDERON_ALPHA2)
-      AIM_TRY(gram_inv_apply(ctxs[i], nrhs[i], ctxs[i]->vec_ws, y[i], st));
-  }
-  return AIM_OK;
+  return gram_inv_apply_multi(last.data(), (int)last.size(), st);
 }
 
 // e^{-2 pi i t / P}, t < P, from its FP64 (re, im) pairs: the FP64, complex64 and double-float
@@ -410,6 +411,7 @@ void aim_destroy(aim_ctx* ctx) {
   if (ctx->kry) cudaFree(ctx->kry);
   if (ctx->red) cudaFree(ctx->red);
   if (ctx->red_host) cudaFreeHost(ctx->red_host);
+  delete ctx->multi;
   delete ctx;
 }
 
@@ -456,6 +458,7 @@ aim_status aim_setup(const aim_geometry* geometry, double k, const aim_grid* gri
   if (!hs.gram_inv.empty()) {
     AIM_TRY(upload(ctx, &ctx->gram_inv, hs.gram_inv, st));
     ctx->gram_band = hs.gram_band;
+    gram_window(ctx, hs.gram_inv.data());
   }
   ctx->n_sc = hs.sc_col.size();
   ctx->n_ga = hs.ga_act.size();
@@ -648,12 +651,14 @@ aim_status aim_matvec_multi(int count, aim_ctx* const* ctxs, const aim_op* ops, 
     AIM_TRY(check_device(ctxs[i]));
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  MultiLauncher ml;
+  if (ctxs[0]->multi == nullptr) ctxs[0]->multi = new (std::nothrow) MultiLauncher();
+  if (ctxs[0]->multi == nullptr) return fail(AIM_ENOMEM, "multi-context launcher");
+  MultiLauncher& ml = *ctxs[0]->multi;
   aim_status s = apply_op_multi(ml, count, ctxs, ops, nrhs, reinterpret_cast<const double2* const*>(x),
                                 reinterpret_cast<double2* const*>(y), precision, st);
   const cudaError_t e = cudaStreamSynchronize(st);
   if (s == AIM_OK && e != cudaSuccess) s = fail(AIM_ECUDA, std::string("multi-context product: ") + cudaGetErrorString(e));
-  if (s == AIM_OK) s = ml.check();
+  if (s == AIM_OK) s = ml.check(st);
   return s;
 }
 

@@ -1,5 +1,7 @@
 // Grid-product helpers shared by every element type: the banded Gram inverse (G^-1 of Eq. 3),
 // workspace sizing, and the feasibility of a launch schedule.
+#include <cmath>
+
 #include "matvec_kernels.cuh"
 
 namespace aim {
@@ -13,24 +15,29 @@ namespace aim {
 // each a chain of cnt dependent loads and FMAs).
 constexpr int kGramLanes = 8;
 
-__global__ void k_gram_inv(const double* __restrict__ gi, int blo, int cnt, int n, int nrhs,
-                           const double2* __restrict__ x, double2* __restrict__ y) {
-  grid_trigger_dependents();
-  grid_dependency_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+struct GramArgs {
+  const double* gi;    // stored rows, `stride` entries each: entry d of row i belongs to column i - blo + d
+  int stride, blo, d0, cnt;   // the entries applied: d0 <= d < d0 + cnt
+  int n, nrhs;
+  const double2* x;
+  double2* y;
+};
+
+// all 32 lanes of every warp call it (the group sums are shuffles)
+__device__ __forceinline__ void gram_item(const GramArgs& a, long long t) {
   const long long o = t / kGramLanes;
   const int g = threadIdx.x & (kGramLanes - 1);
-  const bool valid = o < (long long)n * nrhs;
+  const bool valid = o < (long long)a.n * a.nrhs;
   double re = 0.0, im = 0.0;
   if (valid) {
-    const int r = (int)(o / n), i = (int)(o - (long long)r * n);
-    const double* row = gi + (size_t)i * cnt;
-    const double2* xv = x + (size_t)r * n;
+    const int r = (int)(o / a.n), i = (int)(o - (long long)r * a.n);
+    const double* row = a.gi + (size_t)i * a.stride;
+    const double2* xv = a.x + (size_t)r * a.n;
 #pragma unroll 4
-    for (int d = g; d < cnt; d += kGramLanes) {
-      int j = i - blo + d;
-      if (j < 0) j += n;
-      if (j >= n) j -= n;
+    for (int d = a.d0 + g; d < a.d0 + a.cnt; d += kGramLanes) {
+      int j = i - a.blo + d;
+      if (j < 0) j += a.n;
+      if (j >= a.n) j -= a.n;
       const double gv = row[d];
       const double2 xx = xv[j];
       re = fma(gv, xx.x, re);
@@ -43,7 +50,56 @@ __global__ void k_gram_inv(const double* __restrict__ gi, int blo, int cnt, int 
     re += __shfl_xor_sync(0xffffffffu, re, off);
     im += __shfl_xor_sync(0xffffffffu, im, off);
   }
-  if (valid && g == 0) y[o] = double2{re, im};
+  if (valid && g == 0) a.y[o] = double2{re, im};
+}
+
+__global__ void __launch_bounds__(256) k_gram_inv(GramArgs a) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
+  gram_item(a, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// Several contexts in one launch: the CTAs are dealt out to the jobs in order.
+struct GramMultiArgs {
+  GramArgs jobs[kMaxMultiJobs];
+  int first[kMaxMultiJobs + 1];   // first CTA of each job
+  int njobs;
+};
+
+__global__ void __launch_bounds__(256) k_gram_inv_multi(const __grid_constant__ GramMultiArgs m) {
+  grid_trigger_dependents();
+  grid_dependency_wait();
+  int jb = 0;
+  while (jb + 1 < m.njobs && (int)blockIdx.x >= m.first[jb + 1]) ++jb;   // the same job in every thread of the CTA
+  gram_item(m.jobs[jb], (long long)((int)blockIdx.x - m.first[jb]) * blockDim.x + threadIdx.x);
+}
+
+static GramArgs gram_args(const aim_ctx* ctx, int nrhs, const double2* x, double2* y) {
+  const int blo = ctx->gram_band;
+  return {ctx->gram_inv, (blo * 2 + 1 <= ctx->n) ? 2 * blo + 1 : ctx->n, blo, ctx->gram_d0, ctx->gram_cnt, ctx->n, nrhs, x, y};
+}
+
+// G^-1 decays geometrically off its diagonal (by 0.27 per entry on a uniform mesh), so most of a
+// densely stored row (n <= kGramDenseMax) is far below the rounding of its sum: entries under 2^-70
+// of the row's diagonal at every offset beyond the window are not applied. (n = 400: 75 of 400
+// entries left; seven right-hand sides 21 -> 8 us.) A row stored as a band is applied whole.
+void gram_window(aim_ctx* ctx, const double* gi) {
+  const int n = ctx->n, blo = ctx->gram_band, stride = (blo * 2 + 1 <= n) ? 2 * blo + 1 : n;
+  ctx->gram_d0 = 0;
+  ctx->gram_cnt = stride;
+  if (n > kGramDenseMax) return;
+  int reach = 0;   // largest |d - blo| of an entry that counts
+  for (int i = 0; i < n; ++i) {
+    const double* row = gi + (size_t)i * stride;
+    const double least = std::ldexp(std::fabs(row[blo]), -70);
+    int e = std::max(blo, stride - 1 - blo);
+    while (e > reach && !(blo - e >= 0 && !(std::fabs(row[blo - e]) < least)) &&
+           !(blo + e < stride && !(std::fabs(row[blo + e]) < least)))
+      --e;
+    reach = std::max(reach, e);
+  }
+  ctx->gram_d0 = std::max(0, blo - reach);
+  ctx->gram_cnt = std::min(stride, blo + reach + 1) - ctx->gram_d0;
 }
 
 size_t inter_bytes_needed(const aim_ctx* ctx, int channels, int precision) {
@@ -62,16 +118,31 @@ bool schedule_feasible(int precision, int logH, int logP, const Schedule& s) {
 
 aim_status gram_inv_apply(aim_ctx* ctx, int nrhs, const double2* x, double2* y, cudaStream_t st) {
   if (ctx->gram_inv == nullptr) return fail(AIM_ESTATE, "no Gram matrix on a TM context");
-  const int blo = ctx->gram_band;
-  const int cnt = (blo * 2 + 1 <= ctx->n) ? 2 * blo + 1 : ctx->n;
   const long long threads = (long long)ctx->n * nrhs * kGramLanes;
   const int tpb = gather_threads(threads);
-  {
-    ProfScope ps(K_GRAM, st);
-    AIM_TRY(launch_chained(k_gram_inv, dim3((unsigned)((threads + tpb - 1) / tpb)), tpb, 0, st,
-                           static_cast<const double*>(ctx->gram_inv), blo, cnt, ctx->n, nrhs, x, y));
+  ProfScope ps(K_GRAM, st);
+  return launch_chained(k_gram_inv, dim3((unsigned)((threads + tpb - 1) / tpb)), tpb, 0, st, gram_args(ctx, nrhs, x, y));
+}
+
+aim_status gram_inv_apply_multi(const GramCall* calls, int count, cudaStream_t st) {
+  if (count == 0) return AIM_OK;
+  if (count > kMaxMultiJobs) return fail(AIM_EINVAL, "1 to 32 contexts per multi-context launch");
+  long long threads = 0;
+  for (int i = 0; i < count; ++i) {
+    if (calls[i].ctx->gram_inv == nullptr) return fail(AIM_ESTATE, "no Gram matrix on a TM context");
+    threads += (long long)calls[i].ctx->n * calls[i].nrhs * kGramLanes;
   }
-  return AIM_OK;
+  const int tpb = gather_threads(threads);
+  GramMultiArgs m{};
+  m.njobs = count;
+  for (int i = 0; i < count; ++i) {
+    m.jobs[i] = gram_args(calls[i].ctx, calls[i].nrhs, calls[i].x, calls[i].y);
+    const long long blocks = ((long long)calls[i].ctx->n * calls[i].nrhs * kGramLanes + tpb - 1) / tpb;
+    if (m.first[i] + blocks > 0x7fffffffLL) return fail(AIM_EINVAL, "too many right-hand sides in one multi-context call");
+    m.first[i + 1] = m.first[i] + (int)blocks;
+  }
+  ProfScope ps(K_GRAM, st);
+  return launch_chained(k_gram_inv_multi, dim3((unsigned)m.first[count]), tpb, 0, st, m);
 }
 
 }  // namespace aim

@@ -3,8 +3,8 @@
 
 namespace aim {
 
-extern template aim_status launch_multi_groups<dfc, 1, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
-extern template aim_status launch_multi_groups<dfc, 2, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
+extern template aim_status launch_multi_groups<dfc, 1, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
+extern template aim_status launch_multi_groups<dfc, 2, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
 template aim_status grid_pass_multi<dfc>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
 
 }  // namespace aim

@@ -3,7 +3,7 @@
 
 namespace aim {
 
-template aim_status launch_multi_groups<dfc, 1, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
-template aim_status launch_multi_groups<dfc, 2, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
+template aim_status launch_multi_groups<dfc, 1, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
+template aim_status launch_multi_groups<dfc, 2, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
 
 }  // namespace aim

@@ -3,8 +3,8 @@
 
 namespace aim {
 
-extern template aim_status launch_multi_groups<float2, 1, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
-extern template aim_status launch_multi_groups<float2, 2, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
+extern template aim_status launch_multi_groups<float2, 1, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
+extern template aim_status launch_multi_groups<float2, 2, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
 template aim_status grid_pass_multi<float2>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
 
 }  // namespace aim

@@ -3,7 +3,7 @@
 
 namespace aim {
 
-template aim_status launch_multi_groups<float2, 1, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
-template aim_status launch_multi_groups<float2, 2, 4>(const MultiPassSpec*, int, unsigned*, cudaStream_t);
+template aim_status launch_multi_groups<float2, 1, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
+template aim_status launch_multi_groups<float2, 2, 4>(const MultiPassSpec*, int, unsigned*, int*, cudaStream_t);
 
 }  // namespace aim

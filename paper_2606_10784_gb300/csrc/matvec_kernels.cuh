@@ -1130,8 +1130,6 @@ aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2
 // barrier separates the phases. The launch is cooperative, so all CTAs are resident and the
 // barrier completes; its waits are bounded all the same: after max_spins polls a CTA records the
 // failure in *err and every CTA leaves at its next barrier, and the host reports AIM_ETIMEOUT.
-constexpr int kMaxMultiJobs = 32;
-
 struct MultiJob {
   AntArgs aa;
   RowFwdArgs fa;
@@ -1152,8 +1150,9 @@ struct MultiArgs {
   MultiJob jobs[kMaxMultiJobs];
   int njobs;
   long long off[5][kMaxMultiJobs + 1];   // prefix sums of the items of each phase over the jobs
-  unsigned* bar;                         // [arrivals, generation], zero at launch
-  int* err;                              // 1 when a barrier wait gave up
+  unsigned* bar;                         // [arrivals, generation]: arrivals are zero between launches
+  int* err;                              // 1 when a barrier wait gave up (polled by the other waits)
+  int* err_host;                         // the same for the host (pinned)
   long long max_spins;
 };
 
@@ -1177,6 +1176,7 @@ __device__ __forceinline__ bool multi_grid_barrier(const MultiArgs& m) {
         if (*err != 0) break;
         if (++spins > m.max_spins) {
           atomicExch(m.err, 1);
+          *static_cast<volatile int*>(m.err_host) = 1;
           break;
         }
         __nanosleep(128);
@@ -1230,8 +1230,8 @@ __global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_grid_multi(
 
 // Runs the passes (all of element type CT, all contexts on the schedule geometry of jobs[0]: the
 // same transforms per thread and elements per thread) in one persistent cooperative launch.
-// scratch: 16 device bytes for the barrier and the error flag (zeroed here on the stream);
-// err_host: pinned host int that receives the error flag after the launch (read it after a sync).
+// scratch: 16 device bytes for the barrier and the error flag, err_host: the host's flag, as
+// MultiLauncher keeps them.
 template <typename CT>
 aim_status grid_pass_multi(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host, cudaStream_t st);
 
@@ -1256,7 +1256,7 @@ static bool multi_fits(int B, int H) {
 }
 
 template <typename CT, int TPT, int LOGE>
-static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned* scratch, cudaStream_t st) {
+static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host, cudaStream_t st) {
   using T2 = CT;
   using VT = typename GridT<CT>::VT;
   constexpr int LPT = 3 - TPT;
@@ -1269,6 +1269,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
   m.njobs = count;
   m.bar = scratch;
   m.err = reinterpret_cast<int*>(scratch + 2);
+  m.err_host = err_host;
   m.max_spins = 20000000;   // ~2.5 s of 128 ns polls
   size_t smem = 0;
   for (int i = 0; i < count; ++i) {
@@ -1363,7 +1364,6 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
   long long most = 0;
   for (int ph = 0; ph < 5; ++ph) most = std::max(most, m.off[ph][count]);
   const int grid = (int)std::max(1LL, std::min<long long>((long long)sms * per_sm, most));
-  AIM_CUDA_TRY(cudaMemsetAsync(scratch, 0, 2 * sizeof(unsigned), st));   // the barrier words (not the error flag)
   {
     // one launch: the three grid passes and the gathers of every job
     ProfScope ps(K_MULTI, st);
@@ -1376,7 +1376,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
 // Splits the passes into the fewest launches whose contexts can share one CTA size (longest
 // transforms first; a context too short for the CTA size of a longer one goes to a later launch).
 template <typename CT, int TPT, int LOGE>
-aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned* scratch, cudaStream_t st) {
+aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host, cudaStream_t st) {
   std::vector<int> left(count);
   for (int i = 0; i < count; ++i) left[i] = i;
   std::stable_sort(left.begin(), left.end(), [&](int a, int b) { return passes[a].ctx->H > passes[b].ctx->H; });
@@ -1389,7 +1389,7 @@ aim_status launch_multi_groups(const MultiPassSpec* passes, int count, unsigned*
       if (multi_fits<CT, TPT, LOGE>(B, passes[i].ctx->H)) group.push_back(passes[i]);
       else rest.push_back(i);
     }
-    AIM_TRY((launch_multi<CT, TPT, LOGE>(group.data(), (int)group.size(), scratch, st)));
+    AIM_TRY((launch_multi<CT, TPT, LOGE>(group.data(), (int)group.size(), scratch, err_host, st)));
     left.swap(rest);
   }
   return AIM_OK;
@@ -1408,20 +1408,18 @@ aim_status grid_pass_multi(const MultiPassSpec* passes, int count, unsigned* scr
     if (o.tpt != sc.tpt || loge_of(o) != loge_of(sc))
       return fail(AIM_EINVAL, "contexts of one multi-context launch must share the pass geometry of their schedule");
   }
-  AIM_CUDA_TRY(cudaMemsetAsync(scratch + 2, 0, sizeof(int), st));   // the stage's error flag
   if constexpr (std::is_same<CT, double2>::value) {
-    AIM_TRY((launch_multi_groups<CT, 2, 4>(passes, count, scratch, st)));
+    AIM_TRY((launch_multi_groups<CT, 2, 4>(passes, count, scratch, err_host, st)));
   } else {
     std::vector<MultiPassSpec> of[2];
     for (int i = 0; i < count; ++i) of[loge_of(passes[i].ctx->sched[p]) - 3].push_back(passes[i]);
     if (!of[0].empty())
-      AIM_TRY((sc.tpt == 1 ? launch_multi_groups<CT, 1, 3>(of[0].data(), (int)of[0].size(), scratch, st)
-                           : launch_multi_groups<CT, 2, 3>(of[0].data(), (int)of[0].size(), scratch, st)));
+      AIM_TRY((sc.tpt == 1 ? launch_multi_groups<CT, 1, 3>(of[0].data(), (int)of[0].size(), scratch, err_host, st)
+                           : launch_multi_groups<CT, 2, 3>(of[0].data(), (int)of[0].size(), scratch, err_host, st)));
     if (!of[1].empty())
-      AIM_TRY((sc.tpt == 1 ? launch_multi_groups<CT, 1, 4>(of[1].data(), (int)of[1].size(), scratch, st)
-                           : launch_multi_groups<CT, 2, 4>(of[1].data(), (int)of[1].size(), scratch, st)));
+      AIM_TRY((sc.tpt == 1 ? launch_multi_groups<CT, 1, 4>(of[1].data(), (int)of[1].size(), scratch, err_host, st)
+                           : launch_multi_groups<CT, 2, 4>(of[1].data(), (int)of[1].size(), scratch, err_host, st)));
   }
-  AIM_CUDA_TRY(cudaMemcpyAsync(err_host, scratch + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
   return AIM_OK;
 }
 
