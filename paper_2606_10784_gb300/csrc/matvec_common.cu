@@ -28,21 +28,33 @@ __device__ __forceinline__ void gram_item(const GramArgs& a, long long t) {
   const long long o = t / kGramLanes;
   const int g = threadIdx.x & (kGramLanes - 1);
   const bool valid = o < (long long)a.n * a.nrhs;
+  const int r = valid ? (int)(o / a.n) : 0, i = valid ? (int)(o - (long long)r * a.n) : 0;
+  const double* row = a.gi + (size_t)i * a.stride;
+  // the row belongs to the context: the lane's first kPre entries (a band of 81 has at most 11 per
+  // lane) are loaded before the wait for x
+  constexpr int kPre = 11;
+  double pre[kPre];
+#pragma unroll
+  for (int u = 0; u < kPre; ++u) pre[u] = row[min(a.d0 + g + u * kGramLanes, a.d0 + a.cnt - 1)];
+  grid_dependency_wait();
   double re = 0.0, im = 0.0;
   if (valid) {
-    const int r = (int)(o / a.n), i = (int)(o - (long long)r * a.n);
-    const double* row = a.gi + (size_t)i * a.stride;
     const double2* xv = a.x + (size_t)r * a.n;
-#pragma unroll 4
-    for (int d = a.d0 + g; d < a.d0 + a.cnt; d += kGramLanes) {
+    auto entry = [&](int d, double gv) {
       int j = i - a.blo + d;
       if (j < 0) j += a.n;
       if (j >= a.n) j -= a.n;
-      const double gv = row[d];
       const double2 xx = xv[j];
       re = fma(gv, xx.x, re);
       im = fma(gv, xx.y, im);
+    };
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      const int d = a.d0 + g + u * kGramLanes;
+      if (d < a.d0 + a.cnt) entry(d, pre[u]);
     }
+#pragma unroll 4
+    for (int d = a.d0 + g + kPre * kGramLanes; d < a.d0 + a.cnt; d += kGramLanes) entry(d, row[d]);
   }
   // every lane of the warp takes part in the shuffles (groups past the end carry zeros)
 #pragma unroll
@@ -55,7 +67,6 @@ __device__ __forceinline__ void gram_item(const GramArgs& a, long long t) {
 
 __global__ void __launch_bounds__(256) k_gram_inv(GramArgs a) {
   grid_trigger_dependents();
-  grid_dependency_wait();
   gram_item(a, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -68,7 +79,6 @@ struct GramMultiArgs {
 
 __global__ void __launch_bounds__(256) k_gram_inv_multi(const __grid_constant__ GramMultiArgs m) {
   grid_trigger_dependents();
-  grid_dependency_wait();
   int jb = 0;
   while (jb + 1 < m.njobs && (int)blockIdx.x >= m.first[jb + 1]) ++jb;   // the same job in every thread of the CTA
   gram_item(m.jobs[jb], (long long)((int)blockIdx.x - m.first[jb]) * blockDim.x + threadIdx.x);

@@ -61,25 +61,31 @@ constexpr int kAntChunk = 8, kAntThreads = 64;
 
 template <typename CT, int NP>
 __device__ __forceinline__ void ant_item(const AntArgs& a, long long t) {
-  if (t >= (long long)a.n_act * a.nrhs) return;
-  const int r = (int)(t / a.n_act), ap = (int)(t - (long long)r * a.n_act);
+  const bool valid = t < (long long)a.n_act * a.nrhs;
+  const int r = valid ? (int)(t / a.n_act) : 0, ap = valid ? (int)(t - (long long)r * a.n_act) : 0;
   const double2* xv = a.x + (size_t)r * a.n;
   double re[NP], im[NP];
 #pragma unroll
   for (int q = 0; q < NP; ++q) re[q] = im[q] = 0.0;
-  const int e0 = a.sc_ptr[ap], e1 = a.sc_ptr[ap + 1];
-  for (int e = e0; e < e1; e += kAntChunk) {
-    int col[kAntChunk];
-    double ww[NP][kAntChunk];
-    double2 xx[kAntChunk];
+  const int e0 = a.sc_ptr[ap], e1 = valid ? a.sc_ptr[ap + 1] : e0;
+  int col[kAntChunk];
+  double ww[NP][kAntChunk];
+  auto lists = [&](int e) {   // entries past the end repeat the last one with weight 0
 #pragma unroll
     for (int u = 0; u < kAntChunk; ++u) {
-      col[u] = e + u < e1 ? a.sc_col[e + u] : 0;
+      const int ee = min(e + u, e1 - 1);
+      col[u] = a.sc_col[max(ee, 0)];
 #pragma unroll
-      for (int q = 0; q < NP; ++q) ww[q][u] = e + u < e1 ? a.w[q][e + u] : 0.0;
+      for (int q = 0; q < NP; ++q) ww[q][u] = a.w[q][max(ee, 0)];
     }
+  };
+  lists(e0);
+  grid_dependency_wait();   // the lists belong to the context: only x comes from an earlier kernel
+  for (int e = e0; e < e1; e += kAntChunk) {
+    if (e != e0) lists(e);
+    double2 xx[kAntChunk];
 #pragma unroll
-    for (int u = 0; u < kAntChunk; ++u) xx[u] = e + u < e1 ? xv[col[u]] : double2{0.0, 0.0};
+    for (int u = 0; u < kAntChunk; ++u) xx[u] = xv[col[u]];
 #pragma unroll
     for (int u = 0; u < kAntChunk; ++u) {
       if (e + u < e1) {
@@ -91,6 +97,7 @@ __device__ __forceinline__ void ant_item(const AntArgs& a, long long t) {
       }
     }
   }
+  if (!valid) return;
   CT* out = static_cast<CT*>(a.u) + (size_t)r * a.n_act + ap;
 #pragma unroll
   for (int q = 0; q < NP; ++q) out[(size_t)q * a.nrhs * a.n_act] = cfrom<CT>(re[q], im[q]);
@@ -99,7 +106,6 @@ __device__ __forceinline__ void ant_item(const AntArgs& a, long long t) {
 template <typename CT, int NP>
 __global__ void __launch_bounds__(kAntThreads) k_anterpolate(AntArgs a) {
   grid_trigger_dependents();
-  grid_dependency_wait();
   ant_item<CT, NP>(a, (long long)blockIdx.x * kAntThreads + threadIdx.x);
 }
 
@@ -700,13 +706,30 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vbloc
   double re[RB], im[RB];
 #pragma unroll
   for (int q = 0; q < RB; ++q) re[q] = im[q] = 0.0;
+  // the lists belong to the context: those of the lane's first kPre entries (the usual row has about
+  // 45 entries, six per lane) and of the near row are loaded before the wait for the grid values
+  constexpr int kPre = 6;
+  const int e0 = a.ga_ptr[i], e1 = valid ? a.ga_ptr[i + 1] : e0;
+  int pre_act[kPre];
+#pragma unroll
+  for (int u = 0; u < kPre; ++u) pre_act[u] = a.ga_act[max(min(e0 + g + u * kGatherLanes, e1 - 1), 0)];
+  // one or two right-hand sides: all projections of an entry together (their loads are
+  // independent); more: projection by projection, which keeps the sums in registers. The sums
+  // of a projection run over the same entries in the same order either way.
+  constexpr int PG = RB <= 2 ? NP : 1;
+  double pre_w[PG][kPre];
+#pragma unroll
+  for (int p = 0; p < PG; ++p)
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) pre_w[p][u] = a.w[p][max(min(e0 + g + u * kGatherLanes, e1 - 1), 0)];
+  int n0 = 0, n1 = 0;
+  if (a.nptr != nullptr && valid) {
+    n0 = a.nptr[i];
+    n1 = a.nptr[i + 1];
+  }
+  grid_dependency_wait();
   if (valid) {
-    const int e0 = a.ga_ptr[i], e1 = a.ga_ptr[i + 1];
     const T2* v = static_cast<const T2*>(a.vact) + (size_t)r0 * a.n_act;
-    // one or two right-hand sides: all projections of an entry together (their loads are
-    // independent); more: projection by projection, which keeps the sums in registers. The sums
-    // of a projection run over the same entries in the same order either way.
-    constexpr int PG = RB <= 2 ? NP : 1;
 #pragma unroll
     for (int p0 = 0; p0 < NP; p0 += PG) {
       Acc cr[PG][RB], ci[PG][RB];
@@ -714,12 +737,10 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vbloc
       for (int p = 0; p < PG; ++p)
 #pragma unroll
         for (int q = 0; q < RB; ++q) cr[p][q] = ci[p][q] = Acc(0);
-#pragma unroll 2
-      for (int e = e0 + g; e < e1; e += kGatherLanes) {
-        const int act = a.ga_act[e];
+      auto entry = [&](int act, const double (&w)[PG]) {
 #pragma unroll
         for (int p = 0; p < PG; ++p) {
-          const Acc ww = static_cast<Acc>(a.w[p0 + p][e]);
+          const Acc ww = static_cast<Acc>(w[p]);
 #pragma unroll
           for (int q = 0; q < RB; ++q) {
             if (q < nr) {
@@ -729,6 +750,22 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vbloc
             }
           }
         }
+      };
+#pragma unroll
+      for (int u = 0; u < kPre; ++u) {
+        const int e = e0 + g + u * kGatherLanes;
+        if (e < e1) {
+          double w[PG];
+#pragma unroll
+          for (int p = 0; p < PG; ++p) w[p] = p0 == 0 ? pre_w[p][u] : a.w[p0 + p][e];
+          entry(pre_act[u], w);
+        }
+      }
+      for (int e = e0 + g + kPre * kGatherLanes; e < e1; e += kGatherLanes) {
+        double w[PG];
+#pragma unroll
+        for (int p = 0; p < PG; ++p) w[p] = a.w[p0 + p][e];
+        entry(a.ga_act[e], w);
       }
 #pragma unroll
       for (int p = 0; p < PG; ++p) {
@@ -740,21 +777,18 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vbloc
         }
       }
     }
-    if (a.nptr != nullptr) {
-      const T2* val = static_cast<const T2*>(a.nval);
-      const int n1 = a.nptr[i + 1];
-#pragma unroll 2
-      for (int e = a.nptr[i] + g; e < n1; e += kGatherLanes) {
-        const T2 cv = val[e];
-        const double cx = cv.x, cy = cv.y;
-        const int col = a.ncol[e];
+    const T2* val = static_cast<const T2*>(a.nval);
+#pragma unroll 3
+    for (int e = n0 + g; e < n1; e += kGatherLanes) {
+      const T2 cv = val[e];
+      const double cx = cv.x, cy = cv.y;
+      const int col = a.ncol[e];
 #pragma unroll
-        for (int q = 0; q < RB; ++q) {
-          if (q < nr) {
-            const double2 xx = a.x[(size_t)(r0 + q) * a.n + col];
-            re[q] = fma(cx, xx.x, fma(-cy, xx.y, re[q]));
-            im[q] = fma(cx, xx.y, fma(cy, xx.x, im[q]));
-          }
+      for (int q = 0; q < RB; ++q) {
+        if (q < nr) {
+          const double2 xx = a.x[(size_t)(r0 + q) * a.n + col];
+          re[q] = fma(cx, xx.x, fma(-cy, xx.y, re[q]));
+          im[q] = fma(cx, xx.y, fma(cy, xx.x, im[q]));
         }
       }
     }
@@ -790,7 +824,6 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vbloc
 template <typename T2, int NP, int RB>
 __global__ void __launch_bounds__(256) k_gather(GatherArgs a) {
   grid_trigger_dependents();
-  grid_dependency_wait();
   gather_item<T2, NP, RB>(a, blockIdx.x);
 }
 
@@ -801,9 +834,15 @@ inline int gather_threads(long long threads) {
   return tpb;
 }
 
-// Right-hand sides of a gather group: the power of two at or above their number, at most 8 (64
-// lanes' worth of sums would spill).
-inline int gather_rhs_block(int nrhs) { return nrhs >= 5 ? 8 : nrhs >= 3 ? 4 : nrhs; }
+// Right-hand sides of a gather group: the power of two at or above their number, at most 8 (more
+// sums would spill), and fewer while that leaves fewer warps than four per SM: a group's FP64 work
+// grows with its right-hand sides, and short products are better off on more SMs (N = 400, seven
+// right-hand sides: 19 us in groups of eight).
+inline int gather_rhs_block(int n, int nrhs) {
+  int rb = nrhs >= 5 ? 8 : nrhs >= 3 ? 4 : nrhs;
+  while (rb > 1 && (long long)n * ((nrhs + rb - 1) / rb) * kGatherLanes < 608 * 32) rb >>= 1;
+  return rb;
+}
 
 // ------------------------------------------------------------------------------------
 // launch configuration
@@ -1099,7 +1138,7 @@ aim_status grid_pass(aim_ctx* ctx, const PassSpec& spec, int nrhs, const double2
   AIM_TRY(launch_three_passes<CT>(ctx, channels, spec.filtered, fa, ia, ctx->inter, st));
 
   const GatherArgs ga = gather_args<CT>(ctx, spec, nrhs, x, y);
-  const int rb = gather_rhs_block(nrhs);
+  const int rb = gather_rhs_block(ctx->n, nrhs);
   const long long threads = (long long)ctx->n * ((nrhs + rb - 1) / rb) * kGatherLanes;
   const int tpb = gather_threads(threads);
   const dim3 blocks((unsigned)((threads + tpb - 1) / tpb));
