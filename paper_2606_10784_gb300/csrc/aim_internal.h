@@ -99,6 +99,7 @@ constexpr int kMinP = 64;            // smallest: every half-length transform ha
 constexpr int kMaxProj = 4;          // TE: phi, phi', n_x phi, n_y phi
 constexpr int kGramBand = 40;        // half bandwidth of the banded G^-1 for large N
 constexpr int kGramDenseMax = 512;   // N at or below which G^-1 is stored dense
+constexpr int kGramRingMin = 128;    // N from which its rows are products of elimination ratios around the ring
 
 // column-tile width of the intermediate layout (32-byte chunks)
 template <typename T> struct TileW;
@@ -271,8 +272,9 @@ struct HostSetup {
   std::vector<double> sr_w;
   // near field: unknown pairs (CSR rows) and the segment pairs they need
   std::vector<int> near_ptr, near_col;
-  std::vector<int> seg_e, seg_f;          // unique segment pairs (TE) or point-segment pairs (TM)
-  std::vector<int> pair_seg_idx;          // TE: 4 per near entry (e=i,f=j),(i,j-1),(i-1,j),(i-1,j-1); TM: 1
+  std::vector<int> seg_e, seg_f;          // TE: unique segment pairs, e <= f
+  // TE: 4 per near entry, (e=i,f=j),(i,j-1),(i-1,j),(i-1,j-1): index of the pair, ~index of (f, e)
+  std::vector<int> pair_seg_idx;
   // Gram inverse
   std::vector<double> gram_inv;
   int gram_band = 0;

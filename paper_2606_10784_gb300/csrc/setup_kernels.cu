@@ -432,7 +432,9 @@ __global__ void k_te_near_entries(TENearArgs a) {
   const int as[4] = {0, 0, 1, 1}, bs[4] = {0, 1, 0, 1};
   double2 S{0, 0}, N{0, 0};
   for (int c = 0; c < 4; ++c) {
-    const double2* I = a.I + (size_t)a.pair_seg_idx[(size_t)wid * 4 + c] * 4;
+    // a pair stored the other way round has its two hats exchanged
+    const int id = a.pair_seg_idx[(size_t)wid * 4 + c];
+    const double2* I = a.I + (size_t)(id < 0 ? ~id : id) * 4;
     const int e = es[c], f = fs[c];
     const double2 ve0 = a.nodes[e], ve1 = a.nodes[(e + 1) % n];
     const double2 vf0 = a.nodes[f], vf1 = a.nodes[(f + 1) % n];
@@ -440,7 +442,7 @@ __global__ void k_te_near_entries(TENearArgs a) {
     const double he = hypot(dex, dey), hf = hypot(dfx, dfy);
     // n = (t_y, -t_x): n_e . n_f = t_e . t_f
     const double nn = (dex * dfx + dey * dfy) / (he * hf);
-    const double2 Iab = I[as[c] * 2 + bs[c]];
+    const double2 Iab = I[id < 0 ? bs[c] * 2 + as[c] : as[c] * 2 + bs[c]];
     const double2 J = double2{I[0].x + I[1].x + I[2].x + I[3].x, I[0].y + I[1].y + I[2].y + I[3].y};
     const double dd = ((as[c] ? 1.0 : -1.0) / he) * ((bs[c] ? 1.0 : -1.0) / hf);
     S.x += Iab.x;
