@@ -186,7 +186,7 @@ struct aim_ctx {
   float4* specAdf = nullptr;
   // per column q' = 0..H of the filtered spectrum: 0 when the mask zeroes the whole column
   int* specA_live = nullptr;
-  double2* tw = nullptr;    // e^{-2 pi i t / P}, t < P
+  double2* tw = nullptr;    // e^{-2 pi i t / P}, t < P, then the pass tables (fft_reg.cuh)
   float2* twf = nullptr;
   float4* twdf = nullptr;
   // Gram inverse, row i: entries for columns (i + d) mod n, d = -band..band

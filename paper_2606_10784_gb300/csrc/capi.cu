@@ -7,6 +7,7 @@
 #include <new>
 
 #include "aim_internal.h"
+#include "gridtypes.cuh"
 
 namespace aim {
 
@@ -303,15 +304,21 @@ aim_status apply_op_multi(MultiLauncher& ml, int count, aim_ctx* const* ctxs, co
   return gram_inv_apply_multi(last.data(), (int)last.size(), st);
 }
 
-// e^{-2 pi i t / P}, t < P, from its FP64 (re, im) pairs: the FP64, complex64 and double-float
-// (hi, lo) copies the three grid precisions read.
+// e^{-2 pi i t / P}, t < P, from its FP64 (re, im) pairs, and the pass tables behind it
+// (fft_reg.cuh): the FP64, complex64 and double-float (hi, lo) copies the three grid precisions read.
 aim_status upload_twiddles(aim_ctx* ctx, const double* tw2, cudaStream_t st) {
-  const int P = ctx->P;
-  std::vector<double2> tw(P);
-  std::vector<float2> twf(P);
-  std::vector<float4> twdf(P);
-  for (int t = 0; t < P; ++t) {
-    const double c = tw2[2 * t], s = tw2[2 * t + 1];
+  const int P = ctx->P, count = twiddle_entries(ctx->logP);
+  std::vector<int> from(count, 0);   // entry of the plain table
+  for (int t = 0; t < P; ++t) from[t] = t;
+  for (int q = 1; q < ctx->logP; ++q)
+    for (int r = 1; r < 16 && bit_length(r) <= q; ++r)
+      for (int k = 0; k < 1 << (q - bit_length(r)); ++k)
+        from[pass_table(ctx->logP, q, r) + k] = ((r * k) << (ctx->logP - q)) & (P - 1);
+  std::vector<double2> tw(count);
+  std::vector<float2> twf(count);
+  std::vector<float4> twdf(count);
+  for (int t = 0; t < count; ++t) {
+    const double c = tw2[2 * from[t]], s = tw2[2 * from[t] + 1];
     const float ch = (float)c, sh = (float)s;
     tw[t] = double2{c, s};
     twf[t] = float2{ch, sh};
@@ -769,7 +776,8 @@ static aim_status query_context_bytes(const aim_geometry* geometry, const aim_gr
   b += committed((nact + 1) * 4) + committed(nsc * 4);           // scatter CSR
   b += committed((n + 1) * 4) + committed(nga * 4);              // gather CSR
   b += hs.nproj * (committed(nsc * 8) + committed(nga * 8));     // projection weights
-  b += committed(P * 16) + committed(P * 8) + committed(P * 16); // twiddles
+  const size_t ntw = twiddle_entries(tmp.logP);
+  b += committed(ntw * 16) + committed(ntw * 8) + committed(ntw * 16);   // twiddles and pass tables
   b += committed(hs.gram_inv.size() * 8);
   const size_t nvals = te ? 2 : 1;
   if (nnz > 0) b += committed((n + 1) * 4) + committed(nnz * 4) + nvals * (committed(nnz * 16) + committed(nnz * 8));

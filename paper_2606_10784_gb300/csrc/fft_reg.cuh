@@ -8,7 +8,7 @@
 // length-R DFT in registers and writes X[(b - b mod Ns) R + b mod Ns + r Ns].
 // Shared memory holds the exchange between passes, padded by one element every E so that the
 // stride-E writes of the first pass do not collide in banks. Twiddles come from the
-// host-computed FP64 table tw[t] = exp(-2 pi i t/P).
+// host-computed FP64 table tw[t] = exp(-2 pi i t/P), t < P, and from the pass tables behind it.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -85,12 +85,25 @@ __device__ __forceinline__ void dft_reg(T2 (&v)[R]) {
 }
 
 // Where the twiddles of a pass come from. Complex64: only the powers r = 1, 2, 4, 8 are read
-// from the table and the others are products of at most three of them (a scattered table read
-// per power costs more L1 wavefronts than the products cost FMAs, and the complex64 passes keep
-// L1 busy). Types whose complex product costs tens of FP32-pipe instructions (double-float) or
+// from the table and the others are products of at most three of them (the complex64 passes keep
+// L1 busier than the FP32 pipe). Types whose complex product costs tens of FP32-pipe instructions (double-float) or
 // runs on the slow FP64 pipe (binary64) read every factor from the table instead.
 template <typename T2> struct TwiddleFromTable { static constexpr bool value = false; };
 template <> struct TwiddleFromTable<double2> { static constexpr bool value = true; };
+
+// Pass tables: for each length 2^q of a pass's sub-transforms (q = logNs + LOGR) the rows
+// W_{2^q}^{r k}, r = 1..15, contiguous in k, so that the lanes of a warp (consecutive k) read
+// consecutive entries. Reading tw[(r k) << sh] instead touched a cache line per lane for most r: at
+// 2048 points those wavefronts were half of the complex64 column pass's L1 cycles, which were its
+// busiest unit (72 %). Row r has 2^(q - b) entries, b = bit length of r (a radix-2^b pass or
+// longer reads it); the rows of q start 2^(q+1) - 4 entries behind the P of tw.
+__host__ __device__ constexpr int bit_length(int r) { return r < 2 ? 1 : r < 4 ? 2 : r < 8 ? 3 : 4; }
+__host__ __device__ __forceinline__ int pass_table(int logP, int q, int r) {
+  const int b = bit_length(r);
+  return (1 << logP) + (2 << q) - 4 + ((b - 1) << (q - 1)) + ((r - (1 << (b - 1))) << (q - b));
+}
+// entries of tw and its pass tables (q <= logP - 1)
+__host__ __device__ __forceinline__ int twiddle_entries(int logP) { return (1 << logP) + (2 << logP) - 4; }
 
 // The twiddles W_{Ns R}^{k r}, r = 1..R-1, of butterfly position k (k != 0): app(r, w) for each.
 // All transforms a thread works on at the same butterfly position share them, so callers apply
@@ -98,21 +111,21 @@ template <> struct TwiddleFromTable<double2> { static constexpr bool value = tru
 template <int LOGR, typename T2, typename App>
 __device__ __forceinline__ void twiddles(int k, int logNs, const T2* __restrict__ tw, int logP, App app) {
   constexpr int R = 1 << LOGR;
-  const int sh = logP - logNs - LOGR;
+  const int q = logNs + LOGR;
+  auto load = [&](int r) { return ldro(&tw[pass_table(logP, q, r) + k]); };
   if constexpr (TwiddleFromTable<T2>::value) {
-    // (r k) << sh < R Ns 2^sh = P: inside the table
 #pragma unroll
-    for (int r = 1; r < R; ++r) app(r, ldro(&tw[(r * k) << sh]));
+    for (int r = 1; r < R; ++r) app(r, load(r));
   } else {
-    const T2 w1 = ldro(&tw[k << sh]);
+    const T2 w1 = load(1);
     app(1, w1);
     if constexpr (R > 2) {
-      const T2 w2 = ldro(&tw[(2 * k) << sh]);
+      const T2 w2 = load(2);
       app(2, w2);
       const T2 w3 = cmul(w2, w1);
       app(3, w3);
       if constexpr (R > 4) {
-        const T2 w4 = ldro(&tw[(4 * k) << sh]);
+        const T2 w4 = load(4);
         app(4, w4);
         const T2 w5 = cmul(w4, w1);
         app(5, w5);
@@ -121,7 +134,7 @@ __device__ __forceinline__ void twiddles(int k, int logNs, const T2* __restrict_
         const T2 w7 = cmul(w4, w3);
         app(7, w7);
         if constexpr (R > 8) {
-          const T2 w8 = ldro(&tw[(8 * k) << sh]);
+          const T2 w8 = load(8);
           app(8, w8);
           app(9, cmul(w8, w1));
           app(10, cmul(w8, w2));

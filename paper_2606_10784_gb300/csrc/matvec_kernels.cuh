@@ -889,18 +889,18 @@ struct Supports {
 
 inline int loge_of(const Schedule& sc) { return sc.elems == 8 ? 3 : 4; }
 
-// columns per column-pass CTA: the schedule's choice. By default one column as soon as it has 128
+// columns per column-pass CTA: the schedule's choice. By default one column as soon as it has 256
 // threads (64 with 16 complex64 elements per thread): CTAs of one column wait at barriers of their
 // own, and several fit an SM, which gains more than the half or quarter sectors they load cost
 // (operator N at P = 4096: double-float 1273 -> 1163 us, complex64 329 -> 277 us; complex64 at
-// P = 2048, 32 right-hand sides: 2062 -> 1925 us). Shorter columns: the fewest whole tiles of W
-// columns that give at least 128 threads.
+// P = 2048, 32 right-hand sides: 2062 -> 1925 us; but double-float there 8.26 -> 9.35 ms). Shorter
+// columns: the fewest whole tiles of W columns that give at least 128 threads.
 template <typename CT, int TPT, int LOGE>
 static int col_cols_of(const Schedule& sc, int logH, int logP) {
   constexpr int W = GridT<CT>::W, LPT = 3 - TPT;
   if (sc.col_cols > 0) return sc.col_cols;
   const int tpf = (1 << logH) >> LOGE, ntiles = (1 << logP) / W;
-  if (LPT * tpf >= (std::is_same<CT, float2>::value && LOGE == 4 ? 64 : 128)) return 1;
+  if (LPT * tpf >= (std::is_same<CT, float2>::value && LOGE == 4 ? 64 : 256)) return 1;
   int tpc = 1;
   while (tpc * LPT * W * tpf < 128 && tpc < ntiles) tpc *= 2;
   return tpc * W;
