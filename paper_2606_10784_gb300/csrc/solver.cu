@@ -446,8 +446,7 @@ __global__ void __launch_bounds__(kStepThreads) k_dcgs2_step(const double2* __re
   dfc* Hr = H + (size_t)r * hess_entries(restart);
   __shared__ double2 s[kStepJ + 1], t[kStepJ + 1];
   __shared__ dfc sdf[kStepJ + 1];
-  __shared__ dfc part[kStepWarps][kStepJ];
-  __shared__ double sh[32][3];
+  __shared__ dfc part[kStepWarps - 1][kStepJ];
   __shared__ double2 sc[3];
   // chunk sums in chunk order, and the delayed second pass of column j - 1
   for (int l = tid; l < J; l += kStepThreads) {
@@ -476,50 +475,60 @@ __global__ void __launch_bounds__(kStepThreads) k_dcgs2_step(const double2* __re
     }
   }
   __syncthreads();
-  double ss = 0.0, st_re = 0.0, st_im = 0.0;
-  for (int l = tid; l < j; l += kStepThreads) {
-    ss += s[l].x * s[l].x + s[l].y * s[l].y;
-    const double2 c = zconjmul(s[l], t[l]);
-    st_re += c.x;
-    st_im += c.y;
-  }
-  block_sum3(ss, st_re, st_im, sh);   // its barrier also covers H's column j - 1
-  if (tid == 0) {
-    const double q = s[j].x, b2 = q - ss;
-    // a non-finite value reaches the host through beta (the norm it checks); b2 <= 0 is a breakdown
-    const double beta = !active[r] ? 0.0 : !isfinite(b2) ? b2 : b2 > 0.0 ? sqrt(b2) : 0.0;
-    const double ib = beta > 0.0 ? 1.0 / beta : 0.0;
-    if (j >= 1) {
-      colout[(size_t)j * nrhs + r] = double2{beta, 0.0};
-      Hr[hess_index(j, j - 1)] = to_dfc(double2{beta, 0.0});
+  // warp 0 forms the step's scalars (FP64 sums, a root and two quotients in a chain) while the other
+  // warps form H s: lanes over its rows l, warps over its columns m >= l - 1. (With the scalars summed
+  // over all warps first, 16 warps of FP64 shuffle sums shared the SM's one FP64 pipe.) H[j][j-1] = beta,
+  // which warp 0 writes, has l = j and is not part of H s.
+  const int wid = tid >> 5, lane = tid & 31;
+  if (wid == 0) {
+    double ss = 0.0, st_re = 0.0, st_im = 0.0;
+    for (int l = lane; l < j; l += 32) {
+      ss += s[l].x * s[l].x + s[l].y * s[l].y;
+      const double2 c = zconjmul(s[l], t[l]);
+      st_re += c.x;
+      st_im += c.y;
     }
-    if (!final_step) {
-      const double2 slast = j >= 1 ? s[j - 1] : double2{0.0, 0.0};
-      double2 d = double2{(t[j].x - st_re) * ib * ib - slast.x, (t[j].y - st_im) * ib * ib - slast.y};
-      if (beta == 0.0) d = double2{0.0, 0.0};
-      const double2 kappa = double2{(slast.x + d.x) * ib, (slast.y + d.y) * ib};
-      scal[r] = sc[0] = double2{ib, 0.0};
-      scal[nrhs + r] = sc[1] = kappa;
-      scal[2 * nrhs + r] = d;
-      Hr[hess_index(j, j)] = to_dfc(d);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      st_re += __shfl_xor_sync(0xffffffffu, st_re, off);
+      st_im += __shfl_xor_sync(0xffffffffu, st_im, off);
+    }
+    if (lane == 0) {
+      const double q = s[j].x, b2 = q - ss;
+      // a non-finite value reaches the host through beta (the norm it checks); b2 <= 0 is a breakdown
+      const double beta = !active[r] ? 0.0 : !isfinite(b2) ? b2 : b2 > 0.0 ? sqrt(b2) : 0.0;
+      const double ib = beta > 0.0 ? 1.0 / beta : 0.0;
+      if (j >= 1) {
+        colout[(size_t)j * nrhs + r] = double2{beta, 0.0};
+        Hr[hess_index(j, j - 1)] = to_dfc(double2{beta, 0.0});
+      }
+      if (!final_step) {
+        const double2 slast = j >= 1 ? s[j - 1] : double2{0.0, 0.0};
+        double2 d = double2{(t[j].x - st_re) * ib * ib - slast.x, (t[j].y - st_im) * ib * ib - slast.y};
+        if (beta == 0.0) d = double2{0.0, 0.0};
+        const double2 kappa = double2{(slast.x + d.x) * ib, (slast.y + d.y) * ib};
+        scal[r] = sc[0] = double2{ib, 0.0};
+        scal[nrhs + r] = sc[1] = kappa;
+        scal[2 * nrhs + r] = d;
+        Hr[hess_index(j, j)] = to_dfc(d);
+      }
+    }
+  } else if (!final_step) {
+    for (int l = lane; l < j; l += 32) {
+      dfc acc = dfc{0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+      for (int m = wid - 1; m < j; m += kStepWarps - 1)
+        if (l <= m + 1) acc = cadd(acc, cmul(Hr[hess_index(l, m)], sdf[m]));
+      part[wid - 1][l] = acc;
     }
   }
   if (final_step) return;
-  // H s: lanes over the rows l of H, warps over its columns m >= l - 1, then the warps' sums in order.
-  // H[j][j-1] = beta, which thread 0 is writing, has l = j and is not part of it.
-  const int wid = tid >> 5, lane = tid & 31;
-  for (int l = lane; l < j; l += 32) {
-    dfc acc = dfc{0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int m = wid; m < j; m += kStepWarps)
-      if (l <= m + 1) acc = cadd(acc, cmul(Hr[hess_index(l, m)], sdf[m]));
-    part[wid][l] = acc;
-  }
   __syncthreads();
   for (int l = tid; l < j; l += kStepThreads) {
     dfc acc = part[0][l];
 #pragma unroll
-    for (int w = 1; w < kStepWarps; ++w) acc = cadd(acc, part[w][l]);
+    for (int w = 1; w < kStepWarps - 1; ++w) acc = cadd(acc, part[w][l]);
     const double2 hv = to_d2(acc.xh, acc.xl, acc.yh, acc.yl), sv = s[l], tv = t[l], kappa = sc[1];
     const double ib = sc[0].x;
     const double2 c = double2{(tv.x - hv.x) * ib, (tv.y - hv.y) * ib};
