@@ -212,6 +212,8 @@ struct aim_ctx {
   aim::MultiLauncher* multi = nullptr;   // buffers of the multi-context calls that this context leads
   // bookkeeping
   std::vector<std::pair<const void*, size_t>> smem_raised;   // dynamic shared memory limits raised so far
+  struct CoopSlots { const void* kernel; int threads; size_t smem; int slots; };
+  std::vector<CoopSlots> coop_slots;                         // resident_ctas of multi-context launches led
   std::vector<void*> allocations;
   size_t device_bytes = 0;
   double setup_seconds = 0;

@@ -1228,8 +1228,15 @@ __device__ __forceinline__ bool multi_grid_barrier(const MultiArgs& m) {
   return ok != 0;
 }
 
+// Largest CTA of the persistent kernel: 512 threads, so that five phases' code keeps 128 registers.
+// (With the 1024 threads of the single-context kernels' bound the complex64 kernel spilled 1.3 KB a
+// thread: eight contexts of P = 64..512 took 136 us a launch instead of 102.)
+template <typename CT, int TPT, int LOGE> struct MultiMax {
+  static constexpr int value = LaunchMax<CT, TPT, LOGE>::value < 512 ? LaunchMax<CT, TPT, LOGE>::value : 512;
+};
+
 template <typename CT, int TPT, int LOGE>
-__global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_grid_multi(const __grid_constant__ MultiArgs m) {
+__global__ void __launch_bounds__(MultiMax<CT, TPT, LOGE>::value) k_grid_multi(const __grid_constant__ MultiArgs m) {
   using VT = typename GridT<CT>::VT;
   extern __shared__ __align__(16) unsigned char smraw[];
   for (int phase = 0; phase < 5; ++phase) {
@@ -1279,7 +1286,7 @@ aim_status grid_pass_multi(const MultiPassSpec* passes, int count, unsigned* scr
 template <typename CT, int TPT, int LOGE>
 static int multi_cta_threads(int H) {
   constexpr int LPT = 3 - TPT, W = GridT<CT>::W;
-  constexpr int Lmax = LaunchMax<CT, TPT, LOGE>::value;
+  constexpr int Lmax = MultiMax<CT, TPT, LOGE>::value;
   int B = 32;
   while (B < std::max(2, W) * LPT * (H >> LOGE) && B < Lmax) B *= 2;
   return B;
@@ -1292,6 +1299,28 @@ static bool multi_fits(int B, int H) {
   constexpr int LPT = 3 - TPT;
   const int per_line = LPT * (H >> LOGE);
   return per_line >= 1 && B >= per_line && B / per_line <= 2 * H;
+}
+
+// CTAs of a cooperative kernel that fit the device at once; the context remembers the shapes it has
+// asked for.
+template <typename K>
+static aim_status resident_ctas(aim_ctx* ctx, K kernel, int threads, size_t smem, int* slots) {
+  const void* id = reinterpret_cast<const void*>(kernel);
+  for (const auto& s : ctx->coop_slots)
+    if (s.kernel == id && s.threads == threads && s.smem == smem) {
+      *slots = s.slots;
+      return AIM_OK;
+    }
+  int sms = 0, per_sm = 0, coop = 0;
+  AIM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  AIM_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device));
+  if (!coop) return fail(AIM_ECUDA, "device does not support cooperative launches");
+  AIM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
+  if (per_sm < 1) return fail(AIM_EINVAL, "multi-context kernel does not fit an SM");
+  *slots = sms * per_sm;
+  if (ctx->coop_slots.size() >= 64) ctx->coop_slots.clear();
+  ctx->coop_slots.push_back({id, threads, smem, *slots});
+  return AIM_OK;
 }
 
 template <typename CT, int TPT, int LOGE>
@@ -1393,16 +1422,11 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
   if (smem > kMaxDynSmem) return fail(AIM_EINVAL, "multi-context launch needs too much shared memory");
   auto kernel = k_grid_multi<CT, TPT, LOGE>;
   AIM_TRY(ensure_smem(passes[0].ctx, kernel, smem));
-  int dev = 0, sms = 0, per_sm = 0, coop = 0;
-  AIM_CUDA_TRY(cudaGetDevice(&dev));
-  AIM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  AIM_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-  if (!coop) return fail(AIM_ECUDA, "device does not support cooperative launches");
-  AIM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, B, smem));
-  if (per_sm < 1) return fail(AIM_EINVAL, "multi-context kernel does not fit an SM");
+  int slots = 0;
+  AIM_TRY(resident_ctas(passes[0].ctx, kernel, B, smem, &slots));
   long long most = 0;
   for (int ph = 0; ph < 5; ++ph) most = std::max(most, m.off[ph][count]);
-  const int grid = (int)std::max(1LL, std::min<long long>((long long)sms * per_sm, most));
+  const int grid = (int)std::max(1LL, std::min<long long>(slots, most));
   {
     // one launch: the three grid passes and the gathers of every job
     ProfScope ps(K_MULTI, st);
