@@ -37,6 +37,8 @@ template <typename CT, int TPT, int LOGE> struct LaunchMax {
   static constexpr int value = (base << (4 - LOGE)) > 1024 ? 1024 : (base << (4 - LOGE));
 };
 
+constexpr int kWideMax = 512;   // launch bound of the wide variants (wide_pass)
+
 template <typename CT> __device__ __forceinline__ CT czero();
 template <> __device__ __forceinline__ float2 czero<float2>() { return float2{0.f, 0.f}; }
 template <> __device__ __forceinline__ double2 czero<double2>() { return double2{0.0, 0.0}; }

@@ -3,11 +3,11 @@
 
 namespace aim {
 
-template aim_status launch_row_fwd<float2, 1, 4>(aim_ctx*, int, RowFwdArgs, const Schedule&, cudaStream_t);
-template aim_status launch_row_fwd<float2, 2, 4>(aim_ctx*, int, RowFwdArgs, const Schedule&, cudaStream_t);
-template aim_status launch_col_conv<float2, 1, 4>(aim_ctx*, int, ColArgs, const Schedule&, cudaStream_t);
-template aim_status launch_col_conv<float2, 2, 4>(aim_ctx*, int, ColArgs, const Schedule&, cudaStream_t);
-template aim_status launch_row_inv<float2, 1, 4>(aim_ctx*, int, RowInvArgs, const Schedule&, cudaStream_t);
-template aim_status launch_row_inv<float2, 2, 4>(aim_ctx*, int, RowInvArgs, const Schedule&, cudaStream_t);
+template aim_status launch_row_fwd<float2, 1, 4, false>(aim_ctx*, int, RowFwdArgs, const Schedule&, cudaStream_t);
+template aim_status launch_row_fwd<float2, 2, 4, false>(aim_ctx*, int, RowFwdArgs, const Schedule&, cudaStream_t);
+template aim_status launch_col_conv<float2, 1, 4, false>(aim_ctx*, int, ColArgs, const Schedule&, cudaStream_t);
+template aim_status launch_col_conv<float2, 2, 4, false>(aim_ctx*, int, ColArgs, const Schedule&, cudaStream_t);
+template aim_status launch_row_inv<float2, 1, 4, false>(aim_ctx*, int, RowInvArgs, const Schedule&, cudaStream_t);
+template aim_status launch_row_inv<float2, 2, 4, false>(aim_ctx*, int, RowInvArgs, const Schedule&, cudaStream_t);
 
 }  // namespace aim

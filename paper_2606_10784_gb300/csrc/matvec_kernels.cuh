@@ -344,8 +344,8 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
   });
 }
 
-template <typename CT, int TPT, int LOGE>
-__global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_row_fwd(RowFwdArgs a) {
+template <typename CT, int TPT, int LOGE, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_row_fwd(RowFwdArgs a) {
   grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   row_fwd_item<CT, TPT, LOGE>(a, blockIdx.x, blockIdx.y, smraw);
@@ -460,8 +460,8 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
   });
 }
 
-template <typename CT, int TPT, int LOGE>
-__global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_col_conv(ColArgs a) {
+template <typename CT, int TPT, int LOGE, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_col_conv(ColArgs a) {
   grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   // with many channels they run along x: the channels of one column tile run back to back and
@@ -651,8 +651,8 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
   }
 }
 
-template <typename CT, int TPT, int LOGE>
-__global__ void __launch_bounds__(LaunchMax<CT, TPT, LOGE>::value) k_row_inv(RowInvArgs a) {
+template <typename CT, int TPT, int LOGE, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_row_inv(RowInvArgs a) {
   grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   row_inv_item<CT, TPT, LOGE>(a, blockIdx.x, blockIdx.y, smraw);
@@ -948,7 +948,7 @@ static int rows_per_cta(const aim_ctx* ctx, const Schedule& sc) {
   return rpc;
 }
 
-template <typename CT, int TPT, int LOGE>
+template <typename CT, int TPT, int LOGE, bool WIDE>
 aim_status launch_row_fwd(aim_ctx* ctx, int channels, RowFwdArgs fa, const Schedule& sc, cudaStream_t st) {
   constexpr int LPT = 3 - TPT;
   const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
@@ -956,12 +956,12 @@ aim_status launch_row_fwd(aim_ctx* ctx, int channels, RowFwdArgs fa, const Sched
   fa.rows_per_cta = rpc;
   const size_t smem =
       2 * (size_t)rpc * padded_len<LOGE>(ctx->H) * sizeof(CT) + (fa.sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
-  AIM_TRY(ensure_smem(ctx, k_row_fwd<CT, TPT, LOGE>, smem));
+  AIM_TRY(ensure_smem(ctx, k_row_fwd<CT, TPT, LOGE, WIDE>, smem));
   ProfScope ps(K_ROW_FWD, st);
-  return launch_chained(k_row_fwd<CT, TPT, LOGE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, fa);
+  return launch_chained(k_row_fwd<CT, TPT, LOGE, WIDE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, fa);
 }
 
-template <typename CT, int TPT, int LOGE>
+template <typename CT, int TPT, int LOGE, bool WIDE>
 aim_status launch_col_conv(aim_ctx* ctx, int channels, ColArgs ca, const Schedule& sc, cudaStream_t st) {
   constexpr int LPT = 3 - TPT;
   constexpr int kChanX = 8;   // channels from which the column-pass grid runs channels along x
@@ -970,14 +970,14 @@ aim_status launch_col_conv(aim_ctx* ctx, int channels, ColArgs ca, const Schedul
   while ((1 << ca.log_cols) < cols) ++ca.log_cols;
   if (ctx->P / cols > 65535) return fail(AIM_EINVAL, "too many column tiles for one column-pass grid");
   const size_t smem = 2 * (size_t)cols * padded_len<LOGE>(ctx->H) * sizeof(CT);
-  AIM_TRY(ensure_smem(ctx, k_col_conv<CT, TPT, LOGE>, smem));
+  AIM_TRY(ensure_smem(ctx, k_col_conv<CT, TPT, LOGE, WIDE>, smem));
   ca.chan_x = channels >= kChanX;
   const dim3 grid = ca.chan_x ? dim3(channels, ctx->P / cols) : dim3(ctx->P / cols, channels);
   ProfScope ps(K_COL_CONV, st);
-  return launch_chained(k_col_conv<CT, TPT, LOGE>, grid, cols * LPT * tpf, smem, st, ca);
+  return launch_chained(k_col_conv<CT, TPT, LOGE, WIDE>, grid, cols * LPT * tpf, smem, st, ca);
 }
 
-template <typename CT, int TPT, int LOGE>
+template <typename CT, int TPT, int LOGE, bool WIDE>
 aim_status launch_row_inv(aim_ctx* ctx, int channels, RowInvArgs ia, const Schedule& sc, cudaStream_t st) {
   constexpr int LPT = 3 - TPT;
   const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
@@ -985,9 +985,9 @@ aim_status launch_row_inv(aim_ctx* ctx, int channels, RowInvArgs ia, const Sched
   ia.rows_per_cta = rpc;
   const size_t smem =
       2 * (size_t)rpc * padded_len<LOGE>(ctx->H) * sizeof(CT) + (ia.sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
-  AIM_TRY(ensure_smem(ctx, k_row_inv<CT, TPT, LOGE>, smem));
+  AIM_TRY(ensure_smem(ctx, k_row_inv<CT, TPT, LOGE, WIDE>, smem));
   ProfScope ps(K_ROW_INV, st);
-  return launch_chained(k_row_inv<CT, TPT, LOGE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, ia);
+  return launch_chained(k_row_inv<CT, TPT, LOGE, WIDE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, ia);
 }
 
 // Transforms per thread of a pass of `lines` lines whose two-transform form has tpf threads a line.
@@ -1004,6 +1004,19 @@ static int pass_tpt(const aim_ctx* ctx, const Schedule& sc, bool rows, long long
   const long long threads = lines * (ctx->H >> loge_of(sc));
   const long long most = !rows ? 32 << 10 : std::is_same<CT, float2>::value ? 64 << 10 : 128 << 10;
   return threads <= most ? 1 : 2;
+}
+
+// Whether a double-float pass with one transform of 8 elements per thread runs as its wide variant.
+// The plain kernels are bounded to 1024 threads, 64 registers, and spill; bounded to 512 threads they
+// take 102 (row passes) or 128 registers and none, but half as many threads fit an SM. So the wide ones
+// run launches that fit the GPU at once: 640 and 512 threads on each of 152 SMs. (N = 733 with three
+// right-hand sides 151 -> 132 us, N = 64 62 -> 57 us; a grid product of 157 thousand row-pass threads
+// 108 -> 116 us, so not there.)
+inline bool wide_pass(const aim_ctx* ctx, const Schedule& sc, bool rows, long long lines) {
+  const int per_line = ctx->H >> 2;   // two threads for every 8 elements
+  const long long threads = lines * per_line;
+  if (rows) return rows_per_cta<dfc, 1, 3>(ctx, sc) * per_line <= kWideMax && threads <= 152 * 640;
+  return col_cols_of<dfc, 1, 3>(sc, ctx->logH, ctx->logP) * per_line <= kWideMax && threads <= 152 * 512;
 }
 
 template <typename CT>
@@ -1042,9 +1055,16 @@ static aim_status launch_three_passes(aim_ctx* ctx, int channels, bool filtered,
   const long long rows = (long long)channels * ctx->nrows, cols = (long long)channels * std::min(ctx->P, 2 * qcut + 1);
   auto run = [&](auto tpt, auto loge, int pass) -> aim_status {
     constexpr int TPT = decltype(tpt)::value, LOGE = decltype(loge)::value;
-    if (pass == 0) return launch_row_fwd<CT, TPT, LOGE>(ctx, channels, fa, sc, st);
-    if (pass == 1) return launch_col_conv<CT, TPT, LOGE>(ctx, channels, ca, sc, st);
-    return launch_row_inv<CT, TPT, LOGE>(ctx, channels, ia, sc, st);
+    if constexpr (std::is_same<CT, dfc>::value && TPT == 1 && LOGE == 3) {
+      if (wide_pass(ctx, sc, pass != 1, pass != 1 ? rows : cols)) {
+        if (pass == 0) return launch_row_fwd<CT, TPT, LOGE, true>(ctx, channels, fa, sc, st);
+        if (pass == 1) return launch_col_conv<CT, TPT, LOGE, true>(ctx, channels, ca, sc, st);
+        return launch_row_inv<CT, TPT, LOGE, true>(ctx, channels, ia, sc, st);
+      }
+    }
+    if (pass == 0) return launch_row_fwd<CT, TPT, LOGE, false>(ctx, channels, fa, sc, st);
+    if (pass == 1) return launch_col_conv<CT, TPT, LOGE, false>(ctx, channels, ca, sc, st);
+    return launch_row_inv<CT, TPT, LOGE, false>(ctx, channels, ia, sc, st);
   };
   using I1 = std::integral_constant<int, 1>;
   using I2 = std::integral_constant<int, 2>;
