@@ -120,8 +120,13 @@ __global__ void k_sample_kernel(double2* samp, int H, double eps, double k) {
     samp[t] = double2{0.0, 0.0};     // self term set to zero (Sec. III-C)
     return;
   }
+  // symmetric in i and j: each value is computed once and stored twice (Bessel functions run at the
+  // FP64 rate; whole warps leave where j < i)
+  if (j < i) return;
   const double r = eps * sqrt((double)i * i + (double)j * j);
-  samp[t] = green(k, r);
+  const double2 g = green(k, r);
+  samp[t] = g;
+  samp[(long long)j * (H + 1) + i] = g;
 }
 
 // In-place transform of the even-symmetric P x P array held as its (H+1) x (H+1) quarter:
@@ -384,6 +389,33 @@ __device__ __forceinline__ double2 aim_pair_sum(const double2* samp, int H, cons
   return warp_sum(acc);
 }
 
+// The same for NP weight sets on one pair of lists: each kernel sample is read once for all of them.
+template <int NP>
+__device__ __forceinline__ void aim_pair_sums(const double2* samp, int H, const int* act_ix, const int* act_iy,
+                                              const int* ia, const int* ib, const double* const (&wi)[NP],
+                                              const double* const (&wj)[NP], int ni, int nj, int lane, double2 (&A)[NP]) {
+  double2 acc[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) acc[q] = double2{0.0, 0.0};
+  for (int a = lane; a < ni; a += 32) {
+    const int xa = act_ix[ia[a]], ya = act_iy[ia[a]];
+    double2 inner[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) inner[q] = double2{0.0, 0.0};
+#pragma unroll 4
+    for (int b = 0; b < nj; ++b) {
+      const int dx = abs(xa - act_ix[ib[b]]), dy = abs(ya - act_iy[ib[b]]);
+      const double2 c = samp[(size_t)dy * (H + 1) + dx];
+#pragma unroll
+      for (int q = 0; q < NP; ++q) inner[q] = cmadd(inner[q], wj[q][b], c);
+    }
+#pragma unroll
+    for (int q = 0; q < NP; ++q) acc[q] = cmadd(acc[q], wi[q][a], inner[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < NP; ++q) A[q] = warp_sum(acc[q]);
+}
+
 struct TENearArgs {
   const double2* nodes;
   int n;
@@ -421,35 +453,44 @@ __global__ void k_te_near_entries(TENearArgs a) {
   double2 A[4];
   const int i0 = a.ga_ptr[i], ni = a.ga_ptr[i + 1] - i0;
   const int j0 = a.ga_ptr[j], nj = a.ga_ptr[j + 1] - j0;
+  const double* wi[4];
+  const double* wj[4];
 #pragma unroll
-  for (int pj = 0; pj < 4; ++pj)
-    A[pj] = aim_pair_sum(a.samp, a.H, a.act_ix, a.act_iy, a.ga_act + i0, a.ga_w[pj] + i0, ni,
-                         a.ga_act + j0, a.ga_w[pj] + j0, nj, lane);
-  if (lane != 0) return;
-  // exact entries from the four segment pairs (e, a) x (f, b)
-  const int es[4] = {i, i, (i + n - 1) % n, (i + n - 1) % n};
-  const int fs[4] = {j, (j + n - 1) % n, j, (j + n - 1) % n};
-  const int as[4] = {0, 0, 1, 1}, bs[4] = {0, 1, 0, 1};
+  for (int pj = 0; pj < 4; ++pj) {
+    wi[pj] = a.ga_w[pj] + i0;
+    wj[pj] = a.ga_w[pj] + j0;
+  }
+  aim_pair_sums<4>(a.samp, a.H, a.act_ix, a.act_iy, a.ga_act + i0, a.ga_act + j0, wi, wj, ni, nj, lane, A);
+  // exact entries from the four segment pairs (e, a) x (f, b), one per lane: with all four in one lane
+  // their quotients and roots, FP64 sequences of a whole warp's cost, were most of this kernel
+  const int c = lane & 3;
   double2 S{0, 0}, N{0, 0};
-  for (int c = 0; c < 4; ++c) {
+  {
+    const int e = c < 2 ? i : (i + n - 1) % n, f = (c & 1) ? (j + n - 1) % n : j;
+    const int pa = c >> 1, pb = c & 1;
     // a pair stored the other way round has its two hats exchanged
     const int id = a.pair_seg_idx[(size_t)wid * 4 + c];
     const double2* I = a.I + (size_t)(id < 0 ? ~id : id) * 4;
-    const int e = es[c], f = fs[c];
     const double2 ve0 = a.nodes[e], ve1 = a.nodes[(e + 1) % n];
     const double2 vf0 = a.nodes[f], vf1 = a.nodes[(f + 1) % n];
     const double dex = ve1.x - ve0.x, dey = ve1.y - ve0.y, dfx = vf1.x - vf0.x, dfy = vf1.y - vf0.y;
     const double he = hypot(dex, dey), hf = hypot(dfx, dfy);
     // n = (t_y, -t_x): n_e . n_f = t_e . t_f
     const double nn = (dex * dfx + dey * dfy) / (he * hf);
-    const double2 Iab = I[id < 0 ? bs[c] * 2 + as[c] : as[c] * 2 + bs[c]];
+    const double2 Iab = I[id < 0 ? pb * 2 + pa : pa * 2 + pb];
     const double2 J = double2{I[0].x + I[1].x + I[2].x + I[3].x, I[0].y + I[1].y + I[2].y + I[3].y};
-    const double dd = ((as[c] ? 1.0 : -1.0) / he) * ((bs[c] ? 1.0 : -1.0) / hf);
-    S.x += Iab.x;
-    S.y += Iab.y;
-    N.x += dd * J.x - a.k * a.k * nn * Iab.x;
-    N.y += dd * J.y - a.k * a.k * nn * Iab.y;
+    const double dd = ((pa ? 1.0 : -1.0) / he) * ((pb ? 1.0 : -1.0) / hf);
+    const double k2nn = a.k * a.k * nn;
+    const double2 own = double2{fma(dd, J.x, -(k2nn * Iab.x)), fma(dd, J.y, -(k2nn * Iab.y))};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {   // in the pairs' order
+      S.x += __shfl_sync(0xffffffffu, Iab.x, q);
+      S.y += __shfl_sync(0xffffffffu, Iab.y, q);
+      N.x += __shfl_sync(0xffffffffu, own.x, q);
+      N.y += __shfl_sync(0xffffffffu, own.y, q);
+    }
   }
+  if (lane != 0) return;
   const double k2 = a.k * a.k;
   const double2 cs = double2{S.x - A[0].x, S.y - A[0].y};
   const double2 cn = double2{N.x - (A[1].x - k2 * (A[2].x + A[3].x)), N.y - (A[1].y - k2 * (A[2].y + A[3].y))};
