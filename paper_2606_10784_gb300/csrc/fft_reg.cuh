@@ -176,6 +176,35 @@ struct PlainLoad {
   __device__ __forceinline__ T2 operator()(int f, int i) const { return sm[fb[f] + padi<LOGE>(i)]; }
 };
 
+// The two halves of a pass over ONE transform, for callers that run several transforms through the
+// same code one after the other: a thread's butterflies read (`load(i)`), twiddled and transformed, and,
+// behind a barrier of the caller's, written back.
+template <int LOGR, bool INV, int LOGE, typename T2, typename Load>
+__device__ __forceinline__ void pass_compute(T2 (&v)[1][(1 << LOGE) >> LOGR][1 << LOGR], int j, int tpf, int logH,
+                                             int logNs, const T2* __restrict__ tw, int logP, Load load) {
+  constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
+  const int lognb = logH - LOGR, nsm = (1 << logNs) - 1;
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    const int b = j + t * tpf;
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[0][t][r] = load(b + (r << lognb));
+    bfly_shared<LOGR, INV>(v, t, b & nsm, logNs, tw, logP);
+  }
+}
+template <int LOGR, int LOGE, typename T2>
+__device__ __forceinline__ void pass_store(const T2 (&v)[1][(1 << LOGE) >> LOGR][1 << LOGR], T2* __restrict__ buf, int j,
+                                           int tpf, int logNs) {
+  constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
+  const int nsm = (1 << logNs) - 1;
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    const int b = j + t * tpf, k = b & nsm, base = ((b - k) << LOGR) + k;
+#pragma unroll
+    for (int r = 0; r < R; ++r) buf[padi<LOGE>(base + (r << logNs))] = v[0][t][r];
+  }
+}
+
 // One pass over NF transforms owned by this thread group, shared memory in and out.
 // Each thread works on butterflies b = j + t*tpf (t < E/R) of each of its transforms, whose
 // padded bases in shared memory are fb[f]. `load(f, i)` reads input i of transform f. Barrier

@@ -460,6 +460,133 @@ __device__ __forceinline__ void col_conv_item(const ColArgs& a, int ctile, int c
   });
 }
 
+// The middle of the column pass of one half: last forward pass, product with the spectrum, first
+// inverse pass of the same radix (conv_mid_pass, in two parts around a barrier).
+template <int LOGR, int LOGE, typename T2, typename Mul>
+__device__ __forceinline__ void col_mid_half(T2* buf, int j, int tpf, int logH, const T2* tw, int logP, Mul mul) {
+  constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
+  const int lognb = logH - LOGR;
+  T2 v[1][NB][R];
+  pass_compute<LOGR, false, LOGE>(v, j, tpf, logH, lognb, tw, logP, [&](int i) { return buf[padi<LOGE>(i)]; });
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    const int b = j + t * tpf;
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[0][t][r] = mul(b + (r << lognb), v[0][t][r]);
+    dft_reg<R, true>(v[0][t]);
+  }
+  __syncthreads();
+  pass_store<LOGR, LOGE>(v, buf, j, tpf, 0);
+}
+
+// The column pass with both halves of a column in one thread group, one half after the other through
+// the same code: a thread holds one transform's E elements instead of two and the code of a pass is
+// there once. The odd half's input waits in its own buffer, in the slots its thread reads next, and the
+// even half's result in the slots its thread has just read, so neither needs a barrier; those two extra
+// trips through shared memory are what it costs. The values and their order are those of col_conv_item.
+template <typename CT, int LOGE>
+__device__ __forceinline__ void col_conv_halves(const ColArgs& a, int ctile, int c, unsigned char* smraw) {
+  using T2 = CT;
+  constexpr int W = GridT<CT>::W, E = 1 << LOGE;
+  T2* sm = reinterpret_cast<T2*>(smraw);
+  const int H = 1 << a.logH, P = 1 << a.logP, tpf = H >> LOGE, HS = padded_len<LOGE>(H);
+  const int cw = min(1 << a.log_cols, W);               // columns side by side in the lanes
+  const int per_grp = cw * tpf;
+  const int g = threadIdx.x / per_grp, rem = threadIdx.x - g * per_grp;
+  const int wl = rem & (cw - 1), j = rem / cw;
+  const int colc = g * cw + wl;                         // column within the CTA
+  const int qcol = (ctile << a.log_cols) + colc;        // column of the grid
+  const int w = qcol & (W - 1), tile = qcol / W;
+  {
+    const int qa = ctile << a.log_cols, qb = qa + (1 << a.log_cols) - 1;
+    if (min(min(qa, P - qa), min(qb, P - qb)) > a.qcut) {   // as in col_conv_item
+      grid_dependency_wait();
+      return;
+    }
+  }
+  const T2* tw = static_cast<const T2*>(a.tw);
+  T2* buf0 = sm + 2 * colc * HS;
+  T2* blk = static_cast<T2*>(a.inter) + (size_t)c * P * a.nrows + (size_t)tile * a.nrows * W;
+  const int row_hi = a.row_lo + a.nrows - 1, lognb = a.logH - LOGE;
+  grid_dependency_wait();
+  // pass 0 (radix E, Ns = 1) of a and of a w^n
+#pragma unroll 1
+  for (int f = 0; f < 2; ++f) {
+    T2* buf = buf0 + f * HS;
+    T2 v[1][1][E];
+    if (f == 0) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) {
+        const int nn = j + (r << lognb);
+        v[0][0][r] = (nn >= a.row_lo && nn <= row_hi) ? blk[(nn - a.row_lo) * W + w] : czero<T2>();
+      }
+#pragma unroll
+      for (int r = 0; r < E; ++r) {
+        const int nn = j + (r << lognb);
+        buf0[HS + padi<LOGE>(nn)] = cmul(v[0][0][r], ldro(&tw[nn]));
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[0][0][r] = buf[padi<LOGE>(j + (r << lognb))];
+    }
+    dft_reg<E, false>(v[0][0]);
+    if (f == 1) __syncthreads();
+    pass_store<LOGE, LOGE>(v, buf, j, tpf, 0);
+  }
+  const int np = fft_npass<LOGE>(a.logH), lr0 = fft_logr<LOGE>(np - 1, a.logH);
+  // a pass of half f reads, waits for the others' reads and writes; the next pass of the same half comes
+  // after the other half's wait
+  auto radix_e = [&](auto inv, int logNs) {
+#pragma unroll 1
+    for (int f = 0; f < 2; ++f) {
+      T2* buf = buf0 + f * HS;
+      T2 v[1][1][E];
+      pass_compute<LOGE, decltype(inv)::value, LOGE>(v, j, tpf, a.logH, logNs, tw, a.logP, [&](int i) { return buf[padi<LOGE>(i)]; });
+      __syncthreads();
+      pass_store<LOGE, LOGE>(v, buf, j, tpf, logNs);
+    }
+  };
+  for (int p = 1; p < np - 1; ++p) radix_e(std::false_type{}, LOGE * p);
+  {
+    const T2* col = static_cast<const T2*>(a.spec) + (size_t)min(qcol, P - qcol) * (H + 1);
+#pragma unroll 1
+    for (int f = 0; f < 2; ++f) {
+      T2* buf = buf0 + f * HS;
+      const T2* cf = f ? col + (H >> 1) + 1 : col;
+      auto mul = [&](int k, T2 v) { return cmul(v, ldro(&cf[min(k, H - f - k)])); };
+      if (lr0 == LOGE) {
+        col_mid_half<LOGE, LOGE>(buf, j, tpf, a.logH, tw, a.logP, mul);
+      } else {
+        switch (lr0) {
+          case 3: if constexpr (LOGE > 3) col_mid_half<3, LOGE>(buf, j, tpf, a.logH, tw, a.logP, mul); break;
+          case 2: col_mid_half<2, LOGE>(buf, j, tpf, a.logH, tw, a.logP, mul); break;
+          default: col_mid_half<1, LOGE>(buf, j, tpf, a.logH, tw, a.logP, mul); break;
+        }
+      }
+    }
+  }
+  for (int p = 1; p < np - 1; ++p) radix_e(std::true_type{}, lr0 + LOGE * (p - 1));
+  // last inverse pass (radix E, Ns = H/E: outputs where the inputs were), y[n] = A[n] + conj(w^n) B[n]
+#pragma unroll 1
+  for (int f = 0; f < 2; ++f) {
+    T2* buf = buf0 + f * HS;
+    T2 v[1][1][E];
+    if (f == 1) __syncthreads();   // the odd half's last stores
+    pass_compute<LOGE, true, LOGE>(v, j, tpf, a.logH, lognb, tw, a.logP, [&](int i) { return buf[padi<LOGE>(i)]; });
+    if (f == 0) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) buf[padi<LOGE>(j + (r << lognb))] = v[0][0][r];
+    } else {
+#pragma unroll
+      for (int r = 0; r < E; ++r) {
+        const int nn = j + (r << lognb);
+        const T2 y = cadd(buf0[padi<LOGE>(nn)], cmulc(v[0][0][r], ldro(&tw[nn])));
+        if (nn >= a.row_lo && nn <= row_hi) blk[(nn - a.row_lo) * W + w] = y;
+      }
+    }
+  }
+}
+
 template <typename CT, int TPT, int LOGE, bool WIDE = false>
 __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_col_conv(ColArgs a) {
   grid_trigger_dependents();
@@ -467,7 +594,17 @@ __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::va
   // with many channels they run along x: the channels of one column tile run back to back and
   // share its spectrum column through L2 (64 right-hand sides: 2.82 -> 2.67 ms per launch);
   // with few, column tiles run along x (no gain measured for 3 channels)
-  col_conv_item<CT, TPT, LOGE>(a, a.chan_x ? blockIdx.y : blockIdx.x, a.chan_x ? blockIdx.x : blockIdx.y, smraw);
+  const int tile = a.chan_x ? blockIdx.y : blockIdx.x, channel = a.chan_x ? blockIdx.x : blockIdx.y;
+  if constexpr (std::is_same<CT, dfc>::value && TPT == 2 && LOGE == 3) {
+    // one half after the other where columns are short (double-float, operator N: P = 256 with seven
+    // right-hand sides 34.5 -> 31.1 us, P = 1024 70 -> 65 us); both at once from P = 2048 on (285 against
+    // 291 us, P = 4096 1113 against 1155 us) and in complex64 (P = 4096 263 against 288 us)
+    if (a.logP <= 10) {
+      col_conv_halves<CT, LOGE>(a, tile, channel, smraw);
+      return;
+    }
+  }
+  col_conv_item<CT, TPT, LOGE>(a, tile, channel, smraw);
 }
 
 // ------------------------------------------------------------------------------------
