@@ -787,7 +787,10 @@ static aim_status query_context_bytes(const aim_geometry* geometry, const aim_gr
   if (nnz > 0) {
     t += committed(nact * 4);
     if (te) {
-      const size_t npairs = hs.seg_e.size();
+      // a bound: every pair in both orders. The setup keeps each pair once and so commits less, but limits
+      // that users have set by this figure keep admitting and refusing the same problems.
+      size_t npairs = 2 * hs.seg_e.size();
+      for (size_t p = 0; p < hs.seg_e.size(); ++p) npairs -= hs.seg_e[p] == hs.seg_f[p];
       t += 2 * committed(npairs * 4) + committed(nnz * 4 * 4) + committed(npairs * 4 * 16);
     } else {
       t += committed((n + 1) * 4) + committed(hs.sr_act.size() * 4) + committed(hs.sr_w.size() * 8);
