@@ -61,7 +61,7 @@ E2E_STEPS_MAX = 5
 # ncu capture of the current kernel and default schedule at the single-solve size; the capture and
 # its command are in profiles/col_conv_*_single_solve_n10000.md. None where no capture of the
 # current kernel exists.
-COL_CONV_TRAFFIC = {"fp64": 533945856, "mixed": 201229440, "native": None}
+COL_CONV_TRAFFIC = {"fp64": 492032896, "mixed": 188581120, "native": None}
 
 
 def parse():
@@ -187,9 +187,9 @@ def col_conv_algorithmic(wl, info, precision, channels, filtered=False):
     """Algorithmic bytes and flops of one column-pass launch.
 
     Bytes (the pass model of the method): each channel's m_rows x P intermediate read once and
-    written once over the live columns (zeros written on the others), plus the stored
-    (P/2+1)^2 spectrum read once per launch (all channels share it); b = 8 bytes per complex in
-    mixed precision, 16 otherwise.
+    written once over the live columns (the others are neither read nor written), plus the live
+    columns of the stored (P/2+1)^2 spectrum read once per launch (all channels share it); b = 8
+    bytes per complex in mixed precision, 16 otherwise.
     Flops (the method's own count, the FFT convention 5 L log2 L per length-L transform): per live
     column and channel the pruned forward DFT of the m_rows nonzeros and the inverse DFT keeping
     m_rows outputs, each as two length-H transforms (4 x 5 H log2 H), plus the spectral product
@@ -200,7 +200,7 @@ def col_conv_algorithmic(wl, info, precision, channels, filtered=False):
     rows = info["row_hi"] - info["row_lo"] + 1
     b = 8 if precision == "mixed" else 16
     live, live_half = live_columns(wl, info, filtered)
-    bytes_ = channels * (2 * rows * live * b + rows * (P - live) * b) + live_half * (H + 1) * b
+    bytes_ = channels * 2 * rows * live * b + live_half * (H + 1) * b
     flops = channels * live * (4 * 5 * H * math.log2(H) + 6 * P)
     return bytes_, flops
 

@@ -233,9 +233,12 @@ aim_status aim_reserve(aim_ctx* ctx, int nrhs, int precision);
  * paper). transforms_per_thread: 1 puts the even- and odd-half transforms of a line in
  * adjacent lanes, 2 puts both in one thread (native FP64 allows 2 only). row_threads: the
  * least threads of a row-pass CTA (32..1024; rows are added to a CTA until it has that many).
- * col_cols: columns of one column-pass CTA, a power of two, 0 for the default (the fewest
- * whole 32-byte column tiles that give 128 threads). elems_per_thread: 16 (radix-16 passes)
- * or 8 (radix-8 passes, half the registers per thread; not for native FP64); 0 means 16.
+ * col_cols: columns of one column-pass CTA, a power of two, 0 for the default (by size: the
+ * fewest whole 32-byte column tiles that give 128 threads, or one column where a CTA of one
+ * fills the GPU better). elems_per_thread: 16 (radix-16 passes) or 8 (radix-8 passes, half the
+ * registers per thread; not for native FP64); 0 means 16. A context starts with {2, 128, 0, E},
+ * E = 8 in FP64 and, up to a transform length of 1024, in mixed precision, else 16; under that
+ * schedule a launch too small for the GPU takes one transform per thread.
  * Results are identical under every schedule with the same elems_per_thread: the arithmetic
  * and its order do not depend on the rest; the two pass geometries differ by rounding. */
 typedef struct {
@@ -266,8 +269,8 @@ aim_status aim_rhs_planewave(aim_ctx* ctx, int nrhs, const double* angles, void*
 
 /* y = A x for nrhs vectors (complex128 in and out, n*nrhs each; host or device; x and y
  * must not overlap). A is selected by `op` (see aim_op); precision selects the grid
- * arithmetic. The work is the pipeline of Eq. 8 / Eq. 10: sparse anterpolation fused
- * into a forward row FFT, a column FFT fused with the spectral product and the inverse
+ * arithmetic. The work is the pipeline of Eq. 8 / Eq. 10: a sparse anterpolation, a
+ * forward row FFT, a column FFT fused with the spectral product and the inverse
  * column FFT, an inverse row FFT with restriction, and the interpolation gather fused
  * with the near-field SpMV. Errors: AIM_EINVAL, AIM_ESTATE, AIM_ENOMEM, AIM_ECUDA. */
 aim_status aim_matvec(aim_ctx* ctx, aim_op op, int nrhs, const void* x, void* y,
@@ -284,10 +287,12 @@ aim_status aim_matvec(aim_ctx* ctx, aim_op op, int nrhs, const void* x, void* y,
  * y: host arrays of `count` entries; x[i], y[i]: device pointers to nrhs[i] vectors of context i;
  * a context appears at most once. All contexts must be current on this device and share the pass
  * geometry (transforms and elements per thread) of their schedule in `precision` (otherwise
- * AIM_EINVAL). One launch serves contexts whose transforms fit one CTA size (a CTA takes
+ * AIM_EINVAL); the schedules that contexts start with go together, whatever their sizes. One
+ * launch serves contexts of one elems_per_thread whose transforms fit one CTA size (a CTA takes
  * max(2, 32-byte tile) lines of the longest transform and correspondingly more lines of shorter
  * ones, at most a context's P); a stage whose contexts span more than that (for example P = 64
- * beside P = 2048) is split into the fewest such launches. Synchronises `stream`. */
+ * beside P = 2048) is split into the fewest such launches. The first context of the list keeps the
+ * launch's barrier words (32 bytes of device memory) until it is destroyed. Synchronises `stream`. */
 aim_status aim_matvec_multi(int count, aim_ctx* const* ctxs, const aim_op* ops, const int* nrhs,
                             const void* const* x, void* const* y, int precision, void* stream);
 

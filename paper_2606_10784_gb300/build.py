@@ -16,9 +16,10 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libaimgb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["matvec_dfc.cu", "matvec_dfc_e16.cu", "matvec_dfc_wide.cu", "matvec_dfc_multi.cu", "matvec_dfc_multi_e16.cu", "matvec_f32.cu",
-           "matvec_f32_e16.cu", "matvec_f32_multi.cu", "matvec_f32_multi_e16.cu", "matvec_f64.cu", "capi.cu",
-           "setup_host.cpp", "setup_kernels.cu", "matvec_common.cu", "solver.cu", "prof.cu", "noalloc.cu", "lanczos.cu", "batcher.cu", "setup_cache.cu",
+SOURCES = ["matvec_dfc.cu", "matvec_dfc_e16.cu", "matvec_dfc_wide.cu", "matvec_dfc_multi.cu",
+           "matvec_dfc_multi_e16.cu", "matvec_f32.cu", "matvec_f32_e16.cu", "matvec_f32_multi.cu",
+           "matvec_f32_multi_e16.cu", "matvec_f64.cu", "capi.cu", "setup_host.cpp", "setup_kernels.cu",
+           "matvec_common.cu", "solver.cu", "prof.cu", "noalloc.cu", "lanczos.cu", "batcher.cu", "setup_cache.cu",
            "dft_stage.cu"]
 
 

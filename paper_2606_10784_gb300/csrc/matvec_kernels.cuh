@@ -4,9 +4,10 @@
 //     y = P_t^T [ F^-1( F(c) .* F(b) ) ]_restr ,   b = zero-padded P_s x
 // runs as an anterpolation, three grid passes and a gather:
 //   k_anterpolate  u = P_s x at the active grid points (deterministic, no atomics).
-//   k_row_fwd   the forward P-point row DFT of u. The row has nonzeros
-//               only in its first m <= P/2 entries, so X[2k] = DFT_H(a)[k] and
-//               X[2k+1] = DFT_H(a w^n)[k], H = P/2, w = exp(-2 pi i/P).
+//   k_row_fwd   the forward P-point row DFT of u. The row has nonzeros only in its first
+//               m <= P/2 entries, so X[2k] = DFT_H(a)[k] and X[2k+1] = DFT_H(a w^n)[k],
+//               H = P/2, w = exp(-2 pi i/P). Rows of few active points: only the later
+//               passes are dense (row_fwd_sparse).
 //   k_col_conv  per column q: the same pruned forward DFT along the rows, the product with
 //               the stored spectrum column F(c)[., q] (even symmetric, so only
 //               (P/2+1)^2 values are stored), and the inverse DFT keeping rows < P/2 only:
@@ -17,14 +18,14 @@
 //   k_gather    y_i = sum over projections of coef * (P_t^T v)_i plus the near-field row
 //               (C x)_i, eight lanes per unknown, deterministic.
 // Each length-H transform runs as register-resident radix-E passes (fft_reg.cuh, E = 16 or 8
-// elements per thread, a schedule choice): the first
-// pass reads its operands straight from global memory (column and inverse row passes) and the
-// last pass writes straight to global memory (forward row and column passes; the inverse row
+// elements per thread, a schedule choice): the first pass reads its operands straight from
+// global memory (column and inverse row passes) and the last pass writes straight to global memory (forward row and column passes; the inverse row
 // pass keeps its last pass in shared memory for the restriction), so shared memory carries only
-// the exchanges between passes. A thread owns TPT transforms: with TPT = 2 the even- and odd-half transforms
-// of a line sit in the same thread; with TPT = 1 they sit in adjacent lanes and recombine
-// through a lane shuffle (half the registers per thread, twice the threads). Which one is
-// faster depends on the element type; the autotuner measures both.
+// the exchanges between passes. A thread owns TPT transforms: with TPT = 2 the even- and odd-half
+// transforms of a line sit in the same thread; with TPT = 1 they sit in adjacent lanes and
+// recombine through a lane shuffle (half the registers per thread, twice the threads). Which one
+// is faster depends on the element type and on how much of the GPU a launch fills (pass_tpt); the
+// autotuner measures both.
 // The intermediate m x P grid of a channel is stored as column tiles of W entries
 // (W * sizeof(complex) = 32 bytes) so that the column pass reads contiguous blocks and the
 // row passes touch whole 32-byte sectors. Only grid rows that hold active points are stored.

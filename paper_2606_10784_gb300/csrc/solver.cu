@@ -428,9 +428,10 @@ __global__ void k_dcgs2_coeffs(const double2* __restrict__ D0, const double2* __
 
 // The coefficients of one step in one launch, for the first kStepJ steps of a cycle: one CTA per
 // right-hand side does what k_dcgs2_finish, k_dcgs2_hs_scal and k_dcgs2_coeffs do in three launches
-// (H s is then at most 8 thousand products, a microsecond for one SM, and a launch costs two to three). With the updates in one launch and the
-// columns written to host memory by the kernels, 60 steps of an N = 600 system with 4 right-hand sides
-// went from 50.8 to 33.4 us a step, 400 steps at N = 10000 from 86 to 62 us.
+// (H s is then at most 8 thousand products, a microsecond for one SM, and a launch costs two to three).
+// One warp forms the scalars while the others form H s. With the updates in one launch and the columns
+// written to host memory by the kernels, 60 steps of an N = 600 system with 4 right-hand sides went from
+// 50.8 to 24.7 us a step, 400 steps at N = 10000 from 86 to 60 us.
 constexpr int kStepJ = 128, kStepThreads = 512, kStepWarps = kStepThreads / 32;
 
 __global__ void __launch_bounds__(kStepThreads) k_dcgs2_step(const double2* __restrict__ part0,
