@@ -211,7 +211,7 @@ struct aim_ctx {
   aim::Schedule sched[3] = {};
   aim::MultiLauncher* multi = nullptr;   // buffers of the multi-context calls that this context leads
   // bookkeeping
-  std::vector<std::pair<const void*, size_t>> smem_raised;   // dynamic shared memory limits raised so far
+  std::vector<const void*> smem_raised;   // kernels whose dynamic shared memory limit is raised
   struct CoopSlots { const void* kernel; int threads; size_t smem; int slots; };
   std::vector<CoopSlots> coop_slots;                         // resident_ctas of multi-context launches led
   std::vector<void*> allocations;

@@ -985,20 +985,22 @@ inline int gather_rhs_block(int n, int nrhs) {
 // ------------------------------------------------------------------------------------
 // launch configuration
 // ------------------------------------------------------------------------------------
-// Raises a kernel's dynamic shared memory limit; the context remembers what it has raised.
+constexpr size_t kMaxDynSmem = 227 * 1024;   // opt-in dynamic shared memory per CTA
+
+// Lets a kernel take as much dynamic shared memory as a CTA may have. The limit belongs to the device,
+// not to a context: every context sets the same value, so none lowers another's, and each remembers the
+// kernels for which it has done so (two host calls per launch otherwise).
 template <typename K>
 static aim_status ensure_smem(aim_ctx* ctx, K kernel, size_t bytes) {
   if (bytes <= 48 * 1024) return AIM_OK;
   const void* id = reinterpret_cast<const void*>(kernel);
-  for (auto& kb : ctx->smem_raised)
-    if (kb.first == id && kb.second >= bytes) return AIM_OK;
-  AIM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  for (auto& kb : ctx->smem_raised)
-    if (kb.first == id) {
-      kb.second = bytes;
-      return AIM_OK;
-    }
-  ctx->smem_raised.emplace_back(id, bytes);
+  for (const void* raised : ctx->smem_raised)
+    if (raised == id) return AIM_OK;
+  cudaFuncAttributes fa;
+  AIM_CUDA_TRY(cudaFuncGetAttributes(&fa, kernel));
+  AIM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kMaxDynSmem - fa.sharedSizeBytes)));
+  ctx->smem_raised.push_back(id);
   return AIM_OK;
 }
 
@@ -1015,8 +1017,6 @@ static const void* near_values(const NearField* nf, int which, dfc*) { return nf
 static int precision_of(float2*) { return AIM_MIXED; }
 static int precision_of(double2*) { return AIM_FP64_NATIVE; }
 static int precision_of(dfc*) { return AIM_FP64; }
-
-constexpr size_t kMaxDynSmem = 227 * 1024;   // opt-in dynamic shared memory per CTA
 
 // Which (transforms per thread, elements per thread) pairs are compiled for an element type:
 // native binary64 keeps two transforms of 16 elements per thread

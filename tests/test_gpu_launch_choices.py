@@ -116,3 +116,19 @@ def test_solves_around_the_last_one_launch_step(aimlib, restart):
         assert abs(rel[i] - info[i]["rel_res"]) < 1e-9, (rel[i], info[i])
         assert not info[i]["converged"] or rel[i] < 2.0 * tol
     ctx.close()
+
+
+def test_contexts_of_different_shared_memory_take_turns(aimlib):
+    # the limit of a kernel's dynamic shared memory is the device's: a context that needs less of it must
+    # not take it from one that needs more (147 KB and 74 KB column CTAs of the same kernel)
+    ctxs = []
+    for per, n, m, P in ((100.0, 900, 800, 2048), (60.0, 600, 400, 1024)):
+        c = aimlib.Context(synth.StarContour.from_seed(9).polygon(per, n), K, aimlib.TE, m, fft_P=P, alpha=3.0 * K)
+        c.set_schedule(0, 2, 128, 4, 8)
+        ctxs.append((c, torch.from_numpy(synth.random_coeffs(n, 1, seed=5)).cuda()))
+    first = [product(c, "N", x, 0) for c, x in ctxs]
+    for _ in range(2):
+        for (c, x), want in zip(ctxs, first):
+            assert np.array_equal(product(c, "N", x, 0), want)
+    for c, _ in ctxs:
+        c.close()
