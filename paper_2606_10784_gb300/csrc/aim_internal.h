@@ -235,9 +235,12 @@ inline bool sched_is_default(const aim_ctx* ctx, int precision) {
   const Schedule &a = ctx->sched[precision], b = default_schedule(precision, ctx->P);
   return a.tpt == b.tpt && a.min_row_threads == b.min_row_threads && a.col_cols == b.col_cols && a.elems == b.elems;
 }
-// the geometry a context stands for in the check of a multi-context call
-inline Schedule multi_geometry(const aim_ctx* ctx, int precision) {
-  return sched_is_default(ctx, precision) ? default_schedule(precision, kMaxP) : ctx->sched[precision];
+// The elements per thread that a context can stand for in the check of a multi-context call, a bit for 8
+// and a bit for 16: its own, and on the schedule it starts with also those of the largest grids, so that
+// contexts whose defaults differ by size alone go together.
+inline unsigned multi_elems(const aim_ctx* ctx, int precision) {
+  auto bit = [](const Schedule& s) { return s.elems == 8 ? 1u : 2u; };
+  return bit(ctx->sched[precision]) | (sched_is_default(ctx, precision) ? bit(default_schedule(precision, kMaxP)) : 0u);
 }
 
 // allocation helpers (tracked by the context)

@@ -1620,13 +1620,13 @@ template <typename CT>
 aim_status grid_pass_multi(const MultiPassSpec* passes, int count, unsigned* scratch, int* err_host, cudaStream_t st) {
   if (count < 1 || count > kMaxMultiJobs) return fail(AIM_EINVAL, "1 to 32 passes per multi-context launch");
   const int p = precision_of((CT*)nullptr);
-  // Contexts may share a call when their pass geometries agree, a context on its default schedule
-  // standing for the geometry of the largest grids: such contexts differ in elements per thread by
-  // size, and each runs with its own (so that its results are those of a launch of its own).
-  const Schedule sc = multi_geometry(passes[0].ctx, p);
-  for (int i = 1; i < count; ++i) {
-    const Schedule o = multi_geometry(passes[i].ctx, p);
-    if (o.tpt != sc.tpt || loge_of(o) != loge_of(sc))
+  // Contexts may share a call when there is one pass geometry that all of them stand for; each runs with
+  // its own elements per thread (so that its results are those of a launch of its own).
+  const Schedule& sc = passes[0].ctx->sched[p];
+  unsigned elems = 3;
+  for (int i = 0; i < count; ++i) {
+    elems &= multi_elems(passes[i].ctx, p);
+    if (passes[i].ctx->sched[p].tpt != sc.tpt || elems == 0)
       return fail(AIM_EINVAL, "contexts of one multi-context launch must share the pass geometry of their schedule");
   }
   if constexpr (std::is_same<CT, double2>::value) {
