@@ -359,7 +359,9 @@ struct MultiLauncher {
   unsigned* scratch = nullptr;   // 4 words per stage
   int* err_host = nullptr;       // one flag per stage
   aim_status init(cudaStream_t st);
-  aim_status check(cudaStream_t st);   // after a synchronisation: AIM_ETIMEOUT if a launch gave up
+  // after a synchronisation: whether a launch gave up; buffers as new for the next call
+  bool rearm(cudaStream_t st);
+  aim_status check(cudaStream_t st);   // the same as a status: AIM_ETIMEOUT if a launch gave up
   ~MultiLauncher();
 };
 // y_i = A_i x_i for `count` contexts (device vectors), every grid pass stage of all of them in one

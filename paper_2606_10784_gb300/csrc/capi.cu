@@ -226,15 +226,21 @@ aim_status MultiLauncher::init(cudaStream_t st) {
   return AIM_OK;
 }
 
-aim_status MultiLauncher::check(cudaStream_t st) {
+bool MultiLauncher::rearm(cudaStream_t st) {
   bool bad = false;
-  for (int i = 0; i < kMultiStages; ++i) {
-    bad = bad || (err_host != nullptr && err_host[i] != 0);
-    if (err_host != nullptr) err_host[i] = 0;
+  for (int i = 0; err_host != nullptr && i < kMultiStages; ++i) {
+    bad = bad || err_host[i] != 0;
+    err_host[i] = 0;
   }
-  if (!bad) return AIM_OK;
-  cudaMemsetAsync(scratch, 0, kMultiStages * 4 * sizeof(unsigned), st);
-  cudaStreamSynchronize(st);   // the next call may use another stream
+  if (bad) {
+    cudaMemsetAsync(scratch, 0, kMultiStages * 4 * sizeof(unsigned), st);
+    cudaStreamSynchronize(st);   // the next call may use another stream
+  }
+  return bad;
+}
+
+aim_status MultiLauncher::check(cudaStream_t st) {
+  if (!rearm(st)) return AIM_OK;
   return fail(AIM_ETIMEOUT, "a grid barrier of the multi-context launch gave up waiting");
 }
 
@@ -665,7 +671,10 @@ aim_status aim_matvec_multi(int count, aim_ctx* const* ctxs, const aim_op* ops, 
                                 reinterpret_cast<double2* const*>(y), precision, st);
   const cudaError_t e = cudaStreamSynchronize(st);
   if (s == AIM_OK && e != cudaSuccess) s = fail(AIM_ECUDA, std::string("multi-context product: ") + cudaGetErrorString(e));
+  // a launch that gave up leaves its barrier words and flags set: whatever else went wrong, the context
+  // must not hand them to the next call that it leads (the first error is the one reported)
   if (s == AIM_OK) s = ml.check(st);
+  else ml.rearm(st);
   return s;
 }
 
