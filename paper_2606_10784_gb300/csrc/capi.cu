@@ -212,10 +212,13 @@ constexpr int kMultiStages = 2;
 
 aim_status MultiLauncher::init(cudaStream_t st) {
   if (scratch != nullptr) return AIM_OK;
+  // each buffer is the launcher's as soon as it exists: a call after one that failed half-way takes it up
   void* p = nullptr;
-  AIM_CUDA_TRY(cudaMallocHost(&p, kMultiStages * sizeof(int)));
-  err_host = static_cast<int*>(p);
-  for (int i = 0; i < kMultiStages; ++i) err_host[i] = 0;
+  if (err_host == nullptr) {
+    AIM_CUDA_TRY(cudaMallocHost(&p, kMultiStages * sizeof(int)));
+    err_host = static_cast<int*>(p);
+    for (int i = 0; i < kMultiStages; ++i) err_host[i] = 0;
+  }
   AIM_CUDA_TRY(cudaMalloc(&p, kMultiStages * 4 * sizeof(unsigned)));
   const cudaError_t e = cudaMemsetAsync(p, 0, kMultiStages * 4 * sizeof(unsigned), st);
   if (e != cudaSuccess) {

@@ -7,4 +7,15 @@ extern "C" {
 int* probe_err_host(aim_ctx* ctx) { return ctx->multi ? ctx->multi->err_host : nullptr; }
 void* probe_scratch(aim_ctx* ctx) { return ctx->multi ? ctx->multi->scratch : nullptr; }
 
+// Whether a launcher whose device allocation had failed takes up the pinned flags that it already held.
+int probe_init_keeps_flags() {
+  aim::MultiLauncher first, rest;
+  if (first.init(nullptr) != AIM_OK) return -1;
+  int* flags = first.err_host;
+  rest.scratch = first.scratch;   // freed with `rest`
+  first.scratch = nullptr;        // as after a refused cudaMalloc
+  if (first.init(nullptr) != AIM_OK) return -1;
+  return first.err_host == flags && first.scratch != nullptr;
+}
+
 }  // extern "C"

@@ -32,6 +32,7 @@ def probe(aimlib, tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(os.path.dirname(aimlib.LIB_PATH), "csrc"),
                     "-I", os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"),
                     os.path.join(HERE, "multi_launcher_probe.cpp"), "-o", out], check=True, timeout=120)
+    ctypes.CDLL(aimlib.LIB_PATH, mode=ctypes.RTLD_GLOBAL)
     lib = ctypes.CDLL(out)
     for f, t in ((lib.probe_err_host, ctypes.POINTER(ctypes.c_int)), (lib.probe_scratch, ctypes.c_void_p)):
         f.argtypes, f.restype = [ctypes.c_void_p], t
@@ -88,3 +89,7 @@ def test_a_failed_call_leaves_nothing_to_the_next(aimlib, probe, stage):
     assert all(torch.equal(y, w) for y, w in zip(ys, want))
     for c in ctxs:
         c.close()
+
+
+def test_a_second_init_takes_up_the_pinned_flags(probe):
+    assert probe.probe_init_keeps_flags() == 1
