@@ -359,6 +359,7 @@ struct MultiLauncher {
   unsigned* scratch = nullptr;   // 4 words per stage
   int* err_host = nullptr;       // one flag per stage
   aim_status init(cudaStream_t st);
+  bool gave_up() const;   // whether a launch that is complete gave up (and was not rearmed since)
   // after a synchronisation: whether a launch gave up; buffers as new for the next call
   bool rearm(cudaStream_t st);
   aim_status check(cudaStream_t st);   // the same as a status: AIM_ETIMEOUT if a launch gave up
@@ -377,6 +378,7 @@ struct aim_batcher;
 namespace aim {
 // the batcher attached to the calling thread by aim_solve_batched (nullptr outside it)
 aim_batcher* current_batcher();
+MultiLauncher& batcher_launcher(aim_batcher* b);   // of its fused products
 // y = A x for one solve, fused with the products that other solves of the batcher submit at about
 // the same time; asynchronous: `st` waits for the result on the device
 aim_status batcher_product(aim_batcher* b, aim_ctx* ctx, aim_op op, int nrhs, const double2* x, double2* y,

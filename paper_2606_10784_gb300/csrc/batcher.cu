@@ -69,6 +69,16 @@ static thread_local aim_batcher* tl_batcher = nullptr;
 
 aim_batcher* current_batcher() { return tl_batcher; }
 
+MultiLauncher& batcher_launcher(aim_batcher* b) { return b->ml; }
+
+// A fused launch whose grid barrier gave up leaves its results unwritten, and so does every fused launch
+// queued behind it (their waits poll the same flag). Its flag is never cleared here: from then on the
+// batcher refuses products, and a solve that ended after it reports the timeout. Called with the lock held.
+static aim_status note_give_up(aim_batcher* b) {
+  if (b->broken == AIM_OK && b->ml.gave_up()) b->broken = AIM_ETIMEOUT;
+  return b->broken == AIM_OK ? AIM_OK : fail(b->broken, "a grid barrier of a fused product gave up waiting");
+}
+
 // Launches every pending request: grouped by precision and size class; a group of one runs the
 // single-context path, a larger group one multi-context launch per grid-pass stage. Called with
 // the lock held.
@@ -86,7 +96,7 @@ static void lead(aim_batcher* b) {
            size_class(reqs[j]->ctx) == size_class(reqs[i]->ctx))
       ++j;
     // the batcher's stream waits for every input of the group
-    aim_status s = b->broken;
+    aim_status s = note_give_up(b);
     for (size_t q = i; q < j && s == AIM_OK; ++q)
       if (cudaStreamWaitEvent(b->stream, reqs[q]->in, 0) != cudaSuccess) s = fail(AIM_ECUDA, "batcher: wait for input");
     if (s == AIM_OK) {
@@ -220,13 +230,12 @@ aim_status aim_solve_batched(aim_batcher* b, aim_ctx* ctx, aim_op system, int nr
     b->participants[cls] -= 1;
     b->cv.notify_all();   // partners no longer wait for this solve
   }
-  if (s == AIM_OK) {
-    // a fused launch whose grid barrier gave up (its flag is read once the launches are done)
+  if (fusible && (s == AIM_OK || s == AIM_ENOCONV || s == AIM_ENUMERIC)) {
+    // this solve's launches are complete (aim_solve waits for its stream, and that for each product), so the
+    // flag says whether one of them gave up, however busy other solves keep the batcher's stream
     std::lock_guard<std::mutex> lk(b->mu);
-    if (cudaStreamQuery(b->stream) == cudaSuccess) {
-      const aim_status e = b->ml.check(b->stream);
-      if (e != AIM_OK) b->broken = s = e;
-    }
+    const aim_status e = note_give_up(b);
+    if (e != AIM_OK) s = e;
   }
   return s;
 }

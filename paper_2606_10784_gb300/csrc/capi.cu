@@ -229,13 +229,17 @@ aim_status MultiLauncher::init(cudaStream_t st) {
   return AIM_OK;
 }
 
+bool MultiLauncher::gave_up() const {
+  const volatile int* flags = err_host;
+  for (int i = 0; flags != nullptr && i < kMultiStages; ++i)
+    if (flags[i] != 0) return true;
+  return false;
+}
+
 bool MultiLauncher::rearm(cudaStream_t st) {
-  bool bad = false;
-  for (int i = 0; err_host != nullptr && i < kMultiStages; ++i) {
-    bad = bad || err_host[i] != 0;
-    err_host[i] = 0;
-  }
+  const bool bad = gave_up();
   if (bad) {
+    for (int i = 0; i < kMultiStages; ++i) err_host[i] = 0;
     cudaMemsetAsync(scratch, 0, kMultiStages * 4 * sizeof(unsigned), st);
     cudaStreamSynchronize(st);   // the next call may use another stream
   }

@@ -4,6 +4,8 @@ import ctypes
 import math
 import os
 import subprocess
+import threading
+import time
 
 import pytest
 
@@ -34,7 +36,8 @@ def probe(aimlib, tmp_path_factory):
                     os.path.join(HERE, "multi_launcher_probe.cpp"), "-o", out], check=True, timeout=120)
     ctypes.CDLL(aimlib.LIB_PATH, mode=ctypes.RTLD_GLOBAL)
     lib = ctypes.CDLL(out)
-    for f, t in ((lib.probe_err_host, ctypes.POINTER(ctypes.c_int)), (lib.probe_scratch, ctypes.c_void_p)):
+    flags = ctypes.POINTER(ctypes.c_int)
+    for f, t in ((lib.probe_err_host, flags), (lib.probe_scratch, ctypes.c_void_p), (lib.probe_batcher_err_host, flags)):
         f.argtypes, f.restype = [ctypes.c_void_p], t
     return lib
 
@@ -93,3 +96,37 @@ def test_a_failed_call_leaves_nothing_to_the_next(aimlib, probe, stage):
 
 def test_a_second_init_takes_up_the_pinned_flags(probe):
     assert probe.probe_init_keeps_flags() == 1
+
+
+def solve(aim, ctx, batcher, out, i, max_iter):
+    n = ctx.n
+    b = torch.from_numpy(synth.random_coeffs(n, 1, seed=i)).cuda()
+    x, st = torch.zeros_like(b), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    out[i] = ctx.solve("calderon", b, x, tol=1e-15, restart=60, max_iter=max_iter, stream=st, check=False,
+                       batcher=batcher)[0]
+
+
+def test_a_batcher_that_gave_up_refuses_and_reports(aimlib, probe):
+    sizes = [(150, 64), (160, 64), (1100, 300)]   # P = 128 twice, and P = 1024, which is not fused
+    ctxs, out = contexts(aimlib, sizes), {}
+    batcher = aimlib.Batcher(max_wait_us=100)
+    # the first solve runs for many seconds if nothing stops it; the flag is raised while it keeps the stream busy
+    t = threading.Thread(target=solve, args=(aimlib, ctxs[0], batcher, out, 0, 200000))
+    t.start()
+    while batcher.stats()["launches"] < 50:
+        time.sleep(0.01)
+    probe.probe_batcher_err_host(batcher._h)[1] = 1
+    solve(aimlib, ctxs[1], batcher, out, 1, 40)
+    t.join(timeout=60)
+    assert not t.is_alive()
+    assert out == {0: aimlib.ETIMEOUT, 1: aimlib.ETIMEOUT}
+    # nothing is launched any more, and a solve that never fuses is not concerned
+    before = batcher.stats()["launches"]
+    solve(aimlib, ctxs[1], batcher, out, 1, 40)
+    solve(aimlib, ctxs[2], batcher, out, 2, 40)
+    assert out[1] == aimlib.ETIMEOUT and out[2] == aimlib.ENOCONV
+    assert batcher.stats()["launches"] == before
+    batcher.close()
+    for c in ctxs:
+        c.close()
