@@ -173,6 +173,7 @@ struct aim_ctx {
   int device = 0;
   // active grid set
   int n_act = 0, row_lo = 0, row_hi = -1, nrows = 0;
+  int row_most = 0;         // the most points of a row
   int* row_ptr = nullptr;   // m + 1 : active points of grid row iy are [row_ptr[iy], row_ptr[iy+1])
   int* act_ix = nullptr;    // n_act : column index of each active point
   aim::Projections prj;
@@ -241,6 +242,13 @@ inline bool sched_is_default(const aim_ctx* ctx, int precision) {
 inline unsigned multi_elems(const aim_ctx* ctx, int precision) {
   auto bit = [](const Schedule& s) { return s.elems == 8 ? 1u : 2u; };
   return bit(ctx->sched[precision]) | (sched_is_default(ctx, precision) ? bit(default_schedule(precision, kMaxP)) : 0u);
+}
+
+// the most points of a grid row, from the row pointers
+inline int most_per_row(const int* row_ptr, int m) {
+  int most = 0;
+  for (int iy = 0; iy < m; ++iy) most = row_ptr[iy + 1] - row_ptr[iy] > most ? row_ptr[iy + 1] - row_ptr[iy] : most;
+  return most;
 }
 
 // allocation helpers (tracked by the context)

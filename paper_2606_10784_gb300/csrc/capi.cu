@@ -458,6 +458,7 @@ aim_status aim_setup(const aim_geometry* geometry, double k, const aim_grid* gri
   ctx->row_lo = hs.row_lo;
   ctx->row_hi = hs.row_hi;
   ctx->nrows = hs.row_hi - hs.row_lo + 1;
+  ctx->row_most = most_per_row(hs.row_ptr.data(), ctx->m);
 
   // upload
   std::vector<double2> nodes(ctx->n);

@@ -32,6 +32,7 @@
 #pragma once
 
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 #include <vector>
 
@@ -126,6 +127,7 @@ struct RowFwdArgs {
   int rows_per_cta;
   int qcut;            // columns q with min(q, P - q) > qcut carry a zero spectrum: not stored
   int sparse;          // few active points per row: the first radix runs at the active points only
+  int dense_from;      // sparse: rows of more points than this take the dense passes all the same
 };
 
 // Output k of a row's transforms into the tiled intermediate: X[2k] and X[2k + 1] are neighbours in
@@ -192,6 +194,22 @@ static bool sparse_rows(const aim_ctx* ctx) {
   return 4LL * ctx->n_act <= ((long long)ctx->nrows * l0) << logj;
 }
 
+// A row of a sparse context that holds more points than this takes the dense passes: where a contour runs
+// along the grid a few rows hold hundreds of points each, their sums run in one CTA, and the launch waits
+// for it. The line is at the points that cost kDenseRow times the dense radix of a row: a CTA that holds
+// rows of both kinds runs one after the other, so with a lower line the few dozen points of a curved
+// contour's extreme rows cost more than they save. (Row passes of a square of 2000 points a side, P = 4096,
+// double-float S^alpha 378 -> 182 us; 900 a side, P = 2048, N 195 -> 132 us; complex64, 400 a side, P = 1024,
+// N 41 -> 24 us. A line at 8 leaves the squares of P <= 512 at 22 to 28 us instead of 18 to 27, one at 2
+// takes the star contour of P = 256 from 20 to 30.) It depends on the context alone, so that results depend
+// neither on the number of right-hand sides nor on the launch.
+template <int LOGE>
+static int sparse_row_limit(const aim_ctx* ctx) {
+  constexpr int kDenseRow = 4;
+  const int logj = sparse_logj<LOGE>(ctx->logH), l0 = ctx->logH - logj, limit = (kDenseRow * l0 << logj) / 4;
+  return ctx->row_most > limit ? limit : INT_MAX;
+}
+
 // Forward row pass of sparse rows. The points of a row go to their places j + J r of the row's two
 // buffers (u in the even half's, u w^j in the odd half's) and into the masks that say which r of a j
 // hold one; nothing else is written, so nothing is zeroed. The first dense pass forms its inputs
@@ -201,7 +219,7 @@ static bool sparse_rows(const aim_ctx* ctx) {
 // at 2048 points, and 13 of 33 us at 512 points, where the rows along the contour's tangents set the
 // time of the whole launch.)
 template <typename CT, int TPT, int LOGE>
-__device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_block, int c, unsigned char* smraw) {
+__device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_block, int c, bool skip, unsigned char* smraw) {
   using T2 = CT;
   constexpr int NF = TPT, LPT = 3 - TPT;
   T2* sm = reinterpret_cast<T2*>(smraw);
@@ -210,7 +228,7 @@ __device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_bloc
   const int g = threadIdx.x / per_row, rem = threadIdx.x - g * per_row;
   const int half = TPT == 1 ? (rem & 1) : 0, j = TPT == 1 ? (rem >> 1) : rem;
   const int row0 = row_block * a.rows_per_cta, rloc = row0 + g;
-  const bool live = rloc < a.nrows;
+  const bool live = rloc < a.nrows && !skip;
   const T2* tw = static_cast<const T2*>(a.tw);
   int fb[NF];
 #pragma unroll
@@ -268,10 +286,12 @@ __device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_bloc
 
 // One work item of the forward row pass: rows [row_block * rows_per_cta, +rows_per_cta) of channel c.
 // Every thread of the CTA calls it (it holds barriers); `smraw` is the CTA's dynamic shared memory.
-template <typename CT, int TPT, int LOGE>
+// LONG: rows of more points than a.dense_from may be among the sparse ones (a variant of its own: with the
+// second path behind the first the double-float passes spill more, 469 -> 487 us at P = 4096).
+template <typename CT, int TPT, int LOGE, bool LONG>
 __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block, int c, unsigned char* smraw) {
-  if (a.sparse) {
-    row_fwd_sparse<CT, TPT, LOGE>(a, row_block, c, smraw);
+  if (!LONG && a.sparse) {
+    row_fwd_sparse<CT, TPT, LOGE>(a, row_block, c, false, smraw);
     return;
   }
   using T2 = CT;
@@ -282,7 +302,16 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
   const int g = threadIdx.x / per_row, rem = threadIdx.x - g * per_row;
   const int half = TPT == 1 ? (rem & 1) : 0, j = TPT == 1 ? (rem >> 1) : rem;
   const int rloc = row_block * a.rows_per_cta + g;
-  const bool live = rloc < a.nrows;
+  bool live = rloc < a.nrows;
+  if (LONG && a.sparse) {
+    // each row by its own count: first the CTA's sparse rows, then its dense ones
+    const bool full = live && a.row_ptr[a.row_lo + rloc + 1] - a.row_ptr[a.row_lo + rloc] > a.dense_from;
+    const bool any_full = __syncthreads_or(full), any_sparse = __syncthreads_or(live && !full);
+    if (any_sparse) row_fwd_sparse<CT, TPT, LOGE>(a, row_block, c, full, smraw);
+    if (!any_full) return;
+    __syncthreads();
+    live = full;
+  }
   const int iy = a.row_lo + rloc;
   const T2* tw = static_cast<const T2*>(a.tw);
   const int fbA = (2 * g) * HS;
@@ -345,11 +374,11 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
   });
 }
 
-template <typename CT, int TPT, int LOGE, bool WIDE = false>
+template <typename CT, int TPT, int LOGE, bool WIDE, bool LONG>
 __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_row_fwd(RowFwdArgs a) {
   grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
-  row_fwd_item<CT, TPT, LOGE>(a, blockIdx.x, blockIdx.y, smraw);
+  row_fwd_item<CT, TPT, LOGE, LONG>(a, blockIdx.x, blockIdx.y, smraw);
 }
 
 // ------------------------------------------------------------------------------------
@@ -624,7 +653,7 @@ struct RowInvArgs {
   double scale;
   int rows_per_cta;
   int qcut;            // as in RowFwdArgs
-  int sparse;
+  int sparse, dense_from;
 };
 
 // value of another lane (xor of the lane index); all 32 lanes call it together
@@ -648,7 +677,8 @@ __device__ __forceinline__ dfc shfl_xor_c(dfc v, int off) {
 __device__ __forceinline__ int sparse_point_lanes(int k2) { return max(2, k2 >> 2); }
 
 // One work item of the inverse row pass: rows [row_block * rows_per_cta, +rows_per_cta) of channel c.
-template <typename CT, int TPT, int LOGE>
+// LONG as in row_fwd_item.
+template <typename CT, int TPT, int LOGE, bool LONG>
 __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block, int c, unsigned char* smraw) {
   using T2 = CT;
   using VT = typename GridT<CT>::VT;
@@ -659,7 +689,7 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
   const int g = threadIdx.x / per_row, rem = threadIdx.x - g * per_row;
   const int half = TPT == 1 ? (rem & 1) : 0, j = TPT == 1 ? (rem >> 1) : rem;
   const int rloc = row_block * a.rows_per_cta + g;
-  const bool live = rloc < a.nrows;
+  bool live = rloc < a.nrows;
   const int iy = a.row_lo + rloc;
   const T2* tw = static_cast<const T2*>(a.tw);
   const int fbA = (2 * g) * HS;
@@ -723,6 +753,7 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
     }
     __syncthreads();
   }
+  int p0 = 1;   // the passes done
   if (a.sparse) {
     const int logj = sparse_logj<LOGE>(a.logH), J = 1 << logj, k2 = 2 << (a.logH - logj), tpl = k2 / lpp;
     if (logj > LOGE) smem_pass<LOGE, true, NF, LOGE>(sm, fb, j, tpf, a.logH, LOGE, tw, a.logP);
@@ -733,18 +764,25 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
     const int l = threadIdx.x & (lpp - 1), grp = threadIdx.x / lpp, ngrp = blockDim.x / lpp;
     using VP = decltype(VT::x);
     VP* out = static_cast<VP*>(a.vact) + 2 * (size_t)c * a.n_act;
-    for (int base = A0; base < A1; base += ngrp) {
+    const bool mixed = LONG && a.dense_from != INT_MAX;   // rows of too many points among them (sparse_row_limit)
+    const bool full = mixed && live && rps[g + 1] - rps[g] > a.dense_from;
+    const int a1 = mixed && !__syncthreads_or(live && !full) ? A0 : A1;
+    for (int base = A0; base < a1; base += ngrp) {
       const int ap = base + grp;
-      const bool valid = ap < A1;
-      T2 acc = czero<T2>();
+      bool valid = ap < a1;
+      int lo = 0;
       if (valid) {
-        const int ix = base == A0 ? ix0 : a.act_ix[ap];
-        const T2 z = base == A0 ? z0 : ldro(&tw[ix]);
-        int lo = 0, hi = a.rows_per_cta;
+        int hi = a.rows_per_cta;
         while (hi - lo > 1) {
           const int mid = (lo + hi) >> 1;
           if (rps[mid] <= ap) lo = mid; else hi = mid;
         }
+        valid = !mixed || rps[lo + 1] - rps[lo] <= a.dense_from;
+      }
+      T2 acc = czero<T2>();
+      if (valid) {
+        const int ix = base == A0 ? ix0 : a.act_ix[ap];
+        const T2 z = base == A0 ? z0 : ldro(&tw[ix]);
         const T2* zb = sm + (size_t)(2 * lo) * HS;
         const int jj = ix & (J - 1), k0 = l * tpl;
         for (int t = tpl - 1; t >= 0; --t) {
@@ -759,10 +797,13 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
       // conversions of the double-float types run at the FP64 rate, once per component and warp
       if (valid && l < 2) out[2 * ap + l] = cto_vt_part(acc, l, a.scale);
     }
-    return;
+    if (!mixed || !__syncthreads_or(full)) return;
+    // rows of too many points go on with the dense passes, of which they have those so far
+    live = full;
+    p0 = logj / LOGE;
   }
   const int np = fft_npass<LOGE>(a.logH);
-  smem_passes<true, NF, LOGE>(sm, fb, j, tpf, a.logH, 1, np - 1, LOGE, tw, a.logP);
+  smem_passes<true, NF, LOGE>(sm, fb, j, tpf, a.logH, p0, np - 1, LOGE * p0, tw, a.logP);
   int logNs = 0;
   for (int p = 0; p < np - 1; ++p) logNs += fft_logr<LOGE>(p, a.logH);
   const double sc = a.scale;
@@ -789,11 +830,11 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
   }
 }
 
-template <typename CT, int TPT, int LOGE, bool WIDE = false>
+template <typename CT, int TPT, int LOGE, bool WIDE, bool LONG>
 __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_row_inv(RowInvArgs a) {
   grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
-  row_inv_item<CT, TPT, LOGE>(a, blockIdx.x, blockIdx.y, smraw);
+  row_inv_item<CT, TPT, LOGE, LONG>(a, blockIdx.x, blockIdx.y, smraw);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1091,12 +1132,14 @@ aim_status launch_row_fwd(aim_ctx* ctx, int channels, RowFwdArgs fa, const Sched
   constexpr int LPT = 3 - TPT;
   const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
   fa.sparse = !fa.dense && sparse_rows<LOGE>(ctx);
+  fa.dense_from = sparse_row_limit<LOGE>(ctx);
   fa.rows_per_cta = rpc;
   const size_t smem =
       2 * (size_t)rpc * padded_len<LOGE>(ctx->H) * sizeof(CT) + (fa.sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
-  AIM_TRY(ensure_smem(ctx, k_row_fwd<CT, TPT, LOGE, WIDE>, smem));
+  const auto kernel = fa.sparse && fa.dense_from != INT_MAX ? k_row_fwd<CT, TPT, LOGE, WIDE, true> : k_row_fwd<CT, TPT, LOGE, WIDE, false>;
+  AIM_TRY(ensure_smem(ctx, kernel, smem));
   ProfScope ps(K_ROW_FWD, st);
-  return launch_chained(k_row_fwd<CT, TPT, LOGE, WIDE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, fa);
+  return launch_chained(kernel, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, fa);
 }
 
 template <typename CT, int TPT, int LOGE, bool WIDE>
@@ -1120,12 +1163,14 @@ aim_status launch_row_inv(aim_ctx* ctx, int channels, RowInvArgs ia, const Sched
   constexpr int LPT = 3 - TPT;
   const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
   ia.sparse = !ia.dense && sparse_rows<LOGE>(ctx);
+  ia.dense_from = sparse_row_limit<LOGE>(ctx);
   ia.rows_per_cta = rpc;
   const size_t smem =
       2 * (size_t)rpc * padded_len<LOGE>(ctx->H) * sizeof(CT) + (ia.sparse ? sparse_smem<CT, LOGE>(ctx->logH, rpc) : 0);
-  AIM_TRY(ensure_smem(ctx, k_row_inv<CT, TPT, LOGE, WIDE>, smem));
+  const auto kernel = ia.sparse && ia.dense_from != INT_MAX ? k_row_inv<CT, TPT, LOGE, WIDE, true> : k_row_inv<CT, TPT, LOGE, WIDE, false>;
+  AIM_TRY(ensure_smem(ctx, kernel, smem));
   ProfScope ps(K_ROW_INV, st);
-  return launch_chained(k_row_inv<CT, TPT, LOGE, WIDE>, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, ia);
+  return launch_chained(kernel, dim3((ctx->nrows + rpc - 1) / rpc, channels), rpc * LPT * tpf, smem, st, ia);
 }
 
 // Transforms per thread of a pass of `lines` lines whose two-transform form has tpf threads a line.
@@ -1408,7 +1453,7 @@ __global__ void __launch_bounds__(MultiMax<CT, TPT, LOGE>::value) k_grid_multi(c
         const long long t = local * blockDim.x + threadIdx.x;
         if (J.nproj == 1) ant_item<CT, 1>(J.aa, t); else ant_item<CT, 3>(J.aa, t);
       } else if (phase == 1) {
-        row_fwd_item<CT, TPT, LOGE>(J.fa, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
+        row_fwd_item<CT, TPT, LOGE, true>(J.fa, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
       } else if (phase == 2) {
         // many channels (right-hand sides): the channels of one column tile run back to back and
         // share its spectrum column through L2, as the single-context launch orders them
@@ -1416,7 +1461,7 @@ __global__ void __launch_bounds__(MultiMax<CT, TPT, LOGE>::value) k_grid_multi(c
         const int ch = J.tile_major ? (int)(local % J.channels) : (int)(local / J.col_items);
         col_conv_item<CT, TPT, LOGE>(J.ca, tile, ch, smraw);
       } else if (phase == 3) {
-        row_inv_item<CT, TPT, LOGE>(J.ia, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
+        row_inv_item<CT, TPT, LOGE, true>(J.ia, (int)(local % J.row_items), (int)(local / J.row_items), smraw);
       } else {
         auto gather = [&](auto np) {
           constexpr int NP = decltype(np)::value;
@@ -1533,6 +1578,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
     fa.rows_per_cta = lines;
     fa.qcut = qcut;
     fa.sparse = sparse;
+    fa.dense_from = sparse_row_limit<LOGE>(ctx);
     ColArgs& ca = J.ca;
     ca.inter = ctx->inter;
     ca.spec = spectrum(ctx, spec.filtered, (CT*)nullptr);
@@ -1563,6 +1609,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
     ia.rows_per_cta = lines;
     ia.qcut = qcut;
     ia.sparse = sparse;
+    ia.dense_from = fa.dense_from;
     J.ga = gather_args<CT>(ctx, spec, ps.nrhs, ps.x, ps.y);
     J.gather_rb = ps.nrhs == 1 ? 1 : ps.nrhs <= 4 ? 4 : 8;
     J.row_items = (ctx->nrows + lines - 1) / lines;

@@ -270,6 +270,7 @@ aim_status aim_import_setup(const aim_geometry* geometry, double k, const aim_gr
   if (ok && near_sec >= 0)
     ok = csr_ok(ints(near_sec), n, h.nnz) && all_below(ints(near_sec + 1), (size_t)h.nnz, n);
   if (!ok) return fail(AIM_EINVAL, "setup blob holds an index out of range");
+  ctx->row_most = most_per_row(ints(SEC_ROW_PTR), m);
 
   // device state: the stored arrays, then the copies derived from them
   cudaStream_t st = static_cast<cudaStream_t>(stream);
