@@ -187,11 +187,15 @@ __host__ __device__ __forceinline__ size_t sparse_smem(int logH, int rows) {
 
 // Whether a context's rows take the sparse stages. Counting operations, a point costs 2 R0 products
 // and sums where the dense radix-R0 passes cost about 0.57 J log2(R0) of them per row; the line lies
-// at half of that because the operations on single points are slower than those of the dense passes.
-template <int LOGE>
+// at half of that because the operations on single points are slower than those of the dense passes, and
+// for binary64, where they run on the FP64 pipe of the few SMs that hold the longest rows, at a twelfth: at a
+// twentieth (a contour of 1000 wavelengths, P = 4096) the row passes gain 29 %, at an eighth (100 wavelengths,
+// P = 1024) 2 to 6 %, and at a half (P = 512) they take 79 -> 109 us.
+template <typename CT, int LOGE>
 static bool sparse_rows(const aim_ctx* ctx) {
+  constexpr long long kCost = std::is_same<CT, double2>::value ? 24 : 4;
   const int logj = sparse_logj<LOGE>(ctx->logH), l0 = ctx->logH - logj;
-  return 4LL * ctx->n_act <= ((long long)ctx->nrows * l0) << logj;
+  return kCost * ctx->n_act <= ((long long)ctx->nrows * l0) << logj;
 }
 
 // A row of a sparse context that holds more points than this takes the dense passes: where a contour runs
@@ -1131,7 +1135,7 @@ template <typename CT, int TPT, int LOGE, bool WIDE>
 aim_status launch_row_fwd(aim_ctx* ctx, int channels, RowFwdArgs fa, const Schedule& sc, cudaStream_t st) {
   constexpr int LPT = 3 - TPT;
   const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
-  fa.sparse = !fa.dense && sparse_rows<LOGE>(ctx);
+  fa.sparse = !fa.dense && sparse_rows<CT, LOGE>(ctx);
   fa.dense_from = sparse_row_limit<LOGE>(ctx);
   fa.rows_per_cta = rpc;
   const size_t smem =
@@ -1162,7 +1166,7 @@ template <typename CT, int TPT, int LOGE, bool WIDE>
 aim_status launch_row_inv(aim_ctx* ctx, int channels, RowInvArgs ia, const Schedule& sc, cudaStream_t st) {
   constexpr int LPT = 3 - TPT;
   const int tpf = ctx->H >> LOGE, rpc = rows_per_cta<CT, TPT, LOGE>(ctx, sc);
-  ia.sparse = !ia.dense && sparse_rows<LOGE>(ctx);
+  ia.sparse = !ia.dense && sparse_rows<CT, LOGE>(ctx);
   ia.dense_from = sparse_row_limit<LOGE>(ctx);
   ia.rows_per_cta = rpc;
   const size_t smem =
@@ -1556,7 +1560,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
     if (inter_bytes_needed(ctx, channels, precision) > ctx->inter_bytes ||
         (size_t)channels * ctx->n_act * sizeof(VT) > ctx->vact_bytes)
       return fail(AIM_ESTATE, "grid workspace not reserved for this many right-hand sides");
-    const int sparse = sparse_rows<LOGE>(ctx), qcut = spec.filtered ? ctx->qcut : ctx->H;
+    const int sparse = sparse_rows<CT, LOGE>(ctx), qcut = spec.filtered ? ctx->qcut : ctx->H;
     smem = std::max(smem, 2 * (size_t)lines * HS * sizeof(T2) + (sparse ? sparse_smem<CT, LOGE>(ctx->logH, lines) : 0));
     MultiJob& J = m.jobs[i];
     const void* tw = twiddles(ctx, (CT*)nullptr);
