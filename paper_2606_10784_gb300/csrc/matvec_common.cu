@@ -66,7 +66,6 @@ __device__ __forceinline__ void gram_item(const GramArgs& a, long long t) {
 }
 
 __global__ void __launch_bounds__(256) k_gram_inv(GramArgs a) {
-  grid_trigger_dependents();
   gram_item(a, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -78,7 +77,6 @@ struct GramMultiArgs {
 };
 
 __global__ void __launch_bounds__(256) k_gram_inv_multi(const __grid_constant__ GramMultiArgs m) {
-  grid_trigger_dependents();
   int jb = 0;
   while (jb + 1 < m.njobs && (int)blockIdx.x >= m.first[jb + 1]) ++jb;   // the same job in every thread of the CTA
   gram_item(m.jobs[jb], (long long)((int)blockIdx.x - m.first[jb]) * blockDim.x + threadIdx.x);

@@ -107,7 +107,6 @@ __device__ __forceinline__ void ant_item(const AntArgs& a, long long t) {
 
 template <typename CT, int NP>
 __global__ void __launch_bounds__(kAntThreads) k_anterpolate(AntArgs a) {
-  grid_trigger_dependents();
   ant_item<CT, NP>(a, (long long)blockIdx.x * kAntThreads + threadIdx.x);
 }
 
@@ -380,7 +379,6 @@ __device__ __forceinline__ void row_fwd_item(const RowFwdArgs& a, int row_block,
 
 template <typename CT, int TPT, int LOGE, bool WIDE, bool LONG>
 __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_row_fwd(RowFwdArgs a) {
-  grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   row_fwd_item<CT, TPT, LOGE, LONG>(a, blockIdx.x, blockIdx.y, smraw);
 }
@@ -623,7 +621,6 @@ __device__ __forceinline__ void col_conv_halves(const ColArgs& a, int ctile, int
 
 template <typename CT, int TPT, int LOGE, bool WIDE = false>
 __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_col_conv(ColArgs a) {
-  grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   // with many channels they run along x: the channels of one column tile run back to back and
   // share its spectrum column through L2 (64 right-hand sides: 2.82 -> 2.67 ms per launch);
@@ -836,7 +833,6 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
 
 template <typename CT, int TPT, int LOGE, bool WIDE, bool LONG>
 __global__ void __launch_bounds__(WIDE ? kWideMax : LaunchMax<CT, TPT, LOGE>::value) k_row_inv(RowInvArgs a) {
-  grid_trigger_dependents();
   extern __shared__ __align__(16) unsigned char smraw[];
   row_inv_item<CT, TPT, LOGE, LONG>(a, blockIdx.x, blockIdx.y, smraw);
 }
@@ -1006,7 +1002,6 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, long long vbloc
 
 template <typename T2, int NP, int RB>
 __global__ void __launch_bounds__(256) k_gather(GatherArgs a) {
-  grid_trigger_dependents();
   gather_item<T2, NP, RB>(a, blockIdx.x);
 }
 

@@ -125,7 +125,6 @@ __device__ __forceinline__ double2 to_d2(float h_re, float l_re, float h_im, flo
 }
 
 __global__ void k_to_dfc(const double2* __restrict__ src, int count, dfc* __restrict__ dst) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < count) dst[t] = to_dfc(src[t]);
@@ -227,7 +226,6 @@ __global__ void __launch_bounds__(32 * kDot2Warps) k_multidot2_partial_df(const 
                                                                           const dfc* __restrict__ R1, int n, int nrhs,
                                                                           int J, double2* __restrict__ part0,
                                                                           double2* __restrict__ part1) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = blockIdx.x * kDot2Warps + wid, r = blockIdx.y, z = blockIdx.z;
@@ -265,7 +263,6 @@ __global__ void __launch_bounds__(32 * kDot2Warps) k_multidot2_partial_df(const 
 __global__ void k_dcgs2_finish(const double2* __restrict__ part0, const double2* __restrict__ part1, int nz, int J,
                                int nrhs, int j, int restart, double2* __restrict__ D0, double2* __restrict__ D1,
                                dfc* __restrict__ D0df, dfc* __restrict__ H) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int count = J * nrhs;
@@ -329,7 +326,6 @@ __global__ void __launch_bounds__(256) k_dcgs2_hs_scal(const dfc* H, const dfc* 
                                                        int final_step, double2* __restrict__ hs,
                                                        double2* __restrict__ colout, dfc* Hw,
                                                        double2* __restrict__ scal) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const int r = blockIdx.y;
   const int nrow_blocks = final_step ? 0 : (j + kHsRows - 1) / kHsRows;
@@ -405,7 +401,6 @@ __global__ void k_dcgs2_coeffs(const double2* __restrict__ D0, const double2* __
                                const double2* __restrict__ hs, const double2* __restrict__ scal, int j, int nrhs,
                                int restart, int final_step, dfc* __restrict__ H, double2* __restrict__ colout,
                                dfc* __restrict__ a1, dfc* __restrict__ g) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= j * nrhs) return;
@@ -440,7 +435,6 @@ __global__ void __launch_bounds__(kStepThreads) k_dcgs2_step(const double2* __re
                                                              dfc* __restrict__ H, double2* __restrict__ colout,
                                                              double2* __restrict__ scal, dfc* __restrict__ a1,
                                                              dfc* __restrict__ g) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const bool final_step = part1 == nullptr;
   const int r = blockIdx.x, J = j + 1, count = J * nrhs, tid = threadIdx.x;
@@ -552,7 +546,6 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) k_vcombine2_df(const dfc* _
                                                                    const double2* __restrict__ scal, dfc* Vj,
                                                                    const double2* __restrict__ w, dfc* Vnext,
                                                                    double2* __restrict__ cur) {
-  grid_trigger_dependents();
   grid_dependency_wait();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, r = blockIdx.y;
   const int i = blockIdx.x * 32 + lane;
