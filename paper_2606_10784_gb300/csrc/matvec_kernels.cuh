@@ -176,12 +176,12 @@ __host__ __device__ __forceinline__ SparseGeom sparse_geom(int logH) {
   return s;
 }
 
-// Shared memory of the sparse stages behind the transforms' buffers: the forward pass's K2 roots of
-// unity, w^j for j < J and, per row, the J masks of active r; the inverse pass's row ranges.
+// Shared memory of the sparse stages behind the transforms' buffers: the forward pass's R0 roots of
+// unity and, per row, the J masks of active r; the inverse pass's row ranges.
 template <typename CT, int LOGE>
 __host__ __device__ __forceinline__ size_t sparse_smem(int logH, int rows) {
   const SparseGeom s = sparse_geom<LOGE>(logH);
-  return (size_t)(s.k2 + (1 << s.logj)) * sizeof(CT) + ((size_t)rows << s.logj) * 4 + (size_t)(rows + 1) * 4;
+  return ((size_t)sizeof(CT) << s.l0) + ((size_t)rows << s.logj) * 4 + (size_t)(rows + 1) * 4;
 }
 
 // Whether a context's rows take the sparse stages. Counting operations, a point costs 2 R0 products
@@ -213,11 +213,15 @@ static int sparse_row_limit(const aim_ctx* ctx) {
   return ctx->row_most > limit ? limit : INT_MAX;
 }
 
-// Forward row pass of sparse rows. The points of a row go to their places j + J r of the row's two
-// buffers (u in the even half's, u w^j in the odd half's) and into the masks that say which r of a j
+// Forward row pass of sparse rows. The points of a row go to their places n = j + J r of the row's two
+// buffers (u in the even half's, u w^n in the odd half's) and into the masks that say which r of a j
 // hold one; nothing else is written, so nothing is zeroed. The first dense pass forms its inputs
-//     X0_half[j R0 + k1] = sum over the active r of j of u w^(half j) W_{2 R0}^{r (2 k1 + half)}
-// from them in registers (r ascending) and goes on at Ns = R0. (Scattering every point into the R0
+//     X0_half[j R0 + k1] = sum over the active r of j of u w^(half n) W_R0^(r k1)
+// from them in registers (r ascending) and goes on at Ns = R0. Every factor comes from the table, so a value
+// is rounded as often as in the dense passes, and not at all where W_R0 is 1, -1 or +-i (with w^j in place of
+// w^n and roots of 2 R0 in the odd half, and Horner's rule in the inverse pass, S^alpha at P = 512 was off by
+// 1.83e-14 in double-float instead of 1.65e-14; N at P = 1024 by 6.99e-14 instead of 6.32e-14; the row passes
+// take 469 -> 483 us at P = 4096 and 132 -> 129 us at P = 512 with 16 right-hand sides). (Scattering every point into the R0
 // outputs of its j by read-modify-write of shared memory took 38 of 280 us of the double-float pass
 // at 2048 points, and 13 of 33 us at 512 points, where the rows along the contour's tangents set the
 // time of the whole launch.)
@@ -237,31 +241,33 @@ __device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_bloc
 #pragma unroll
   for (int f = 0; f < NF; ++f) fb[f] = (2 * g + (TPT == 1 ? half : f)) * HS;
   const SparseGeom sg = sparse_geom<LOGE>(a.logH);
-  const int J = 1 << sg.logj;
+  const int J = 1 << sg.logj, R0 = 1 << sg.l0;
   T2* roots = sm + 2 * a.rows_per_cta * HS;
-  T2* wjs = roots + sg.k2;
-  unsigned* masks = reinterpret_cast<unsigned*>(wjs + J);
+  unsigned* masks = reinterpret_cast<unsigned*>(roots + R0);
   {
     const int p0 = live ? a.row_ptr[a.row_lo + rloc] : 0, p1 = live ? a.row_ptr[a.row_lo + rloc + 1] : 0;
-    for (int i = threadIdx.x; i < sg.k2; i += blockDim.x) roots[i] = ldro(&tw[i << sg.logj]);
-    for (int i = threadIdx.x; i < J; i += blockDim.x) wjs[i] = ldro(&tw[i]);
+    for (int i = threadIdx.x; i < R0; i += blockDim.x) roots[i] = ldro(&tw[i << (sg.logj + 1)]);
     for (int i = rem; i < J; i += per_row) masks[(g << sg.logj) + i] = 0;
     int ix = p0 + rem < p1 ? a.act_ix[p0 + rem] : 0;
+    T2 w = ldro(&tw[ix]);
     const T2* uv = static_cast<const T2*>(a.u) + (size_t)c * a.n_act;
     __syncthreads();
     grid_dependency_wait();
     for (int ap = p0 + rem; ap < p1; ap += per_row) {
-      if (ap != p0 + rem) ix = a.act_ix[ap];
+      if (ap != p0 + rem) {
+        ix = a.act_ix[ap];
+        w = ldro(&tw[ix]);
+      }
       const T2 u = uv[ap];
       sm[2 * g * HS + padi<LOGE>(ix)] = u;
-      sm[(2 * g + 1) * HS + padi<LOGE>(ix)] = cmul(u, wjs[ix & (J - 1)]);
+      sm[(2 * g + 1) * HS + padi<LOGE>(ix)] = cmul(u, w);
       atomicOr(&masks[(g << sg.logj) + (ix & (J - 1))], 1u << (ix >> sg.logj));
     }
   }
   __syncthreads();
   const unsigned* rowmask = masks + (g << sg.logj);
   auto load = [&](int f, int i) {
-    const int jj = i >> sg.l0, kk = 2 * (i & ((1 << sg.l0) - 1)) + (TPT == 1 ? half : f);
+    const int jj = i >> sg.l0, kk = i & (R0 - 1);
     const T2* src = sm + fb[f];
     unsigned m = rowmask[jj];
     T2 acc = czero<T2>();
@@ -269,7 +275,7 @@ __device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_bloc
     while (m) {
       const int r = __ffs(m) - 1;
       m &= m - 1;
-      const T2 v = cmul(src[padi<LOGE>(jj + (r << sg.logj))], roots[(r * kk) & (sg.k2 - 1)]);
+      const T2 v = cmul(src[padi<LOGE>(jj + (r << sg.logj))], roots[(r * kk) & (R0 - 1)]);
       acc = first ? v : cadd(acc, v);
       first = false;
     }
@@ -699,10 +705,9 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
   for (int f = 0; f < NF; ++f) fb[f] = (2 * g + (TPT == 1 ? half : f)) * HS;
   const T2* blk = static_cast<const T2*>(a.inter) + (size_t)c * P * a.nrows;
   // sparse rows: the CTA's active points, flat over its rows, lpp lanes each; the first
-  // round's point and its root are loaded here, so that their latency overlaps the transforms
+  // round's point is loaded here, so that its latency overlaps the transforms
   const int lpp = sparse_point_lanes(sparse_geom<LOGE>(a.logH).k2);
   int A0 = 0, A1 = 0, ix0 = 0;
-  T2 z0 = czero<T2>();
   int* rps = reinterpret_cast<int*>(sm + 2 * a.rows_per_cta * HS);
   if (a.sparse) {
     const int row0 = row_block * a.rows_per_cta;
@@ -732,10 +737,7 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
     }
     if (a.sparse) {   // behind the loads above: their latencies overlap
       const int ap = A0 + threadIdx.x / lpp;
-      if (ap < A1) {
-        ix0 = a.act_ix[ap];
-        z0 = ldro(&tw[ix0]);
-      }
+      if (ap < A1) ix0 = a.act_ix[ap];
     }
     if (!live || a.qcut < (P >> 1)) {   // zero the columns beyond the mask's disc
 #pragma unroll
@@ -760,8 +762,9 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
     if (logj > LOGE) smem_pass<LOGE, true, NF, LOGE>(sm, fb, j, tpf, a.logH, LOGE, tw, a.logP);
     // now sub-transform k1 of half h holds its J outputs at k1 J of the half's buffer, and
     //     y[n] = sum over k' = 2 k1 + h of Z_h[k1][n mod J] W_P^{-n k'}:
-    // each lane of a point sums tpl consecutive k' by Horner's rule in W_P^{-n}, and the lanes add
-    // up over a fixed shuffle tree (the order depends on the transform length alone)
+    // each lane of a point sums tpl <= 4 consecutive k', and the lanes add up over a fixed shuffle tree
+    // (the order depends on the transform length alone). Each term has its factor from the table, rounded
+    // once: Horner's rule in W_P^{-n} takes as many products in a chain, each rounding all terms so far
     const int l = threadIdx.x & (lpp - 1), grp = threadIdx.x / lpp, ngrp = blockDim.x / lpp;
     using VP = decltype(VT::x);
     VP* out = static_cast<VP*>(a.vact) + 2 * (size_t)c * a.n_act;
@@ -783,15 +786,19 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
       T2 acc = czero<T2>();
       if (valid) {
         const int ix = base == A0 ? ix0 : a.act_ix[ap];
-        const T2 z = base == A0 ? z0 : ldro(&tw[ix]);
         const T2* zb = sm + (size_t)(2 * lo) * HS;
         const int jj = ix & (J - 1), k0 = l * tpl;
-        for (int t = tpl - 1; t >= 0; --t) {
-          const int kk = k0 + t;
-          const T2 v = zb[(kk & 1) * HS + padi<LOGE>(((kk >> 1) << logj) + jj)];
-          acc = t == tpl - 1 ? v : cadd(cmulc(acc, z), v);
+        T2 root[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) root[t] = ldro(&tw[(ix * (k0 + min(t, tpl - 1))) & (P - 1)]);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          if (t < tpl) {
+            const int kk = k0 + t;
+            const T2 v = cmulc(zb[(kk & 1) * HS + padi<LOGE>(((kk >> 1) << logj) + jj)], root[t]);
+            acc = t == 0 ? v : cadd(acc, v);
+          }
         }
-        acc = cmulc(acc, ldro(&tw[(ix * k0) & (P - 1)]));
       }
       for (int off = lpp >> 1; off > 0; off >>= 1) acc = cadd(acc, shfl_xor_c(acc, off));
       // lane 0 stores the real part, lane 1 the imaginary part (every lane holds the sum): the
@@ -1190,7 +1197,7 @@ static int pass_tpt(const aim_ctx* ctx, const Schedule& sc, bool rows, long long
 
 // Whether a double-float pass with one transform of 8 elements per thread runs as its wide variant.
 // The plain kernels are bounded to 1024 threads, 64 registers, and spill; bounded to 512 threads they
-// take 102 (row passes) or 128 registers and none, but half as many threads fit an SM. So the wide ones
+// take 102 to 128 registers and none, but half as many threads fit an SM. So the wide ones
 // run launches that fit the GPU at once: 640 and 512 threads on each of 152 SMs. (N = 733 with three
 // right-hand sides 151 -> 132 us, N = 64 62 -> 57 us; a grid product of 157 thousand row-pass threads
 // 108 -> 116 us, so not there.)

@@ -110,3 +110,22 @@ def test_binary64_rows_take_no_longer_than_those_of_a_full_grid(aimlib):
     took = row_time(aimlib, ctx, n, 2)
     ctx.close()
     assert took < 1.2 * full, (took, full)
+
+
+# mean error of six random vectors with every row dense (operators N_alpha, S_alpha), against binary64
+DENSE = [(100.0, 1000, 230, 512, 0, 4.43e-14, 1.66e-14), (150.0, 1500, 512, 1024, 0, 6.54e-14, 1.69e-14),
+         (400.0, 4000, 1024, 2048, 0, 6.36e-14, 2.03e-14)]
+
+
+@pytest.mark.parametrize("per,n,m,P,precision,dense_N,dense_S", DENSE)
+def test_sparse_rows_are_as_accurate_as_dense_ones(aimlib, per, n, m, P, precision, dense_N, dense_S):
+    # a random walk of roundings: the two orders of the same sums differ by a few per cent of their error
+    ctx = aimlib.Context(synth.StarContour.from_seed(8).polygon(per, n), K, aimlib.TE, m, fft_P=P, alpha=3.0 * K)
+    for op, dense in (("N_alpha", dense_N), ("S_alpha", dense_S)):
+        errs = []
+        for seed in range(6):
+            x = torch.from_numpy(synth.random_coeffs(n, 1, seed=seed)).cuda()
+            want = product(ctx, op, x, 2)
+            errs.append(float((product(ctx, op, x, precision) - want).norm() / want.norm()))
+        assert np.mean(errs) < 1.04 * dense, (op, np.mean(errs), dense)
+    ctx.close()
