@@ -84,10 +84,12 @@ __device__ __forceinline__ void dft_reg(T2 (&v)[R]) {
   for (int k = 0; k < R; ++k) v[k] = t[k];
 }
 
-// Where the twiddles of a pass come from. Complex64: only the powers r = 1, 2, 4, 8 are read
-// from the table and the others are products of at most three of them (the complex64 passes keep
-// L1 busier than the FP32 pipe). Types whose complex product costs tens of FP32-pipe instructions (double-float) or
-// runs on the slow FP64 pipe (binary64) read every factor from the table instead.
+// Where the twiddles of a pass come from. Complex64 passes of radix 16: only the powers r = 1, 2, 4, 8
+// are read from the table and the others are products of at most three of them (the complex64 passes keep
+// L1 busier than the FP32 pipe). Types whose complex product costs tens of FP32-pipe instructions
+// (double-float) or runs on the slow FP64 pipe (binary64) read every factor from the table instead, and so do
+// the radix-8 passes of complex64, which follow one another more often: with products of rounded factors
+// operator S^alpha at P = 128 was off by 1.83e-7, with radix-16 passes by 1.70e-7.
 template <typename T2> struct TwiddleFromTable { static constexpr bool value = false; };
 template <> struct TwiddleFromTable<double2> { static constexpr bool value = true; };
 
@@ -108,12 +110,12 @@ __host__ __device__ __forceinline__ int twiddle_entries(int logP) { return (1 <<
 // The twiddles W_{Ns R}^{k r}, r = 1..R-1, of butterfly position k (k != 0): app(r, w) for each.
 // All transforms a thread works on at the same butterfly position share them, so callers apply
 // each factor to all of them before the next one is formed.
-template <int LOGR, typename T2, typename App>
+template <int LOGR, bool TAB, typename T2, typename App>
 __device__ __forceinline__ void twiddles(int k, int logNs, const T2* __restrict__ tw, int logP, App app) {
   constexpr int R = 1 << LOGR;
   const int q = logNs + LOGR;
   auto load = [&](int r) { return ldro(&tw[pass_table(logP, q, r) + k]); };
-  if constexpr (TwiddleFromTable<T2>::value) {
+  if constexpr (TAB) {
 #pragma unroll
     for (int r = 1; r < R; ++r) app(r, load(r));
   } else {
@@ -150,12 +152,12 @@ __device__ __forceinline__ void twiddles(int k, int logNs, const T2* __restrict_
 }
 
 // Twiddles of position k applied to the NF transforms v[f][t][.] (one set of factors for all),
-// then their length-R DFTs.
-template <int LOGR, bool INV, int NF, int NB, typename T2>
+// then their length-R DFTs. TAB: every factor from the table, whatever the type.
+template <int LOGR, bool INV, bool TAB, int NF, int NB, typename T2>
 __device__ __forceinline__ void bfly_shared(T2 (&v)[NF][NB][1 << LOGR], int t, int k, int logNs,
                                             const T2* __restrict__ tw, int logP) {
   if (k != 0)
-    twiddles<LOGR>(k, logNs, tw, logP, [&](int r, const T2& w) {
+    twiddles<LOGR, TAB || TwiddleFromTable<T2>::value>(k, logNs, tw, logP, [&](int r, const T2& w) {
 #pragma unroll
       for (int f = 0; f < NF; ++f) v[f][t][r] = INV ? cmulc(v[f][t][r], w) : cmul(v[f][t][r], w);
     });
@@ -189,7 +191,7 @@ __device__ __forceinline__ void pass_compute(T2 (&v)[1][(1 << LOGE) >> LOGR][1 <
     const int b = j + t * tpf;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[0][t][r] = load(b + (r << lognb));
-    bfly_shared<LOGR, INV>(v, t, b & nsm, logNs, tw, logP);
+    bfly_shared<LOGR, INV, LOGE == 3>(v, t, b & nsm, logNs, tw, logP);
   }
 }
 template <int LOGR, int LOGE, typename T2>
@@ -209,7 +211,7 @@ __device__ __forceinline__ void pass_store(const T2 (&v)[1][(1 << LOGE) >> LOGR]
 // Each thread works on butterflies b = j + t*tpf (t < E/R) of each of its transforms, whose
 // padded bases in shared memory are fb[f]. `load(f, i)` reads input i of transform f. Barrier
 // before and after the stores.
-template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Load>
+template <int LOGR, bool INV, int NF, int LOGE, bool TAB = false, typename T2, typename Load>
 __device__ __forceinline__ void smem_pass_from(T2* __restrict__ sm, const int (&fb)[NF], int j, int tpf, int logH,
                                                int logNs, const T2* __restrict__ tw, int logP, Load load) {
   constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
@@ -223,7 +225,7 @@ __device__ __forceinline__ void smem_pass_from(T2* __restrict__ sm, const int (&
     for (int f = 0; f < NF; ++f)
 #pragma unroll
       for (int r = 0; r < R; ++r) v[f][t][r] = load(f, b + (r << lognb));
-    bfly_shared<LOGR, INV>(v, t, b & nsm, logNs, tw, logP);
+    bfly_shared<LOGR, INV, TAB || LOGE == 3>(v, t, b & nsm, logNs, tw, logP);
   }
   __syncthreads();
 #pragma unroll
@@ -250,7 +252,7 @@ __device__ __forceinline__ void smem_pass(T2* __restrict__ sm, const int (&fb)[N
 
 // Last pass: `load(f, i)` in, `emit(out_index, values[NF])` out (no stores to shared memory here;
 // callers that write shared memory in `emit` must place a barrier first).
-template <int LOGR, bool INV, int NF, int LOGE, typename T2, typename Load, typename Emit>
+template <int LOGR, bool INV, int NF, int LOGE, bool TAB = false, typename T2, typename Load, typename Emit>
 __device__ __forceinline__ void last_pass_from(int j, int tpf, int logH, int logNs, const T2* __restrict__ tw, int logP,
                                                Load load, Emit emit) {
   constexpr int R = 1 << LOGR, NB = (1 << LOGE) >> LOGR;
@@ -265,7 +267,7 @@ __device__ __forceinline__ void last_pass_from(int j, int tpf, int logH, int log
     for (int f = 0; f < NF; ++f)
 #pragma unroll
       for (int r = 0; r < R; ++r) v[f][0][r] = load(f, b + (r << lognb));
-    bfly_shared<LOGR, INV>(v, 0, k, logNs, tw, logP);
+    bfly_shared<LOGR, INV, TAB || LOGE == 3>(v, 0, k, logNs, tw, logP);
     const int base = ((b - k) << LOGR) + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -337,7 +339,7 @@ __device__ __forceinline__ void conv_mid_pass(T2* __restrict__ sm, const int (&f
     for (int f = 0; f < NF; ++f)
 #pragma unroll
       for (int r = 0; r < R; ++r) v[f][t][r] = sm[fb[f] + padi<LOGE>(b + (r << lognb))];
-    bfly_shared<LOGR, false>(v, t, b, lognb, tw, logP);   // Ns = H/R, so b mod Ns = b
+    bfly_shared<LOGR, false, LOGE == 3>(v, t, b, lognb, tw, logP);   // Ns = H/R, so b mod Ns = b
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
 #pragma unroll

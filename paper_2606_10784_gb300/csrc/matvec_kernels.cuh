@@ -283,11 +283,12 @@ __device__ __forceinline__ void row_fwd_sparse(const RowFwdArgs& a, int row_bloc
   };
   T2* out = static_cast<T2*>(a.inter) + (size_t)c * P * a.nrows;
   auto emit = [&](int k, const T2 (&v)[NF]) { store_row<CT, TPT>(out, a, rloc, live, half, k, v); };
+  // both dense passes have twiddles here, the first of a dense row has none: every factor from the table
   if (sg.logj == LOGE) {
-    last_pass_from<LOGE, false, NF, LOGE>(j, tpf, a.logH, sg.l0, tw, a.logP, load, emit);
+    last_pass_from<LOGE, false, NF, LOGE, true>(j, tpf, a.logH, sg.l0, tw, a.logP, load, emit);
   } else {
-    smem_pass_from<LOGE, false, NF, LOGE>(sm, fb, j, tpf, a.logH, sg.l0, tw, a.logP, load);
-    last_pass<LOGE, false, NF, LOGE>(sm, fb, j, tpf, a.logH, sg.l0 + LOGE, tw, a.logP, emit);
+    smem_pass_from<LOGE, false, NF, LOGE, true>(sm, fb, j, tpf, a.logH, sg.l0, tw, a.logP, load);
+    last_pass_from<LOGE, false, NF, LOGE, true>(j, tpf, a.logH, sg.l0 + LOGE, tw, a.logP, PlainLoad<NF, LOGE, T2>{sm, fb}, emit);
   }
 }
 

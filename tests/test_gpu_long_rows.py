@@ -129,3 +129,13 @@ def test_sparse_rows_are_as_accurate_as_dense_ones(aimlib, per, n, m, P, precisi
             errs.append(float((product(ctx, op, x, precision) - want).norm() / want.norm()))
         assert np.mean(errs) < 1.04 * dense, (op, np.mean(errs), dense)
     ctx.close()
+
+
+# the same for complex64 before radix-8 passes and sparse rows, P = 64 to 2048
+DENSE32 = [(5.0, 50, 32, 64, 2.79e-7, 1.72e-7), (12.0, 120, 50, 128, 2.76e-7, 1.71e-7),
+           (40.0, 400, 128, 256, 3.18e-7, 1.85e-7), (400.0, 4000, 1024, 2048, 4.02e-7, 2.48e-7)]
+
+
+@pytest.mark.parametrize("per,n,m,P,dense_N,dense_S", DENSE32)
+def test_complex64_is_as_accurate_as_radix_16_passes_of_dense_rows(aimlib, per, n, m, P, dense_N, dense_S):
+    test_sparse_rows_are_as_accurate_as_dense_ones(aimlib, per, n, m, P, 1, dense_N, dense_S)
