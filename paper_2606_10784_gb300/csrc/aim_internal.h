@@ -197,7 +197,6 @@ struct aim_ctx {
   // Gram inverse, row i: entries for columns (i + d) mod n, d = -band..band
   double* gram_inv = nullptr;
   int gram_band = 0;
-  int gram_d0 = 0, gram_cnt = 0;   // the offsets [d0, d0 + cnt) of a row that are applied (gram_window)
   // entry counts of the scatter and gather lists and of gram_inv (for aim_export_setup)
   size_t n_sc = 0, n_ga = 0, n_gram = 0;
   // geometry: host copy and device vertices
@@ -343,8 +342,6 @@ struct GramCall {
   double2* y;
 };
 aim_status gram_inv_apply_multi(const GramCall* calls, int count, cudaStream_t st);
-// the applied window of the stored rows of G^-1 (host values), set in the context
-void gram_window(aim_ctx* ctx, const double* gi);
 size_t inter_bytes_needed(const aim_ctx* ctx, int channels, int precision);
 
 // several grid passes of several contexts in one persistent launch (matvec_kernels.cuh)

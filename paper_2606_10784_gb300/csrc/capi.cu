@@ -479,7 +479,6 @@ aim_status aim_setup(const aim_geometry* geometry, double k, const aim_grid* gri
   if (!hs.gram_inv.empty()) {
     AIM_TRY(upload(ctx, &ctx->gram_inv, hs.gram_inv, st));
     ctx->gram_band = hs.gram_band;
-    gram_window(ctx, hs.gram_inv.data());
   }
   ctx->n_sc = hs.sc_col.size();
   ctx->n_ga = hs.ga_act.size();

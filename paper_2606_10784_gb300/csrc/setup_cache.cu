@@ -284,7 +284,6 @@ aim_status aim_import_setup(const aim_geometry* geometry, double k, const aim_gr
       continue;
     }
     if (s.count == 0) continue;
-    if (s.slot == reinterpret_cast<void**>(&ctx->gram_inv)) gram_window(ctx, reinterpret_cast<const double*>(pay + s.offset));
     AIM_TRY(dev_alloc(ctx, s.slot, s.elem * s.count));
     AIM_CUDA_TRY(cudaMemcpyAsync(*s.slot, pay + s.offset, s.elem * s.count, cudaMemcpyHostToDevice, st));
   }

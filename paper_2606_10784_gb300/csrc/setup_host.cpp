@@ -516,13 +516,14 @@ aim_status host_setup(aim_ctx* ctx, HostSetup* hs) {
         }
       }
     } else {
-      // Elimination around the ring from either side: x_t = -pl[t] x_{t+1} left of a unit right-hand
+      // Elimination along the unrolled ring from either side: x_t = -pl[t] x_{t+1} left of a unit right-hand
       // side, x_t = -pr[t] x_{t-1} right of it. The ratios are below 1/2 on any mesh (the row sums of
       // the off-diagonals are half the diagonal; 0.27 on a uniform one) and forget their start by their
-      // square per step, so kLead steps ahead of the first one that is used stand for the whole ring,
-      // and what comes back around it is below 2^-n. A row of G^-1 is then a product of ratios on
-      // either side of its diagonal: a band of half-width kGramBand for large n; for smaller n whole
-      // rows, whose entries below 2^-90 of the diagonal stay zero. (n divisions in place of a window
+      // square per step, so kLead steps ahead of the first one that is used stand for the whole line. On the
+      // ring an unknown is reached from both sides, over d and over n - d segments: its entry is the sum of the
+      // two products of ratios (a third, once around the ring more, is below 2^-n of them). A row is a band of
+      // half-width kGramBand for large n, where what comes the other way round is below 2^-(n - kGramBand) of
+      // the diagonal, and whole for smaller n. (n divisions in place of a window
       // system per row: 2.6 -> 0.7 ms at n = 1500.)
       const bool band = n > kGramDenseMax;
       const int stride = band ? 2 * kGramBand + 1 : n, mid = band ? kGramBand : n / 2;
@@ -542,15 +543,33 @@ aim_status host_setup(aim_ctx* ctx, HostSetup* hs) {
         r = off((g + n - 1) % n) / (diag(g) - off(g) * r);
         if (t < n) pr[g] = r;
       }
-      for (int i = 0; i < n; ++i) {
-        const int il = (i + n - 1) % n, ir = (i + 1) % n;
-        double* row = &hs->gram_inv[(size_t)i * stride + mid];
-        row[0] = 1.0 / (diag(i) - off(il) * pl[il] - off(i) * pr[ir]);
-        const double least = band ? 0.0 : std::ldexp(std::fabs(row[0]), -90);
-        for (int d = 1, g = il; d <= mid && std::fabs(row[-d + 1]) >= least; ++d, g = g == 0 ? n - 1 : g - 1)
-          row[-d] = -pl[g] * row[-d + 1];
-        for (int d = 1, g = ir; d < stride - mid && std::fabs(row[d - 1]) >= least; ++d, g = g + 1 == n ? 0 : g + 1)
-          row[d] = -pr[g] * row[d - 1];
+      // kRows rows at a time: the products along a row are a chain
+      constexpr int kRows = 8;
+      const int len = band ? kGramBand : n - 1;
+      std::vector<double> left((size_t)(len + 1) * kRows), right(left.size());   // d segments away, row by row
+      for (int i0 = 0; i0 < n; i0 += kRows) {
+        int gl[kRows], gr[kRows];
+        for (int q = 0; q < kRows; ++q) {
+          const int i = (i0 + q) % n, il = (i + n - 1) % n, ir = (i + 1) % n;
+          left[q] = right[q] = 1.0 / (diag(i) - off(il) * pl[il] - off(i) * pr[ir]);
+          gl[q] = il;
+          gr[q] = ir;
+        }
+        for (int d = 1; d <= len; ++d)
+          for (int q = 0; q < kRows; ++q) {
+            left[(size_t)d * kRows + q] = -pl[gl[q]] * left[(size_t)(d - 1) * kRows + q];
+            right[(size_t)d * kRows + q] = -pr[gr[q]] * right[(size_t)(d - 1) * kRows + q];
+            gl[q] = gl[q] == 0 ? n - 1 : gl[q] - 1;
+            gr[q] = gr[q] + 1 == n ? 0 : gr[q] + 1;
+          }
+        for (int q = 0; q < kRows && i0 + q < n; ++q) {
+          double* row = &hs->gram_inv[(size_t)(i0 + q) * stride + mid];
+          row[0] = left[q];
+          for (int d = 1; d <= mid; ++d)
+            row[-d] = left[(size_t)d * kRows + q] + (band ? 0.0 : right[(size_t)(n - d) * kRows + q]);
+          for (int d = 1; d < stride - mid; ++d)
+            row[d] = right[(size_t)d * kRows + q] + (band ? 0.0 : left[(size_t)(n - d) * kRows + q]);
+        }
       }
     }
   }
