@@ -10,7 +10,7 @@ namespace aim {
 // order of every sum is fixed whatever the number of right-hand sides. FP64 throughput sets the cost of this
 // kernel on this GPU: a whole warp per output spends more FP64 operations on its shuffle tree than it gains
 // (a band: twice as many as on the band itself; rows of 512 entries, 64 right-hand sides 77 us with a warp,
-// @@ with sixteen lanes, 66 with eight, where one vector then takes 18 instead of @@ us), and a thread per
+// 67 with sixteen lanes, 66 with eight, where one vector takes 18 us instead of 5), and a thread per
 // output left the GPU idle for one vector (n threads, each a chain of cnt dependent loads and FMAs).
 // Whole rows are applied whole: G^-1 decays by 0.27 per entry on a uniform mesh, but the far entries are the
 // result for a vector of one nonzero, and carry what is not finite to every unknown.
