@@ -1184,10 +1184,13 @@ aim_status launch_row_inv(aim_ctx* ctx, int channels, RowInvArgs ia, const Sched
 // The results do not depend on it. A schedule that the caller or the autotuner set is obeyed; with
 // the context's default, one transform per thread where two leave the SMs short of warps: one has
 // half the serial work per thread, two share their twiddles. The lines lie between the sizes where
-// either was faster: row passes in double-float 26.0 against 28.7 us at 81 thousand threads and 76.0
-// against more at 324 thousand, in complex64 9.7 against 13.9 us at 27 thousand and 14.0 against 14.7 at
-// 81 thousand; column passes 14.5 against 18.5 us at 16 thousand (S^alpha, P = 512) and 26.6 against
-// 22.5 at 65 thousand (P = 1024).
+// either was faster, one against two: forward row passes of full grids in double-float 14.4 against 16.5 us at
+// 12 thousand threads, 33.7 against 41.7 at 93 thousand and 51 against 57 at 125 thousand, then 174 against 160
+// at 500 thousand; in complex64 9.1 against 10.3 us at 7 thousand and 18.4 against 16.4 at 62 thousand; column
+// passes 14.5 against 18.5 us at 16 thousand (S^alpha, P = 512) and 26.6 against 22.5 at 65 thousand
+// (P = 1024). The inverse row pass of a full grid always takes two: with one, half of the lanes recombine and
+// store every output (double-float 48 against 36 us at 125 thousand threads, 14.7 against 12.6 at 12 thousand;
+// complex64 26 against 20 us at 62 thousand).
 template <typename CT>
 static int pass_tpt(const aim_ctx* ctx, const Schedule& sc, bool rows, long long lines) {
   if (std::is_same<CT, double2>::value || !sched_is_default(ctx, precision_of((CT*)nullptr))) return sc.tpt;
@@ -1261,7 +1264,8 @@ static aim_status launch_three_passes(aim_ctx* ctx, int channels, bool filtered,
   using I3 = std::integral_constant<int, 3>;
   using I4 = std::integral_constant<int, 4>;
   for (int pass = 0; pass < 3; ++pass) {
-    const int tpt = pass_tpt<CT>(ctx, sc, pass != 1, pass != 1 ? rows : cols);
+    const bool full_inverse = pass == 2 && ia.dense && sched_is_default(ctx, precision_of((CT*)nullptr));
+    const int tpt = full_inverse ? 2 : pass_tpt<CT>(ctx, sc, pass != 1, pass != 1 ? rows : cols);
     aim_status s;
     if constexpr (std::is_same<CT, double2>::value) {
       s = run(I2{}, I4{}, pass);
