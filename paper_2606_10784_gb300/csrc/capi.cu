@@ -797,7 +797,7 @@ static aim_status query_context_bytes(const aim_geometry* geometry, const aim_gr
   b += committed(hs.gram_inv.size() * 8);
   const size_t nvals = te ? 2 : 1;
   if (nnz > 0) b += committed((n + 1) * 4) + committed(nnz * 4) + nvals * (committed(nnz * 16) + committed(nnz * 8));
-  b += 2 * (committed(nq * 16) + committed(nq * 8) + committed(nq * 16)) + committed((H + 1) * 4);   // spectra
+  b += 2 * (committed(nq * 16) + committed(nq * 8) + committed(nq * 16)) + committed((H + 1) * 4);   // spectra, and a page to spare
   // setup temporaries (freed before aim_setup returns)
   size_t t = committed(nq * 16);                                 // kernel samples
   if (nnz > 0) {

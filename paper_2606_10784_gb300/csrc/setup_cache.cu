@@ -3,6 +3,7 @@
 // reloaded, so that a restarted process skips the setup. The key and the checksum are
 // FNV-1a (Fowler, Noll, Vo), the checksum taken over 64-bit words in four interleaved lanes.
 #include <chrono>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <new>
@@ -77,7 +78,7 @@ uint64_t payload_checksum(const unsigned char* p, size_t bytes) {
 
 // One array of the payload: the context field it belongs to, its element size and count.
 struct Section {
-  void** slot;
+  void** slot;         // null: not kept by a context (live_columns)
   size_t elem;
   size_t count;
   size_t offset = 0;   // from the payload's start, a multiple of 16
@@ -112,13 +113,21 @@ size_t layout(aim_ctx* c, int nproj, long long nnz, std::vector<Section>* out) {
   }
   v.push_back({reinterpret_cast<void**>(&c->specU), sizeof(double2), nq});
   v.push_back({reinterpret_cast<void**>(&c->specA), sizeof(double2), nq});
-  v.push_back({reinterpret_cast<void**>(&c->specA_live), sizeof(int), (size_t)c->H + 1});
+  v.push_back({nullptr, sizeof(int), (size_t)c->H + 1});
   size_t off = 0;
   for (Section& sct : v) {
     sct.offset = off;
     off += (sct.elem * sct.count + 15) & ~size_t(15);
   }
   return off;
+}
+
+// The payload's last array: per column q' = 0..H of the filtered spectrum 0 where the mask zeroes all of it,
+// that is, its entry p = 0 (kappa grows with p). The grid passes go by qcut instead; blobs keep the array, so
+// that a blob is read by every build of this format version.
+void live_columns(const aim_ctx* c, int* live) {
+  for (int q = 0; q <= c->H; ++q)
+    live[q] = c->filter_enabled != AIM_FILTER_NUMERICAL || (2.0 * M_PI / ((double)c->P * c->eps)) * q <= c->alpha;
 }
 
 // A CSR row pointer: starts at 0, never decreases, ends at `total`.
@@ -172,7 +181,13 @@ aim_status aim_export_setup(const aim_ctx* ctx_in, void* buf, size_t* bytes, voi
   unsigned char* pay = out + sizeof(BlobHeader);
   for (const Section& s : secs) {
     const size_t len = s.elem * s.count, padded = (len + 15) & ~size_t(15);
-    if (len > 0) AIM_CUDA_TRY(cudaMemcpyAsync(pay + s.offset, *s.slot, len, cudaMemcpyDeviceToHost, st));
+    if (s.slot == nullptr) {
+      std::vector<int> live(s.count);
+      live_columns(ctx, live.data());
+      std::memcpy(pay + s.offset, live.data(), len);
+    } else if (len > 0) {
+      AIM_CUDA_TRY(cudaMemcpyAsync(pay + s.offset, *s.slot, len, cudaMemcpyDeviceToHost, st));
+    }
     if (padded > len) std::memset(pay + s.offset + len, 0, padded - len);
   }
   AIM_CUDA_TRY(cudaStreamSynchronize(st));
@@ -279,6 +294,7 @@ aim_status aim_import_setup(const aim_geometry* geometry, double k, const aim_gr
   ctx->near.nnz = h.nnz;
   ctx->nnz_near = h.nnz;
   for (const Section& s : secs) {
+    if (s.slot == nullptr) continue;
     if (s.slot == reinterpret_cast<void**>(&ctx->tw)) {
       AIM_TRY(upload_twiddles(ctx, reinterpret_cast<const double*>(pay + s.offset), st));
       continue;

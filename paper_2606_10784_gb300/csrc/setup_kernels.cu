@@ -176,14 +176,11 @@ aim_status derive_narrow_copies(const double2* src, size_t count, float2* f, flo
   return AIM_OK;
 }
 
-// live[q'] = 0 when the mask zeroes column q' entirely. kappa(p, q') >= kappa(0, q') holds in
-// floating point as well (sqrt is exact on the perfect square q'^2 and monotone, and both are
-// scaled by the same factor), so the column has a kept entry exactly when its p = 0 entry is kept.
 // CA (may be null): the transform of the analytically filtered samples, which then becomes the
-// filtered spectrum as it is (no mask; every column live).
+// filtered spectrum as it is (no mask).
 __global__ void k_pack_spectrum(const double2* C, const double2* CA, int H, int P, double eps, double alpha,
                                 int filter, double2* specU, double2* specA, float2* specUf, float2* specAf,
-                                float4* specUdf, float4* specAdf, int* live) {
+                                float4* specUdf, float4* specAdf) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long total = (long long)(H + 1) * (H + 1);
   if (t >= total) return;
@@ -200,7 +197,6 @@ __global__ void k_pack_spectrum(const double2* C, const double2* CA, int H, int 
   specAf[t] = float2{(float)va.x, (float)va.y};
   specUdf[t] = split_df(v);
   specAdf[t] = split_df(va);
-  if (off == 0) live[qq] = (CA != nullptr || keep) ? 1 : 0;   // p = 0
 }
 
 // ------------------------------------------------------------------------------------
@@ -837,14 +833,13 @@ aim_status device_spectra_and_near(aim_ctx* ctx, const HostSetup& hs, cudaStream
   AIM_TRY(dev_alloc_t(ctx, &ctx->specAf, nq));
   AIM_TRY(dev_alloc_t(ctx, &ctx->specUdf, nq));
   AIM_TRY(dev_alloc_t(ctx, &ctx->specAdf, nq));
-  AIM_TRY(dev_alloc_t(ctx, &ctx->specA_live, (size_t)H + 1));
   {
     const int tpb = 256;
     ProfScope ps(K_SETUP_PACK, st);
     k_pack_spectrum<<<(unsigned)((nq + tpb - 1) / tpb), tpb, 0, st>>>(samp, sampA, H, P, ctx->eps, ctx->alpha,
                                                                       ctx->filter_enabled, ctx->specU, ctx->specA,
                                                                       ctx->specUf, ctx->specAf, ctx->specUdf,
-                                                                      ctx->specAdf, ctx->specA_live);
+                                                                      ctx->specAdf);
     AIM_CUDA_TRY(cudaGetLastError());
   }
   // temporaries are freed when `tmp` goes out of scope: wait for the kernels first
