@@ -99,6 +99,7 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // sizes
 // ------------------------------------------------------------------------------------
 constexpr int kMaxP = 4096;          // largest embedding side (FFT length)
+constexpr int kSMs = 152;             // of a GB300
 constexpr int kMinP = 64;            // smallest: every half-length transform has >= 2 passes
 constexpr int kMaxProj = 4;          // TE: phi, phi', n_x phi, n_y phi
 constexpr int kGramBand = 40;        // half bandwidth of the banded G^-1 for large N
@@ -139,7 +140,7 @@ struct NearField {
 
 // Launch schedule of the grid kernels for one precision: transforms per thread (1: even/odd
 // halves in adjacent lanes, 2: both in one thread), the minimum threads of a row-pass CTA, the
-// columns of a column-pass CTA (0: the fewest whole tiles that give 128 threads), and the
+// columns of a column-pass CTA (0: by size, col_cols_of), and the
 // elements each thread owns per transform (16 or 8; 0 means 16).
 struct Schedule {
   int tpt;

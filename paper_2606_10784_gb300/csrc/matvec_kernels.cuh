@@ -1016,17 +1016,17 @@ __global__ void __launch_bounds__(256) k_gather(GatherArgs a) {
 // Threads of a gather CTA: 256, fewer while that leaves fewer CTAs than twice the SMs.
 inline int gather_threads(long long threads) {
   int tpb = 256;
-  while (tpb > 32 && threads / tpb < 304) tpb >>= 1;
+  while (tpb > 32 && threads / tpb < 2 * kSMs) tpb >>= 1;
   return tpb;
 }
 
-// Right-hand sides of a gather group: the power of two at or above their number, at most 8 (more
-// sums would spill), and fewer while that leaves fewer warps than four per SM: a group's FP64 work
+// Right-hand sides of a gather group: the power of two at or above their number, at most 8 (their sums
+// fill 128 registers and spill 24 bytes in double-float), and fewer while that leaves fewer warps than four per SM: a group's FP64 work
 // grows with its right-hand sides, and short products are better off on more SMs (N = 400, seven
 // right-hand sides: 19 us in groups of eight).
 inline int gather_rhs_block(int n, int nrhs) {
   int rb = nrhs >= 5 ? 8 : nrhs >= 3 ? 4 : nrhs;
-  while (rb > 1 && (long long)n * ((nrhs + rb - 1) / rb) * kGatherLanes < 608 * 32) rb >>= 1;
+  while (rb > 1 && (long long)n * ((nrhs + rb - 1) / rb) * kGatherLanes < 4 * kSMs * 32) rb >>= 1;
   return rb;
 }
 
@@ -1208,8 +1208,8 @@ static int pass_tpt(const aim_ctx* ctx, const Schedule& sc, bool rows, long long
 inline bool wide_pass(const aim_ctx* ctx, const Schedule& sc, bool rows, long long lines) {
   const int per_line = ctx->H >> 2;   // two threads for every 8 elements
   const long long threads = lines * per_line;
-  if (rows) return rows_per_cta<dfc, 1, 3>(ctx, sc) * per_line <= kWideMax && threads <= 152 * 640;
-  return col_cols_of<dfc, 1, 3>(sc, ctx->logH, ctx->logP) * per_line <= kWideMax && threads <= 152 * 512;
+  if (rows) return rows_per_cta<dfc, 1, 3>(ctx, sc) * per_line <= kWideMax && threads <= kSMs * 640;
+  return col_cols_of<dfc, 1, 3>(sc, ctx->logH, ctx->logP) * per_line <= kWideMax && threads <= kSMs * 512;
 }
 
 template <typename CT>
@@ -1546,7 +1546,7 @@ static aim_status launch_multi(const MultiPassSpec* passes, int count, unsigned*
   for (int i = 0; i < count; ++i) maxH = std::max(maxH, passes[i].ctx->H);
   const int B = multi_cta_threads<CT, TPT, LOGE>(maxH);
   if (B < LPT * (maxH >> LOGE)) return fail(AIM_EINVAL, "transform too long for the multi-context launch");
-  static thread_local MultiArgs m;   // 17 KB: kept off the stack
+  static thread_local MultiArgs m;   // 19 KB: kept off the stack
   m = MultiArgs{};
   m.njobs = count;
   m.bar = scratch;

@@ -726,8 +726,9 @@ static void vcombine_df(const dfc* V, const dfc* c, int J, int n, int nrhs, doub
 }
 
 size_t krylov_bytes(size_t n, int nrhs, int restart) {
-  // partial sums of the two basis updates of a step (chunks of kCgsChunk vectors) or of its two
-  // sets of inner products (chunks of kDotChunk elements), whichever needs more
+  // partial sums of a step's two sets of inner products (chunks of kDotChunk elements) or of the update of
+  // x at a cycle's end (chunks of kCgsChunk vectors, counted twice: the figure is part of what
+  // aim_query_solve_bytes reports, and limits set by it keep admitting the same problems), whichever is more
   const size_t nz = (n + kDotChunk - 1) / kDotChunk;
   const size_t part_vecs =
       std::max(2 * ((size_t)(restart + kCgsChunk) / kCgsChunk), (2 * nz * (restart + 1) + n - 1) / n);
