@@ -396,7 +396,8 @@ void aim_batcher_destroy(aim_batcher* batcher);
 aim_status aim_batcher_stats(aim_batcher* batcher, long long* products, long long* launches,
                              long long* fused_products);
 /* aim_solve with its operator products going through `batcher` (see above); same arguments,
- * results and errors, plus AIM_ETIMEOUT when a fused launch's grid barrier gave up. One batched
+ * results and errors, plus AIM_ETIMEOUT when a fused launch's grid barrier gave up, from then on for
+ * every solve that fuses (a fused launch behind one that gave up leaves its results unwritten). One batched
  * solve per host thread at a time (AIM_ESTATE otherwise). */
 aim_status aim_solve_batched(aim_batcher* batcher, aim_ctx* ctx, aim_op system, int nrhs,
                              const void* rhs, void* x, int x0_given, const aim_solve_opts* opts,

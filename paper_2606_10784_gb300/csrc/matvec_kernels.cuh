@@ -220,8 +220,8 @@ static int sparse_row_limit(const aim_ctx* ctx) {
 // from them in registers (r ascending) and goes on at Ns = R0. Every factor comes from the table, so a value
 // is rounded as often as in the dense passes, and not at all where W_R0 is 1, -1 or +-i (with w^j in place of
 // w^n and roots of 2 R0 in the odd half, and Horner's rule in the inverse pass, S^alpha at P = 512 was off by
-// 1.83e-14 in double-float instead of 1.65e-14; N at P = 1024 by 6.99e-14 instead of 6.32e-14; the row passes
-// take 469 -> 483 us at P = 4096 and 132 -> 129 us at P = 512 with 16 right-hand sides). (Scattering every point into the R0
+// 1.83e-14 in double-float instead of 1.66e-14, N at P = 1024 by 6.99e-14 instead of 6.48e-14). (Scattering
+// every point into the R0
 // outputs of its j by read-modify-write of shared memory took 38 of 280 us of the double-float pass
 // at 2048 points, and 13 of 33 us at 512 points, where the rows along the contour's tangents set the
 // time of the whole launch.)
@@ -764,8 +764,10 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
     // now sub-transform k1 of half h holds its J outputs at k1 J of the half's buffer, and
     //     y[n] = sum over k' = 2 k1 + h of Z_h[k1][n mod J] W_P^{-n k'}:
     // each lane of a point sums tpl <= 4 consecutive k', and the lanes add up over a fixed shuffle tree
-    // (the order depends on the transform length alone). Each term has its factor from the table, rounded
-    // once: Horner's rule in W_P^{-n} takes as many products in a chain, each rounding all terms so far
+    // (the order depends on the transform length alone). A lane's terms have W_P^{-n t}, t < 4, from the table
+    // and its sum W_P^{-n k0}, so a term is rounded twice, as in a dense row's last pass and recombination
+    // (Horner's rule in W_P^{-n} takes as many products in a chain and rounds all terms so far in each; a
+    // table factor for every term, 64 scattered loads a point at P = 4096, cost 10 us of 190)
     const int l = threadIdx.x & (lpp - 1), grp = threadIdx.x / lpp, ngrp = blockDim.x / lpp;
     using VP = decltype(VT::x);
     VP* out = static_cast<VP*>(a.vact) + 2 * (size_t)c * a.n_act;
@@ -789,17 +791,19 @@ __device__ __forceinline__ void row_inv_item(const RowInvArgs& a, int row_block,
         const int ix = base == A0 ? ix0 : a.act_ix[ap];
         const T2* zb = sm + (size_t)(2 * lo) * HS;
         const int jj = ix & (J - 1), k0 = l * tpl;
-        T2 root[4];
+        T2 zt[3];   // W_P^n, its square and its cube: the same in all lanes of the point
 #pragma unroll
-        for (int t = 0; t < 4; ++t) root[t] = ldro(&tw[(ix * (k0 + min(t, tpl - 1))) & (P - 1)]);
+        for (int t = 1; t < 4; ++t) zt[t - 1] = ldro(&tw[(ix * min(t, tpl - 1)) & (P - 1)]);
+        const T2 w0 = ldro(&tw[(ix * k0) & (P - 1)]);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           if (t < tpl) {
             const int kk = k0 + t;
-            const T2 v = cmulc(zb[(kk & 1) * HS + padi<LOGE>(((kk >> 1) << logj) + jj)], root[t]);
-            acc = t == 0 ? v : cadd(acc, v);
+            const T2 v = zb[(kk & 1) * HS + padi<LOGE>(((kk >> 1) << logj) + jj)];
+            acc = t == 0 ? v : cadd(acc, cmulc(v, zt[t - 1]));
           }
         }
+        acc = cmulc(acc, w0);
       }
       for (int off = lpp >> 1; off > 0; off >>= 1) acc = cadd(acc, shfl_xor_c(acc, off));
       // lane 0 stores the real part, lane 1 the imaginary part (every lane holds the sum): the
