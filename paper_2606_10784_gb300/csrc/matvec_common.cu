@@ -21,7 +21,7 @@ struct GramArgs {
   const double2* x;
   double2* y;
 };
-constexpr int kGramWideRows = 256;   // entries from which a row gets 16 lanes
+constexpr int kGramWideRows = 89;   // entries from which a row gets 16 lanes: eight load 88 before the wait for x
 
 // all 32 lanes of every warp call it (the group sums are shuffles)
 __device__ __forceinline__ void gram_item(const GramArgs& a, long long t) {
