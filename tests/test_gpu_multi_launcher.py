@@ -115,6 +115,7 @@ def test_a_batcher_that_gave_up_refuses_and_reports(aimlib, probe):
     t = threading.Thread(target=solve, args=(aimlib, ctxs[0], batcher, out, 0, 200000))
     t.start()
     while batcher.stats()["launches"] < 50:
+        assert t.is_alive()
         time.sleep(0.01)
     probe.probe_batcher_err_host(batcher._h)[1] = 1
     solve(aimlib, ctxs[1], batcher, out, 1, 40)
